@@ -169,6 +169,10 @@ extern "C" int sdq_plan_create(const sdq_layer_desc* desc, const int8_t* had_sig
     sdq_plan_destroy(p);
     return SDQ_ERR_CUDA;
   }
+  if (prefill_occupancy(p) != cudaSuccess) {
+    sdq_plan_destroy(p);
+    return SDQ_ERR_CUDA;
+  }
   for (int M = 1; M <= kMaxDecodeM; ++M) p->dcfg[M] = decode_config_search(p, M);
   *out = p;
   return SDQ_OK;
@@ -234,7 +238,7 @@ static int contract(sdq_plan p, const uint32_t* codes_tiled, const float* alpha,
   if (!codes_tiled || !alpha || !y || !aligned16(codes_tiled) || !aligned16(y)) return SDQ_ERR_INVALID_ARG;
   cudaError_t e = M <= kMaxDecodeM
                       ? launch_decode(p, codes_tiled, alpha, M, y, ws, (cudaStream_t)stream, early, y_mode)
-                      : launch_prefill(p, codes_tiled, alpha, M, y, ws, (cudaStream_t)stream);
+                      : launch_prefill(p, codes_tiled, alpha, M, y, ws, (cudaStream_t)stream, early);
   if (e == cudaErrorNotSupported) return SDQ_ERR_UNSUPPORTED;
   return cuda_status(e);
 }

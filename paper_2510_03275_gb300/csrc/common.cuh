@@ -69,7 +69,9 @@ cudaError_t launch_decode(const sdq_plan_s* p, const uint32_t* codes, const floa
 // multiple of 64), so that each decode CTA copies its chunk's part.
 bool decode_image(const sdq_plan_s* p);
 cudaError_t launch_prefill(const sdq_plan_s* p, const uint32_t* codes, const float* alpha, int M,
-                           float* y, void* ws, cudaStream_t st);
+                           float* y, void* ws, cudaStream_t st, int early);
+// Fills the plan's pf_clusters (launch-shape facts of the device).
+cudaError_t prefill_occupancy(sdq_plan_s* p);
 cudaError_t launch_read_prep(const sdq_plan_s* p, int M, const void* ws, float* out, cudaStream_t st);
 
 // Raise `kernel`'s dynamic shared-memory limit to `bytes` once per device:
@@ -336,6 +338,58 @@ __host__ __device__ constexpr uint32_t mxf4_idesc(int n) {
 }
 // ue8m0 1.0 in every byte of a scale-factor column.
 constexpr uint32_t kUnitScales = 0x7F7F7F7Fu;
+
+// Issue from a whole converged warp: the instructions below take their
+// operands from the warp's uniform registers.  Inside an `if (lane == 0)`
+// branch the compiler has to move every operand there at each issue, which
+// costs the issuing thread 130 - 150 cycles per MMA or copy; in a loop that
+// all 32 lanes run with the same values, only the instruction itself is
+// predicated on one elected lane (always the same one, so that a commit
+// covers the MMAs before it).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
+#define SDQ_ELECT "{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n @q "
+__device__ __forceinline__ void umma_bf16_warp(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                               uint32_t accumulate) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n" SDQ_ELECT
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n}\n" ::"r"(d_tmem),
+               "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// (A in tensor memory)
+__device__ __forceinline__ void umma_bf16_ts_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                                  uint32_t accumulate) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n" SDQ_ELECT
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n}\n" ::"r"(d_tmem),
+               "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void umma_commit_warp(uint64_t* bar) {
+  asm volatile(SDQ_ELECT "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
+                   smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx_warp(uint64_t* bar, uint32_t bytes) {
+  asm volatile(SDQ_ELECT "mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(smem_u32(bar)),
+               "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_warp(void* dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar) {
+  asm volatile(SDQ_ELECT
+               "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+               " [%0], [%1, {%2, %3}], [%4];\n}\n" ::"r"(smem_u32(dst)),
+               "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void bulk_g2s_warp(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(SDQ_ELECT
+               "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n}\n" ::"r"(
+                   smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void bulk_g2s_hint_warp(void* dst, const void* src, uint32_t bytes, uint64_t* bar,
+                                                   uint64_t policy) {
+  asm volatile(SDQ_ELECT
+               "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+               " [%0], [%1], %2, [%3], %4;\n}\n" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)),
+               "l"(policy) : "memory");
+}
 
 // Two fp32 values to a byte of e2m1 codes (round to nearest even, saturating
 // at +-6): `lo` in bits 0-3, `hi` in bits 4-7; `q` receives the two values

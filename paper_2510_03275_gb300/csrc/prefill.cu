@@ -12,11 +12,12 @@
 // 64-code stage order the expansion yields) is the B operand, loaded by TMA
 // in the canonical K-major 128-byte-swizzled layout.
 //
-// CTA tile 128 code rows (M of the MMA = TMEM lanes) x 256 batch rows (N),
-// 64 codes per pipeline stage, kStages stages:
-//   warp 0      TMEM allocation; lane 0 issues the TMA load of the stage's
-//               x_tilde tile and the bulk copy of its code slab (tiled
-//               layout: 128 rows x 64 codes, contiguous)
+// CTA tile 128 code rows (M of the MMA = TMEM lanes) x `bn` batch rows (N, a
+// multiple of 16 up to 256: the batch in equal tiles), 64 codes per pipeline
+// stage; a cluster of S CTAs splits K, and the sum of its S accumulators goes
+// through distributed shared memory in CTA order (the same bits every run):
+//   warp 0      TMEM allocation; lane 0 issues the TMA loads of the stages'
+//               x_tilde tiles
 //   warp 1      lane 0 issues tcgen05.mma (4 x K = 16 per stage, A from the
 //               stage's TMEM slot), commits to the stage's "empty" barrier,
 //               finally to the accumulator one
@@ -24,11 +25,24 @@
 //               thread = code row: its 64 codes become 32 TMEM columns of
 //               bf16 pairs (one x32 store); then the epilogue: accumulator
 //               column m -> y[m, r] scaled by alpha_r / 2, each warp one lane
-//               quadrant and half of the 256 columns
-// TMEM: accumulator columns 0..255, A slot s at 256 + 32 s.
+//               quadrant and half of the columns
+//   warp 10     lane 0 streams the codes, 4 stages (tiled layout: 4 slabs of
+//               128 rows x 64 codes, contiguous) per bulk copy, into a ring
+//               of its own that runs ahead of the x_tilde stages: codes come
+//               from HBM, x_tilde from the L2
+// TMEM: accumulator columns 0 .. bn - 1, A slot s at bn + 32 s; 256 columns
+// and two CTAs per SM for bn up to 128 (one CTA's prologue and epilogue then
+// run beside the other's MMAs), else 512 and one.
+// At M = 201 on the LLaMA-7B linears (4096 x 8192 codes, 32 row tiles): 52 us
+// as one 256-row tile per 128 x K, 15 us with S = 4 and 208 columns; 12288
+// rows 53 -> 34, 22016 rows 103 -> 64, 4096 x 22016 codes 125 -> 27.  Two
+// things bound the stages: an issuing thread needs its operands in uniform
+// registers (warp_index, *_warp: 630 -> 360 cycles a stage), and the two
+// expander sets take about 350 cycles per stage, so that below 160 batch rows
+// per tile the expansion and not the tensor core is the limit.
 // Every wait on an mbarrier is bounded (about 2 s); a timeout writes the call
-// number into the workspace's call record and the CTA finishes without
-// further waits.
+// number into the workspace's call record and the CTA waits (again bounded)
+// for its own copies and MMAs before it frees TMEM and ends.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -41,13 +55,17 @@ namespace sdq {
 
 namespace {
 
-constexpr int kBM = 128, kBN = 256, kBK = 64, kStages = 6;
-constexpr int kXTile = kBN * kBK * 2;     // 32 KB: 256 batch rows x 64 codes of bf16 x_tilde
-constexpr int kCTile = kBM * 16;          // packed codes of a stage: 128 rows x 64 codes, at most 2 KB
-constexpr int kSmem = kStages * (kXTile + kCTile) + 1024;
-constexpr int kThreads = 320;   // 2 control warps + 8 expander / epilogue warps
-constexpr uint32_t kAcol = kBN;           // first TMEM column of the A slots
+constexpr int kBM = 128, kBK = 64;
+constexpr int kCodeStages = 4;            // stages per code copy
+constexpr int kCodeSlots = 4;             // code ring
+constexpr int kCSlab = kBM * 16;          // packed codes of a stage: 128 rows x 64 codes, at most 2 KB
+constexpr int kCSlot = kCodeStages * kCSlab;
+constexpr int kMaxStages = 6;             // x_tilde tiles and TMEM A slots
+constexpr int kExpWarps = 8;
+constexpr int kThreads = 32 * (3 + kExpWarps);   // 2 control warps, 8 expander / epilogue warps, the code stream
 constexpr uint32_t kAslot = kBK / 2;      // TMEM columns per A slot (bf16 pairs)
+constexpr int kMaxSplit = 8;              // k chunks (portable cluster size)
+constexpr int kSmemSm = 227 * 1024;       // shared memory of an SM that blocks can have
 
 struct PrefillParams {
   const uint32_t* codes;
@@ -55,142 +73,185 @@ struct PrefillParams {
   float* y;
   uint64_t* rec;       // call record
   uint64_t call;
-  int M, N, ntiles, ngroups, wpg, nks, quantizer;
+  int M, N, ngroups, wpg, nks, quantizer;
+  int bn, stages, split, early;
 };
 
-// Instruction descriptor, kind::f16: D fp32, A and B bf16, both K-major,
-// M = 128, N = 256.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) |
-                            ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-
-__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                             uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+// 16 bytes of the shared memory of the cluster's CTA `rank`, at this CTA's address `a`.
+__device__ __forceinline__ float4 ld_cluster4(uint32_t a, uint32_t rank) {
+  uint32_t r;
+  float4 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(r) : "memory");
+  return v;
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, 2)
     prefill_kernel(const __grid_constant__ CUtensorMap xmap, PrefillParams p) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full[kStages], empty[kStages], a_full[kStages], acc_bar;
+  __shared__ __align__(8) uint64_t x_full[kMaxStages], empty[kMaxStages], a_full[kMaxStages], c_full[kCodeSlots],
+      c_empty[kCodeSlots], acc_bar;
   __shared__ uint32_t tmem_base;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tile = blockIdx.x, n0 = tile * kBM, m0 = blockIdx.y * kBN;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  const int tile = blockIdx.x, n0 = tile * kBM, m0 = blockIdx.y * p.bn, z = blockIdx.z;
+  const int kb = (int)((int64_t)p.nks * z / p.split), nst = (int)((int64_t)p.nks * (z + 1) / p.split) - kb;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (sbase - smem_u32(smem_raw));
-  uint8_t* x_tiles = base;
-  uint8_t* c_tiles = base + kStages * kXTile;
+  const uint32_t xtile = (uint32_t)p.bn * 128u;           // bn batch rows x 64 codes of bf16 x_tilde
+  uint8_t* c_ring = base + p.stages * xtile;
   const uint32_t slab_bytes = (uint32_t)(kTileRows * p.wpg * 4);
+  const uint32_t tcols = p.bn <= 128 ? 256u : 512u;
 
   if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&full[s], 1);
+    for (int s = 0; s < kMaxStages; ++s) {
+      mbar_init(&x_full[s], 1);
       mbar_init(&empty[s], 1);
       mbar_init(&a_full[s], 4);
+    }
+    for (int s = 0; s < kCodeSlots; ++s) {
+      mbar_init(&c_full[s], 1);
+      mbar_init(&c_empty[s], kExpWarps);
     }
     mbar_init(&acc_bar, 1);
     fence_mbar_init();
   }
   if (warp == 0) {
-    tmem_alloc(&tmem_base, 512);
+    tmem_alloc(&tmem_base, tcols);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  pdl_wait();
+  // with `early` the codes (which the preceding grid does not write) start at once
+  if (!(p.early && warp == 2 + kExpWarps)) pdl_wait();
   pdl_launch_dependents();
-  call_record_start(p.rec, p.call, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0);
+  call_record_start(p.rec, p.call, blockIdx.x == 0 && blockIdx.y == 0 && z == 0 && tid == 0);
   const uint32_t tmem = tmem_base;
+  const uint32_t acol = tmem + (uint32_t)p.bn;
   bool ok = true;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // Producer: TMA of the x_tilde tile [m0, m0 + 256) x [64 ks, 64 ks + 64)
-      // (rows past M read as zeros) and the bulk copy of code slab (tile, ks).
-      for (int ks = 0; ks < p.nks && ok; ++ks) {
-        const int s = ks % kStages, r = ks / kStages;
-        if (r > 0) ok = mbar_wait(&empty[s], (r - 1) & 1);
-        if (!ok) break;
-        mbar_expect_tx(&full[s], kXTile + slab_bytes);
-        tma_load_2d(x_tiles + s * kXTile, &xmap, ks * kBK, m0, &full[s]);
-        const uint32_t* src = p.codes + (size_t)((int64_t)tile * p.ngroups + ks) * (slab_bytes / 4);
-        bulk_g2s(c_tiles + s * kCTile, src, slab_bytes, &full[s]);
-      }
+    // x_tilde tile [m0, m0 + bn) x [64 k, 64 k + 64) (rows past M read as zeros)
+    int s = 0, r = 0, i = 0;
+    for (; i < nst; ++i) {
+      if (r > 0) ok = mbar_wait_warp(&empty[s], (r - 1) & 1);
+      if (!ok) break;
+      mbar_expect_tx_warp(&x_full[s], xtile);
+      tma_load_2d_warp(base + s * xtile, &xmap, (kb + i) * kBK, m0, &x_full[s]);
+      if (++s == p.stages) { s = 0; ++r; }
     }
+    // every copy issued has landed before the CTA ends
+    for (int j = max(0, i - p.stages); j < i; ++j)
+      if (!mbar_wait_warp(&x_full[j % p.stages], (j / p.stages) & 1)) ok = false;
   } else if (warp == 1) {
-    if (lane == 0) {
-      for (int ks = 0; ks < p.nks && ok; ++ks) {
-        const int s = ks % kStages, r = ks / kStages;
-        ok = mbar_wait(&full[s], r & 1) && mbar_wait(&a_full[s], r & 1);
-        if (!ok) break;
-        tc_fence_after();
-        const uint64_t bd = sw128_desc(sbase + s * kXTile);
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.bn >> 3) << 17) |
+                           ((uint32_t)(kBM >> 4) << 24);   // D fp32, A and B bf16, both K-major
+    const uint64_t bd0 = sw128_desc(sbase);
+    int s = 0, r = 0;
+    for (int i = 0; i < nst; ++i) {
+      ok = mbar_wait_warp(&x_full[s], r & 1) && mbar_wait_warp(&a_full[s], r & 1);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t bd = bd0 + (uint64_t)((uint32_t)s * xtile >> 4);
 #pragma unroll
-        for (int kk = 0; kk < kBK / 16; ++kk)
-          umma_bf16_ts(tmem, tmem + kAcol + kAslot * s + 8 * kk, bd + 2 * kk, kIdesc, (ks | kk) != 0);
-        umma_commit(&empty[s]);
-      }
-      umma_commit(&acc_bar);
+      for (int kk = 0; kk < kBK / 16; ++kk)
+        umma_bf16_ts_warp(tmem, acol + kAslot * s + 8 * kk, bd + 2 * kk, idesc, (i | kk) != 0);
+      umma_commit_warp(&empty[s]);
+      if (++s == p.stages) { s = 0; ++r; }
     }
+    umma_commit_warp(&acc_bar);
+    if (!mbar_wait_warp(&acc_bar, 0)) ok = false;
+  } else if (warp == 2 + kExpWarps) {
+    const uint64_t pol = l2_policy_evict_first();
+    const uint8_t* src = reinterpret_cast<const uint8_t*>(p.codes) +
+                         ((size_t)tile * p.ngroups + kb) * slab_bytes;
+    const int ng = (nst + kCodeStages - 1) / kCodeStages;
+    int g = 0;
+    for (; g < ng; ++g) {
+      const int s = g % kCodeSlots, r = g / kCodeSlots;
+      if (r > 0) ok = mbar_wait_warp(&c_empty[s], (r - 1) & 1);
+      if (!ok) break;
+      const uint32_t bytes = (uint32_t)min(kCodeStages, nst - kCodeStages * g) * slab_bytes;
+      mbar_expect_tx_warp(&c_full[s], bytes);
+      if (p.M <= p.bn) bulk_g2s_hint_warp(c_ring + s * kCSlot, src, bytes, &c_full[s], pol);   // codes read once
+      else bulk_g2s_warp(c_ring + s * kCSlot, src, bytes, &c_full[s]);
+      src += kCodeStages * slab_bytes;
+    }
+    if (p.early) pdl_wait();
+    for (int j = max(0, g - kCodeSlots); j < g; ++j)
+      if (!mbar_wait_warp(&c_full[j % kCodeSlots], (j / kCodeSlots) & 1)) ok = false;
   } else {
-    // Expanders: set x = (warp - 2) / 4 expands stages ks = x (mod 2); the
+    // Expanders: set x = (warp - 2) / 4 expands stages i = x (mod 2); the
     // thread of lane quadrant q = warp % 4 expands code row 32 q + lane.
     const int x = (warp - 2) >> 2, q = warp & 3, rr = 32 * q + lane;
-    const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16);
-    for (int ks = x; ks < p.nks && ok; ks += 2) {
-      const int s = ks % kStages, r = ks / kStages;
-      ok = mbar_wait(&full[s], r & 1);                         // the code slab has landed
+    const uint32_t lane_addr = (uint32_t)(32 * q) << 16;
+    int s = x, r = 0;   // stage slot and round (stages is even)
+    for (int i = x; i < nst; i += 2) {
+      const int g = i / kCodeStages, cs = g % kCodeSlots;
+      ok = mbar_wait(&c_full[cs], (g / kCodeSlots) & 1);          // the codes have landed
       if (ok && r > 0) ok = mbar_wait(&empty[s], (r - 1) & 1);   // TMEM slot s: its MMAs are done
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      const uint8_t* cs = c_tiles + s * kCTile;
+      const uint8_t* slab = c_ring + cs * kCSlot + (i % kCodeStages) * slab_bytes;
       uint32_t v[32];
       if (p.quantizer == SDQ_TERNARY) {
         // 16 codes per word, code 2 bits: (w << 2 j) & 0xC000C000 puts two
         // codes into the sign and exponent-MSB bits of a bf16 pair (+-2 / 0)
-        const uint4 w4 = *reinterpret_cast<const uint4*>(cs + rr * 16);
+        const uint4 w4 = *reinterpret_cast<const uint4*>(slab + rr * 16);
         const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int k = 0; k < 4; ++k)
 #pragma unroll
-          for (int j = 0; j < 8; ++j) v[8 * i + j] = (w[i] << (2 * j)) & 0xC000C000u;
+          for (int j = 0; j < 8; ++j) v[8 * k + j] = (w[k] << (2 * j)) & 0xC000C000u;
       } else {   // words hold the inverted bits: 1 = -1
-        const uint2 w2 = *reinterpret_cast<const uint2*>(cs + rr * 8);
+        const uint2 w2 = *reinterpret_cast<const uint2*>(slab + rr * 8);
         const uint32_t w[2] = {~w2.x, ~w2.y};
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+        for (int k = 0; k < 2; ++k)
 #pragma unroll
-          for (int j = 0; j < 16; ++j) v[16 * i + j] = ((w[i] << j) & 0x80008000u) | 0x40004000u;
+          for (int j = 0; j < 16; ++j) v[16 * k + j] = ((w[k] << j) & 0x80008000u) | 0x40004000u;
       }
-      tmem_st32(lane_addr + kAcol + kAslot * s, v);
+      // this warp's last stage of the code slot: the slot goes back
+      if (i + 2 >= min(nst, kCodeStages * (g + 1))) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&c_empty[cs]);
+      }
+      tmem_st32(acol + lane_addr + kAslot * s, v);
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&a_full[s]);
+      s += 2;
+      if (s >= p.stages) { s -= p.stages; ++r; }
     }
     // Epilogue: TMEM lane quadrant q holds code rows n0 + 32 q + lane; this
-    // warp writes accumulator columns (batch rows) 128 x .. 128 x + 127.
+    // warp takes half of the accumulator columns (batch rows).
     if (ok) ok = mbar_wait(&acc_bar, 0);
     ok = __all_sync(0xffffffffu, ok);
     tc_fence_after();
     if (ok) {
-      const int row = n0 + rr;
-      const float sa = row < p.N ? 0.5f * __ldg(p.alpha + row) : 0.f;
-      for (int c0 = 128 * x; c0 < 128 * x + 128; c0 += 16) {
+      const int row = n0 + rr, half = (p.bn / 16 + 1) / 2 * 16;
+      const int mv = min(p.bn, p.M - m0), c1 = x ? mv : min(half, mv);
+      const float sa = p.split == 1 && row < p.N ? 0.5f * __ldg(p.alpha + row) : 0.f;
+      float* part = reinterpret_cast<float*>(base) + rr;   // [column][code row], over the drained x_tilde tiles
+      for (int c0 = x ? half : 0; c0 < c1; c0 += 16) {
         uint32_t a[16];
-        tmem_ld16(lane_addr + (uint32_t)c0, a);
+        tmem_ld16(tmem + lane_addr + (uint32_t)c0, a);
         tmem_ld_wait();
-        if (row < p.N) {
+        if (p.split > 1) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int m = m0 + c0 + i;
-            if (m < p.M) p.y[(size_t)m * p.N + row] = __uint_as_float(a[i]) * sa;
-          }
+          for (int i = 0; i < 16; ++i)
+            if (c0 + i < c1) part[(c0 + i) * kBM] = __uint_as_float(a[i]);
+        } else if (row < p.N) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (c0 + i < c1) p.y[(size_t)(m0 + c0 + i) * p.N + row] = __uint_as_float(a[i]) * sa;
         }
       }
     }
@@ -199,10 +260,96 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
-    __syncwarp();   // warp-collective: lane 0 ran the producer loop alone
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc(tmem, tcols);
   }
+  if (p.split == 1) return;
+  // The cluster's partial sums, in CTA order: CTA z adds columns z, z + S, ...
+  // of all S accumulators, a warp one column (128 code rows) at a time.
+  cluster_sync();
+  {
+    const int mv = min(p.bn, p.M - m0), row = n0 + 4 * lane;
+    float al[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) al[i] = row + i < p.N ? 0.5f * __ldg(p.alpha + row + i) : 0.f;
+    const bool vec = (p.N & 3) == 0 && row + 3 < p.N;
+    for (int c = z + p.split * warp; c < mv; c += p.split * (kThreads / 32)) {
+      const uint32_t a = sbase + (uint32_t)(c * kBM + 4 * lane) * 4u;
+      float4 v[kMaxSplit];
+#pragma unroll
+      for (int i = 0; i < kMaxSplit; ++i)
+        if (i < p.split) v[i] = ld_cluster4(a, (uint32_t)i);
+      float4 t = v[0];
+#pragma unroll
+      for (int i = 1; i < kMaxSplit; ++i)
+        if (i < p.split) { t.x += v[i].x; t.y += v[i].y; t.z += v[i].z; t.w += v[i].w; }
+      float* o = p.y + (size_t)(m0 + c) * p.N + row;
+      if (vec) {
+        *reinterpret_cast<float4*>(o) = make_float4(t.x * al[0], t.y * al[1], t.z * al[2], t.w * al[3]);
+      } else {
+        if (row < p.N) o[0] = t.x * al[0];
+        if (row + 1 < p.N) o[1] = t.y * al[1];
+        if (row + 2 < p.N) o[2] = t.z * al[2];
+        if (row + 3 < p.N) o[3] = t.w * al[3];
+      }
+    }
+  }
+  cluster_sync();   // no CTA ends while its accumulator is being read
+}
+
+// Launch shape at batch M: the batch in equal tiles of bn rows, S k chunks.
+// Time model in ns, fitted to forced splits of LLaMA-7B linears at M = 65 ..
+// 500 (within ~10 % of them): a stage takes its MMAs (1.09 bn, one CTA per
+// SM) or its code expansion (165 + bn / 4 alone on an SM, 230 + 0.7 bn with
+// two CTAs there); a CTA adds a prologue and an epilogue, a split one the
+// cluster's sum.  CTAs run in waves of what the device holds of such
+// clusters; with two per SM the last wave overlaps the one before.
+struct PrefillShape {
+  int bn, mt, stages, split, smem;
+};
+constexpr int kFixedSmem = 1024 + kCodeSlots * kCSlot;
+PrefillShape prefill_shape(const sdq_plan_s* pl, int M) {
+  const Geometry& g = pl->geo;
+  PrefillShape s{};
+  s.mt = (M + 255) / 256;
+  s.bn = ((M + s.mt - 1) / s.mt + 15) / 16 * 16;
+  const int occ = s.bn <= 128 ? 2 : 1;
+  const int by_smem = (kSmemSm / occ - 1024 - kFixedSmem) / (s.bn * 128);   // 1 KB a block for the static part
+  const int by_tmem = ((occ == 2 ? 256 : 512) - s.bn) / (int)kAslot;
+  s.stages = std::min(kMaxStages, std::min(by_smem, by_tmem)) & ~1;
+  const int64_t nks = g.k_eff_pad / kBK, tiles = (int64_t)g.ntiles * s.mt;
+  double best = 0;
+  for (int S = 1; S <= kMaxSplit && S <= nks; ++S) {
+    const int64_t held = (int64_t)occ * std::max(1, pl->pf_clusters[S]);
+    const double x = (double)tiles / held, up = (double)((tiles + held - 1) / held);
+    const double waves = occ == 2 ? std::max(1.0, 0.5 * (x + up)) : up;
+    const bool shared = occ == 2 && tiles * S > pl->sm_count;
+    const double stage = std::max(1.09 * s.bn, shared ? 230.0 + 0.7 * s.bn : 165.0 + 0.25 * s.bn);
+    const double t = waves * ((S == 1 ? 4100.0 : 5900.0 + 400.0 * S) + (double)((nks + S - 1) / S) * stage);
+    if (S == 1 || t < best * 0.98) {
+      best = t;
+      s.split = S;
+    }
+  }
+  s.smem = kFixedSmem + std::max(s.stages * s.bn * 128, s.split > 1 ? s.bn * kBM * 4 - kCodeSlots * kCSlot : 0);
+  return s;
+}
+constexpr int kPfSmemLimit = kSmemSm - 1024;
+
+void prefill_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, dim3 grid, int smem, cudaStream_t st) {
+  *cfg = {};
+  cfg->gridDim = grid;
+  cfg->blockDim = dim3(kThreads);
+  cfg->dynamicSmemBytes = (size_t)smem;
+  cfg->stream = st;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 1;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = grid.z;
+  cfg->attrs = attr;
+  cfg->numAttrs = grid.z > 1 ? 2 : 1;
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -217,6 +364,11 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
       fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
   });
   return fn;
+}
+
+cudaError_t prefill_smem_limit(int device) {
+  static std::atomic<int> smem_set[64];   // per device: limit raised to the largest shape's
+  return smem_limit_once(prefill_kernel, kPfSmemLimit, device, smem_set);
 }
 
 // ------------------------------------------ prefill prepare, tensor cores
@@ -415,18 +567,19 @@ __global__ void __launch_bounds__(kPtThreads, 1)
 void* tensor_map_encoder() { return reinterpret_cast<void*>(encode_fn()); }
 
 cudaError_t launch_prefill(const sdq_plan_s* pl, const uint32_t* codes, const float* alpha, int M,
-                           float* y, void* ws, cudaStream_t st) {
+                           float* y, void* ws, cudaStream_t st, int early) {
   const Geometry& g = pl->geo;
   const WsLayout L = workspace_layout(pl, M);
   uint8_t* wbase = static_cast<uint8_t*>(ws);
   auto enc = encode_fn();
   if (!enc) return cudaErrorNotSupported;
-  CUtensorMap amap;
+  const PrefillShape sh = prefill_shape(pl, M);
+  CUtensorMap xmap;
   const cuuint64_t dims[2] = {(cuuint64_t)g.k_eff_pad, (cuuint64_t)M};
   const cuuint64_t strides[1] = {(cuuint64_t)g.k_eff_pad * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kBN};
+  const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)sh.bn};
   const cuuint32_t estr[2] = {1, 1};
-  CUresult cr = enc(&amap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, wbase + L.xt, dims, strides, box, estr,
+  CUresult cr = enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, wbase + L.xt, dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) return cudaErrorInvalidValue;
@@ -434,15 +587,33 @@ cudaError_t launch_prefill(const sdq_plan_s* pl, const uint32_t* codes, const fl
   p.codes = codes; p.alpha = alpha; p.y = y;
   p.rec = reinterpret_cast<uint64_t*>(wbase + L.err);
   p.call = call_tag(next_call_number());
-  p.M = M; p.N = g.n_out; p.ntiles = g.ntiles; p.ngroups = g.ngroups; p.wpg = g.wpg;
+  p.M = M; p.N = g.n_out; p.ngroups = g.ngroups; p.wpg = g.wpg;
   p.nks = (int)(g.k_eff_pad / kBK);
   p.quantizer = pl->desc.quantizer;
-  cudaError_t e = cudaFuncSetAttribute(prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  p.bn = sh.bn; p.stages = sh.stages; p.split = sh.split; p.early = early;
+  cudaError_t e = prefill_smem_limit(pl->device);
   if (e != cudaSuccess) return e;
-  dim3 grid(g.ntiles, (M + kBN - 1) / kBN);
-  return launch_pdl(prefill_kernel, grid, dim3(kThreads), (size_t)kSmem, st, amap, p);
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  prefill_config(&cfg, attr, dim3(g.ntiles, sh.mt, sh.split), sh.smem, st);
+  return cudaLaunchKernelEx(&cfg, prefill_kernel, xmap, p);
 }
 
+// Clusters of S CTAs, one CTA per SM, that the device holds at once (GPCs of
+// different sizes leave SMs over: asked, not computed).
+cudaError_t prefill_occupancy(sdq_plan_s* pl) {
+  cudaError_t e = prefill_smem_limit(pl->device);
+  pl->pf_clusters[1] = pl->sm_count;
+  for (int S = 2; S <= kMaxSplit && e == cudaSuccess; ++S) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    prefill_config(&cfg, attr, dim3(1, 1, S), kPfSmemLimit - 1024, 0);
+    cfg.attrs = attr + 1;   // the cluster alone
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&pl->pf_clusters[S], prefill_kernel, &cfg);
+  }
+  return e;
+}
 
 // The prefill prepare kernel on the tensor cores where it applies (B = 128,
 // n_b a multiple of 64, x 16-byte aligned), one launch per 256 or fewer of
