@@ -28,16 +28,17 @@
 //   D (TMEM)  fp32, 128 lanes x NP columns
 // so that y[m, r] = alpha_r / 2 * sum_t D[r, m T + t].
 //
-// Issuing one of these MMAs occupies the issuing thread for about 130 cycles
-// whatever N is, while MMAs issued from different warps proceed side by
-// side; so the stages (sb <= 4 blocks of 128 codes each, 2 sb MMAs: large
-// stages, since every stage costs each thread it passes through a few
-// hundred cycles of waits and signals) of a row tile
-// are dealt round-robin to `npipe` (1, 2 or 4) MMA pipelines, each with its
-// own issuing warp and accumulator, and the epilogue adds the pipelines'
-// accumulators.  Stage i of the CTA uses
+// MMAs issued from different warps proceed side by side; so the stages (sb <=
+// 4 blocks of 128 codes each, 2 sb MMAs: large stages, since every stage costs
+// each warp it passes through a few hundred cycles of waits and signals) of a
+// row tile are dealt round-robin to `npipe` (1, 2 or 4) MMA pipelines, each
+// with its own issuing warp and accumulator, and the epilogue adds the
+// pipelines' accumulators.  The issuing and copying warps stay converged
+// (common.cuh: *_warp): from a divergent lane an MMA took its thread 130 - 270
+// cycles and a copy about 600, and the LLaMA-70B layer at M = 1 115 us (102
+// converged), the LLaMA-7B layer at M = 64 178 (159).  Stage i of the CTA uses
 //   ring slot i mod ring      (codes in shared memory; ring a multiple of 4)
-//   producer i mod 4          (one thread issuing its bulk copies)
+//   producer i mod 4          (one warp issuing its bulk copies)
 //   expander set i mod 4      (4 warps, one per TMEM lane quadrant)
 //   TMEM A slot i mod ns      (ns = 4 or 8 slots of 16 sb columns: with 4,
 //                             each expander set refills its one slot once
@@ -48,7 +49,7 @@
 // phases in order.
 //
 // CTA (k chunk s, row set p) of one SM, 28 warps:
-//   warps 0..3    lane 0 of warp e issues pipeline e's MMAs (e < npipe),
+//   warps 0..3    warp e issues pipeline e's MMAs (e < npipe),
 //                 commits to the stage's TMEM slot and, after its last stage
 //                 of a row tile, to its accumulator; warp 0 also owns the
 //                 TMEM allocation
@@ -61,11 +62,9 @@
 //                 order (deterministic: sdq_contract)
 //   warps 8..23   first the B operand and its scales, then the expanders:
 //                 set x (warps 8 + 4x .. 11 + 4x) expands stages i = x mod 4
-//   warps 24..27  lane 0 of warp 24 + x streams stages i = x mod 4 (one
-//                 128-row tile x sb * 128 codes = contiguous slabs of the
-//                 tiled layout) into the ring with bulk copies: a thread
-//                 starts a bulk copy only every ~600 cycles, four side by
-//                 side keep an SM's share of HBM busy
+//   warps 24..27  warp 24 + x streams stages i = x mod 4 (one 128-row tile x
+//                 sb * 128 codes = contiguous slabs of the tiled layout)
+//                 into the ring with bulk copies
 // With `early` set the producers start the code stream (one stage each)
 // before waiting for the preceding grid (codes are never written by the
 // prep kernels), except with bstream, where each stage also copies B rows
@@ -237,7 +236,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
   __shared__ int sblk[kMaxSpu + 1];         // first block of stage j of a tile
   __shared__ float s_alpha[kAlphaAhead][kTileRows];   // epilogue: alpha of the next row tiles
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int sidx = blockIdx.x % p.S, prow = blockIdx.x / p.S;
   const int kb0 = sidx * p.CB;
   const int ncb = min(p.CB, p.KB - kb0);                        // blocks of this chunk
@@ -308,63 +307,61 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
   bool ok = true;
 
   if (warp >= kProducerWarp0) {
-    if (lane == 0) {
-      // Producer x: stages i = x (mod 4), stage i = (unit u, j) being the
-      // slabs (tile, 2 b) .. (tile, 2 b' - 1) of its blocks [b, b'), adjacent
-      // in the tiled layout, into ring slot i mod ring (round r = i / ring).
-      const int x = warp - kProducerWarp0;
-      int last_i = -1, u = 0, j = x, slot = x, r = 0;
-      while (j >= spu) { j -= spu; ++u; }
-      const uint64_t pol = l2_policy_evict_first();   // codes are read once per call
-      bool waited = !early;
-      for (int i = x; i < nstages && ok; i += kExpSets) {
-        // with `early`, kEarlyStages stages ahead of the preceding grid: more
-        // would queue ahead of the loads that grid and this CTA's prologue
-        // make once it completes
-        if (!waited && i >= x + kExpSets * kEarlyStages) { pdl_wait(); waited = true; }
-        if (r > 0) ok = mbar_wait(&c_empty[slot], (r - 1) & 1);
-        if (!ok) break;
-        const int b0 = sblk[j], b1 = sblk[j + 1];
-        const int tile = prow + (u + rot < nunits ? u + rot : u + rot - nunits) * p.P;
-        const uint8_t* src = reinterpret_cast<const uint8_t*>(p.codes) +
-                             ((size_t)tile * p.KB + kb0 + b0) * p.blk_bytes;
-        const uint32_t bytes = (uint32_t)(b1 - b0) * p.blk_bytes;
-        uint8_t* dst = ring + (size_t)slot * p.slot_bytes;
-        if (p.bstream) {
-          // the stage's image pairs and scale words (L2 hits: the prepare
-          // kernel wrote them, every CTA of the k chunk reads them)
-          const int pa0 = (kb0 + b0) >> 1, pa1 = (kb0 + b1 + 1) >> 1;
-          const uint32_t bb = (uint32_t)(pa1 - pa0) * (uint32_t)p.NP * 128u;
-          const uint32_t sbytes = (uint32_t)(b1 - b0) * (uint32_t)p.NP * 4u;
-          mbar_expect_tx(&c_full[slot], bytes + bb + sbytes);
-          bulk_g2s_hint(dst, src, bytes, &c_full[slot], pol);
-          bulk_g2s(dst + p.boff, p.bimg + (size_t)pa0 * p.NP * 128, bb, &c_full[slot]);
-          bulk_g2s(dst + p.soff, p.sfbw + (size_t)(kb0 + b0) * p.NP * 4, sbytes, &c_full[slot]);
-        } else {
-          mbar_expect_tx(&c_full[slot], bytes);
-          bulk_g2s_hint(dst, src, bytes, &c_full[slot], pol);
-        }
-        last_i = i;
-        j += kExpSets;
-        while (j >= spu) { j -= spu; ++u; }
-        slot += kExpSets;
-        if (slot >= p.ring) { slot -= p.ring; ++r; }
+    // Producer x: stages i = x (mod 4), stage i = (unit u, j) being the
+    // slabs (tile, 2 b) .. (tile, 2 b' - 1) of its blocks [b, b'), adjacent
+    // in the tiled layout, into ring slot i mod ring (round r = i / ring).
+    const int x = warp - kProducerWarp0;
+    int last_i = -1, u = 0, j = x, slot = x, r = 0;
+    while (j >= spu) { j -= spu; ++u; }
+    const uint64_t pol = l2_policy_evict_first();   // codes are read once per call
+    bool waited = !early;
+    for (int i = x; i < nstages && ok; i += kExpSets) {
+      // with `early`, kEarlyStages stages ahead of the preceding grid: more
+      // would queue ahead of the loads that grid and this CTA's prologue
+      // make once it completes
+      if (!waited && i >= x + kExpSets * kEarlyStages) { pdl_wait(); waited = true; }
+      if (r > 0) ok = mbar_wait_warp(&c_empty[slot], (r - 1) & 1);
+      if (!ok) break;
+      const int b0 = sblk[j], b1 = sblk[j + 1];
+      const int tile = prow + (u + rot < nunits ? u + rot : u + rot - nunits) * p.P;
+      const uint8_t* src = reinterpret_cast<const uint8_t*>(p.codes) +
+                           ((size_t)tile * p.KB + kb0 + b0) * p.blk_bytes;
+      const uint32_t bytes = (uint32_t)(b1 - b0) * p.blk_bytes;
+      uint8_t* dst = ring + (size_t)slot * p.slot_bytes;
+      if (p.bstream) {
+        // the stage's image pairs and scale words (L2 hits: the prepare
+        // kernel wrote them, every CTA of the k chunk reads them)
+        const int pa0 = (kb0 + b0) >> 1, pa1 = (kb0 + b1 + 1) >> 1;
+        const uint32_t bb = (uint32_t)(pa1 - pa0) * (uint32_t)p.NP * 128u;
+        const uint32_t sbytes = (uint32_t)(b1 - b0) * (uint32_t)p.NP * 4u;
+        mbar_expect_tx_warp(&c_full[slot], bytes + bb + sbytes);
+        bulk_g2s_hint_warp(dst, src, bytes, &c_full[slot], pol);
+        bulk_g2s_warp(dst + p.boff, p.bimg + (size_t)pa0 * p.NP * 128, bb, &c_full[slot]);
+        bulk_g2s_warp(dst + p.soff, p.sfbw + (size_t)(kb0 + b0) * p.NP * 4, sbytes, &c_full[slot]);
+      } else {
+        mbar_expect_tx_warp(&c_full[slot], bytes);
+        bulk_g2s_hint_warp(dst, src, bytes, &c_full[slot], pol);
       }
-      if (!waited) pdl_wait();
-      // Every copy this thread issued has landed before the CTA may exit.
-      for (int i = last_i; i >= 0 && i > last_i - p.ring; i -= kExpSets)
-        if (!mbar_wait(&c_full[i % p.ring], (i / p.ring) & 1)) ok = false;
+      last_i = i;
+      j += kExpSets;
+      while (j >= spu) { j -= spu; ++u; }
+      slot += kExpSets;
+      if (slot >= p.ring) { slot -= p.ring; ++r; }
     }
+    if (!waited) pdl_wait();
+    // Every copy this warp issued has landed before the CTA may exit.
+    for (int i = last_i; i >= 0 && i > last_i - p.ring; i -= kExpSets)
+      if (!mbar_wait_warp(&c_full[i % p.ring], (i / p.ring) & 1)) ok = false;
   } else if (warp < kMaxPipes) {
-    if (lane == 0 && warp < np) {
+    if (warp < np) {
       // MMA issuer of pipeline e: stages i = e (mod np) in order, stage i's
       // codes in TMEM slot i mod 8, into the pipeline's accumulator.
       const int e = warp;
-      ok = mbar_wait(&b_full, 0);
+      ok = mbar_wait_warp(&b_full, 0);
       tc_fence_after();
       const uint32_t idesc0 = mxf4_idesc(p.NP), idesc1 = idesc0 | (2u << 4);   // B scale bytes 0-1 / 2-3
       // Per stage: one wait, 2 nb MMAs, one commit; stage bookkeeping is
-      // kept incremental (a single thread's scalar latency is on the path).
+      // kept incremental (the issuing warp's scalar latency is on the path).
       const uint64_t bd0 = sw128_desc(sbase);
       const uint32_t ring_s = smem_u32(ring);
       const uint64_t astep = (uint64_t)((p.brow * 128) >> 4);   // descriptor units per image row pair
@@ -378,13 +375,13 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
         if (first) {
           buf = p.nbuf == 2 ? (k & 1) : 0;
           if (k >= p.nbuf) {
-            ok = mbar_wait(&acc_empty[e][buf], ((k / p.nbuf) - 1) & 1);
+            ok = mbar_wait_warp(&acc_empty[e][buf], ((k / p.nbuf) - 1) & 1);
             if (!ok) break;
           }
           dt = tmem + (uint32_t)(p.dbase + (e * p.nbuf + buf) * p.NP);
         }
         const int s = i & (p.ns - 1);
-        ok = mbar_wait(&a_full[s], (i >> p.ns_log2) & 1);
+        ok = mbar_wait_warp(&a_full[s], (i >> p.ns_log2) & 1);
         if (!ok) break;
         tc_fence_after();
         const int b0 = sblk[j], nb = sblk[j + 1] - b0;
@@ -398,27 +395,27 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
         for (int bb = 0; bb < nb; ++bb, at += kAColsPerBlk, sfb += (uint32_t)p.ss) {
           const int bl = b0 + bb, kb = kb0 + bl;
           const uint64_t bd = bdb + (uint64_t)((kb >> 1) - pbase) * astep + 4u * (uint32_t)(kb & 1);
-          umma_mxf4_ts(dt, at, bd, idesc0, sfa, sfb, (first && bb == 0) ? 0u : 1u);
-          umma_mxf4_ts(dt, at + 8, bd + 2, idesc1, sfa, sfb, 1u);
+          umma_mxf4_ts_warp(dt, at, bd, idesc0, sfa, sfb, (first && bb == 0) ? 0u : 1u);
+          umma_mxf4_ts_warp(dt, at + 8, bd + 2, idesc1, sfa, sfb, 1u);
         }
-        umma_commit(&a_empty[s]);
-        if (p.bstream) umma_commit(&c_empty[rslot]);
+        umma_commit_warp(&a_empty[s]);
+        if (p.bstream) umma_commit_warp(&c_empty[rslot]);
         last = i;
         const int u0 = u;
         j += np;
         while (j >= spu) { j -= spu; ++u; }
         first = u != u0;
         if (first) {   // this pipeline's last stage of the tile
-          umma_commit(&acc_full[e][buf]);
+          umma_commit_warp(&acc_full[e][buf]);
           ++k;
         }
       }
-      umma_commit(&mma_done[e]);   // every MMA issued has finished before TMEM is freed
-      if (!mbar_wait(&mma_done[e], 0)) ok = false;
+      umma_commit_warp(&mma_done[e]);   // every MMA issued has finished before TMEM is freed
+      if (!mbar_wait_warp(&mma_done[e], 0)) ok = false;
       // ... and the last commit to each of this pipeline's TMEM slots has
       // arrived (those phases have no other waiter).
       for (int i = last; i >= 0 && i > last - p.ns; i -= np)
-        if (!mbar_wait(&a_empty[i & (p.ns - 1)], (i >> p.ns_log2) & 1)) ok = false;
+        if (!mbar_wait_warp(&a_empty[i & (p.ns - 1)], (i >> p.ns_log2) & 1)) ok = false;
     }
   } else if (warp >= kExpWarp0) {
     // ------------------------------------------------ builders, then expanders
@@ -802,7 +799,6 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
     }
   }
   if (warp == 0) {
-    __syncwarp();   // warp-collective: lane 0 ran the issuer loop alone
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }

@@ -18,8 +18,8 @@
 // (row tile, block) item, two of them so that an item's epilogue (bf16 W',
 // 16-byte stores) overlaps the next item's MMAs.  Persistent CTAs over the
 // items.
-//   warp 0     TMEM allocation; lane 0: G^T once (TMA), then the code slabs
-//   warp 1     lane 0: 8 MMAs per 64 codes (4 K steps x hi / lo)
+//   warp 0     TMEM allocation; G^T once (TMA), then the code slabs
+//   warp 1     8 MMAs per 64 codes (4 K steps x hi / lo)
 //   warps 2-9  two expander sets (stages of one parity each)
 //   warps 10-13 epilogue
 // K7: a plain tcgen05 GEMM, D[r, m] = W' x^T per CTA tile of 128 (or 2 x 128)
@@ -40,14 +40,6 @@ namespace sdq {
 namespace {
 
 constexpr int kBK = 64;                    // codes (K6) or inputs (K7) per stage
-
-__device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
 
 // kind::f16 instruction descriptor: D fp32, A and B bf16, both K-major,
 // M = 128, N = n.
@@ -79,7 +71,7 @@ __global__ void __launch_bounds__(kRbThreads, 1)
   __shared__ __align__(8) uint64_t g_full, full[kRbStages], empty[kRbStages], a_full[kRbStages],
       acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (sbase - smem_u32(smem_raw));
   const int spb = p.n_b / kBK;                        // stages (64-code chunks) per block
@@ -116,49 +108,45 @@ __global__ void __launch_bounds__(kRbThreads, 1)
   const int nst = nmine * spb;
 
   if (warp == 0) {
-    if (lane == 0) {
-      mbar_expect_tx(&g_full, 2u * spb * gchunk);
-      for (int c = 0; c < spb; ++c) {
-        tma_load_2d(base + c * gchunk, &ghmap, c * kBK, 0, &g_full);
-        tma_load_2d(base + (spb + c) * gchunk, &glmap, c * kBK, 0, &g_full);
-      }
-      for (int i = 0; i < nst && ok; ++i) {
-        const int s = i % kRbStages, r = i / kRbStages;
-        const int item = (int)blockIdx.x + (i / spb) * (int)gridDim.x, sc = i % spb;
-        const int tile = item / p.nblk, b = item - tile * p.nblk;
-        if (r > 0) ok = mbar_wait(&empty[s], (r - 1) & 1);
-        if (!ok) break;
-        mbar_expect_tx(&full[s], slab_bytes);
-        const uint32_t* src = p.codes + (size_t)((int64_t)tile * p.ngroups + b * spb + sc) * (slab_bytes / 4);
-        bulk_g2s(c_tiles + s * kRbCTile, src, slab_bytes, &full[s]);
-      }
+    mbar_expect_tx_warp(&g_full, 2u * spb * gchunk);
+    for (int c = 0; c < spb; ++c) {
+      tma_load_2d_warp(base + c * gchunk, &ghmap, c * kBK, 0, &g_full);
+      tma_load_2d_warp(base + (spb + c) * gchunk, &glmap, c * kBK, 0, &g_full);
+    }
+    for (int i = 0; i < nst && ok; ++i) {
+      const int s = i % kRbStages, r = i / kRbStages;
+      const int item = (int)blockIdx.x + (i / spb) * (int)gridDim.x, sc = i % spb;
+      const int tile = item / p.nblk, b = item - tile * p.nblk;
+      if (r > 0) ok = mbar_wait_warp(&empty[s], (r - 1) & 1);
+      if (!ok) break;
+      mbar_expect_tx_warp(&full[s], slab_bytes);
+      const uint32_t* src = p.codes + (size_t)((int64_t)tile * p.ngroups + b * spb + sc) * (slab_bytes / 4);
+      bulk_g2s_warp(c_tiles + s * kRbCTile, src, slab_bytes, &full[s]);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = f16_idesc(128);
-      ok = mbar_wait(&g_full, 0);
-      for (int i = 0; i < nst && ok; ++i) {
-        const int s = i % kRbStages, r = i / kRbStages;
-        const int it = i / spb, sc = i % spb, a = it & 1;
-        if (sc == 0 && it >= 2) {
-          ok = mbar_wait(&acc_empty[a], ((it >> 1) - 1) & 1);
-          if (!ok) break;
-        }
-        ok = mbar_wait(&full[s], r & 1) && mbar_wait(&a_full[s], r & 1);
+    constexpr uint32_t idesc = f16_idesc(128);
+    ok = mbar_wait_warp(&g_full, 0);
+    for (int i = 0; i < nst && ok; ++i) {
+      const int s = i % kRbStages, r = i / kRbStages;
+      const int it = i / spb, sc = i % spb, a = it & 1;
+      if (sc == 0 && it >= 2) {
+        ok = mbar_wait_warp(&acc_empty[a], ((it >> 1) - 1) & 1);
         if (!ok) break;
-        tc_fence_after();
-        const uint64_t bh = sw128_desc(sbase + sc * gchunk);
-        const uint64_t bl = sw128_desc(sbase + (spb + sc) * gchunk);
-        const uint32_t d = tmem + (uint32_t)a * kRbAcc;
-#pragma unroll
-        for (int kk = 0; kk < kBK / 16; ++kk) {
-          const uint32_t at = tmem + kRbAcol + kRbAslot * s + 8 * kk;
-          umma_f16_ts(d, at, bh + 2 * kk, idesc, (sc | kk) != 0);
-          umma_f16_ts(d, at, bl + 2 * kk, idesc, 1u);
-        }
-        umma_commit(&empty[s]);
-        if (sc == spb - 1) umma_commit(&acc_full[a]);
       }
+      ok = mbar_wait_warp(&full[s], r & 1) && mbar_wait_warp(&a_full[s], r & 1);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t bh = sw128_desc(sbase + sc * gchunk);
+      const uint64_t bl = sw128_desc(sbase + (spb + sc) * gchunk);
+      const uint32_t d = tmem + (uint32_t)a * kRbAcc;
+#pragma unroll
+      for (int kk = 0; kk < kBK / 16; ++kk) {
+        const uint32_t at = tmem + kRbAcol + kRbAslot * s + 8 * kk;
+        umma_bf16_ts_warp(d, at, bh + 2 * kk, idesc, (sc | kk) != 0);
+        umma_bf16_ts_warp(d, at, bl + 2 * kk, idesc, 1u);
+      }
+      umma_commit_warp(&empty[s]);
+      if (sc == spb - 1) umma_commit_warp(&acc_full[a]);
     }
   } else if (warp < kRbEpiWarp0) {
     // Expanders: set x = (warp - 2) / 4 expands stages i = x (mod 2), thread
@@ -241,7 +229,6 @@ __global__ void __launch_bounds__(kRbThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
-    __syncwarp();   // warp-collective: lane 0 ran the producer loop alone
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
@@ -282,7 +269,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[kStages], empty[kStages], acc_bar;
   __shared__ uint32_t tmem_base;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   int unit = blockIdx.x, nt = WT, sub = 0;
   if (unit >= p.nfull) {
     sub = (unit - p.nfull) % WT;
@@ -313,41 +300,37 @@ __global__ void __launch_bounds__(kDnThreads, 1)
   const uint32_t tmem = tmem_base;
   bool ok = true;
   if (warp == 0) {
-    if (lane == 0) {
-      for (int ks = 0; ks < p.nks && ok; ++ks) {
-        const int s = ks % kStages, r = ks / kStages;
-        if (r > 0) ok = mbar_wait(&empty[s], (r - 1) & 1);
-        if (!ok) break;
-        mbar_expect_tx(&full[s], (uint32_t)(nt * kDnATile + kDnBTile));
-        uint8_t* st = base + s * kStage;
+    for (int ks = 0; ks < p.nks && ok; ++ks) {
+      const int s = ks % kStages, r = ks / kStages;
+      if (r > 0) ok = mbar_wait_warp(&empty[s], (r - 1) & 1);
+      if (!ok) break;
+      mbar_expect_tx_warp(&full[s], (uint32_t)(nt * kDnATile + kDnBTile));
+      uint8_t* st = base + s * kStage;
 #pragma unroll
-        for (int w = 0; w < WT; ++w)
-          if (w < nt) tma_load_2d(st + w * kDnATile, &wmap, ks * kBK, n0 + 128 * w, &full[s]);
-        tma_load_2d(st + WT * kDnATile, &xmap, ks * kBK, m0, &full[s]);
-      }
+      for (int w = 0; w < WT; ++w)
+        if (w < nt) tma_load_2d_warp(st + w * kDnATile, &wmap, ks * kBK, n0 + 128 * w, &full[s]);
+      tma_load_2d_warp(st + WT * kDnATile, &xmap, ks * kBK, m0, &full[s]);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = f16_idesc(kDnBN);
-      for (int ks = 0; ks < p.nks && ok; ++ks) {
-        const int s = ks % kStages, r = ks / kStages;
-        ok = mbar_wait(&full[s], r & 1);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t st = sbase + s * kStage;
-        const uint64_t bd = sw128_desc(st + WT * kDnATile);
+    constexpr uint32_t idesc = f16_idesc(kDnBN);
+    for (int ks = 0; ks < p.nks && ok; ++ks) {
+      const int s = ks % kStages, r = ks / kStages;
+      ok = mbar_wait_warp(&full[s], r & 1);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t st = sbase + s * kStage;
+      const uint64_t bd = sw128_desc(st + WT * kDnATile);
 #pragma unroll
-        for (int w = 0; w < WT; ++w) {
-          if (w >= nt) break;
-          const uint64_t ad = sw128_desc(st + w * kDnATile);
+      for (int w = 0; w < WT; ++w) {
+        if (w >= nt) break;
+        const uint64_t ad = sw128_desc(st + w * kDnATile);
 #pragma unroll
-          for (int kk = 0; kk < kBK / 16; ++kk)
-            umma_bf16(tmem + (uint32_t)(w * kDnBN), ad + 2 * kk, bd + 2 * kk, idesc, (ks | kk) != 0);
-        }
-        umma_commit(&empty[s]);
+        for (int kk = 0; kk < kBK / 16; ++kk)
+          umma_bf16_warp(tmem + (uint32_t)(w * kDnBN), ad + 2 * kk, bd + 2 * kk, idesc, (ks | kk) != 0);
       }
-      umma_commit(&acc_bar);
+      umma_commit_warp(&empty[s]);
     }
+    umma_commit_warp(&acc_bar);
   } else {
     // Epilogue: lane quadrant q holds weight rows n0 + 128 w + 32 q + lane of
     // accumulator w; this warp writes its columns (batch rows) 128 h .. 128 h + 127.
@@ -380,7 +363,6 @@ __global__ void __launch_bounds__(kDnThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
-    __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, DnShape<WT>::kCols);
   }

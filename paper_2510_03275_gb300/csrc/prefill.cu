@@ -16,9 +16,8 @@
 // multiple of 16 up to 256: the batch in equal tiles), 64 codes per pipeline
 // stage; a cluster of S CTAs splits K, and the sum of its S accumulators goes
 // through distributed shared memory in CTA order (the same bits every run):
-//   warp 0      TMEM allocation; lane 0 issues the TMA loads of the stages'
-//               x_tilde tiles
-//   warp 1      lane 0 issues tcgen05.mma (4 x K = 16 per stage, A from the
+//   warp 0      TMEM allocation; the TMA loads of the stages' x_tilde tiles
+//   warp 1      issues tcgen05.mma (4 x K = 16 per stage, A from the
 //               stage's TMEM slot), commits to the stage's "empty" barrier,
 //               finally to the accumulator one
 //   warps 2..9  two expander sets (set x expands the stages of parity x),
@@ -26,7 +25,7 @@
 //               bf16 pairs (one x32 store); then the epilogue: accumulator
 //               column m -> y[m, r] scaled by alpha_r / 2, each warp one lane
 //               quadrant and half of the columns
-//   warp 10     lane 0 streams the codes, 4 stages (tiled layout: 4 slabs of
+//   warp 10     streams the codes, 4 stages (tiled layout: 4 slabs of
 //               128 rows x 64 codes, contiguous) per bulk copy, into a ring
 //               of its own that runs ahead of the x_tilde stages: codes come
 //               from HBM, x_tilde from the L2
@@ -379,10 +378,10 @@ cudaError_t prefill_smem_limit(int device) {
 // into bf16 hi and lo parts accumulated into the same fp32 accumulator (the
 // pair carries G to ~2^-16; x is bf16, exact).  Persistent CTAs, one per SM,
 // over tiles of 128 rows:
-//   warp 0     TMEM allocation (two accumulators of n_b columns); lane 0
+//   warp 0     TMEM allocation (two accumulators of n_b columns);
 //              loads G hi / lo once, then the x tiles into a 3-slot ring
 //              (TMA, 128-byte swizzle: the canonical K-major operand layout)
-//   warp 1     lane 0 issues each tile's 16 MMAs into accumulator t mod 2
+//   warp 1     issues each tile's 16 MMAs into accumulator t mod 2
 //   warps 2-9  epilogue, two warps per TMEM lane quadrant (half of the n_b
 //              columns each): bf16 x_tilde (round to nearest even) in the
 //              prefill operand order (prefill_pos64) with 16-byte stores;
@@ -410,7 +409,7 @@ __global__ void __launch_bounds__(kPtThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t g_full, x_full[kPtSlots], x_empty[kPtSlots], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (sbase - smem_u32(smem_raw));
   const uint32_t gchunk = (uint32_t)p.ncol * 128u;  // one 64-wide K chunk of G^T: ncol rows x 128 B
@@ -442,53 +441,49 @@ __global__ void __launch_bounds__(kPtThreads, 1)
   bool ok = true;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // G (the plan's table, never written by the stream) before the wait
-      // for the preceding grid; x and the workspace after it
-      mbar_expect_tx(&g_full, 4 * gchunk);
-      for (int c = 0; c < 2; ++c) {
-        tma_load_2d(gh + c * gchunk, &ghmap, 64 * c, 0, &g_full);
-        tma_load_2d(gl + c * gchunk, &glmap, 64 * c, 0, &g_full);
-      }
-      pdl_wait();
-      pdl_launch_dependents();
-      int i = 0;
-      for (int t = blockIdx.x; t < p.ntile && ok; t += gridDim.x, ++i) {
-        const int s = i % kPtSlots, r = i / kPtSlots;
-        if (r > 0) ok = mbar_wait(&x_empty[s], (r - 1) & 1);
-        if (!ok) break;
-        mbar_expect_tx(&x_full[s], kPtXTile);
-        tma_load_2d(xs + s * kPtXTile, &xmap, 0, t * kPtRows, &x_full[s]);
-        tma_load_2d(xs + s * kPtXTile + kPtXTile / 2, &xmap, 64, t * kPtRows, &x_full[s]);
-      }
+    // G (the plan's table, never written by the stream) before the wait
+    // for the preceding grid; x and the workspace after it
+    mbar_expect_tx_warp(&g_full, 4 * gchunk);
+    for (int c = 0; c < 2; ++c) {
+      tma_load_2d_warp(gh + c * gchunk, &ghmap, 64 * c, 0, &g_full);
+      tma_load_2d_warp(gl + c * gchunk, &glmap, 64 * c, 0, &g_full);
+    }
+    pdl_wait();
+    pdl_launch_dependents();
+    int i = 0;
+    for (int t = blockIdx.x; t < p.ntile && ok; t += gridDim.x, ++i) {
+      const int s = i % kPtSlots, r = i / kPtSlots;
+      if (r > 0) ok = mbar_wait_warp(&x_empty[s], (r - 1) & 1);
+      if (!ok) break;
+      mbar_expect_tx_warp(&x_full[s], kPtXTile);
+      tma_load_2d_warp(xs + s * kPtXTile, &xmap, 0, t * kPtRows, &x_full[s]);
+      tma_load_2d_warp(xs + s * kPtXTile + kPtXTile / 2, &xmap, 64, t * kPtRows, &x_full[s]);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.ncol >> 3) << 17) |
-                             ((uint32_t)(kPtRows >> 4) << 24);
-      ok = mbar_wait(&g_full, 0);
-      int i = 0;
-      for (int t = blockIdx.x; t < p.ntile && ok; t += gridDim.x, ++i) {
-        const int s = i % kPtSlots, r = i / kPtSlots, a = i & 1, ra = i >> 1;
-        ok = mbar_wait(&x_full[s], r & 1);
-        if (ok && ra > 0) ok = mbar_wait(&acc_empty[a], (ra - 1) & 1);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(a * p.ncol);
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.ncol >> 3) << 17) |
+                           ((uint32_t)(kPtRows >> 4) << 24);
+    ok = mbar_wait_warp(&g_full, 0);
+    int i = 0;
+    for (int t = blockIdx.x; t < p.ntile && ok; t += gridDim.x, ++i) {
+      const int s = i % kPtSlots, r = i / kPtSlots, a = i & 1, ra = i >> 1;
+      ok = mbar_wait_warp(&x_full[s], r & 1);
+      if (ok && ra > 0) ok = mbar_wait_warp(&acc_empty[a], (ra - 1) & 1);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d = tmem + (uint32_t)(a * p.ncol);
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const uint64_t ad = sw128_desc(sbase + 4 * gchunk + s * kPtXTile + c * (kPtXTile / 2));
-          const uint64_t bh = sw128_desc(sbase + c * gchunk);
-          const uint64_t bl = sw128_desc(sbase + (2 + c) * gchunk);
+      for (int c = 0; c < 2; ++c) {
+        const uint64_t ad = sw128_desc(sbase + 4 * gchunk + s * kPtXTile + c * (kPtXTile / 2));
+        const uint64_t bh = sw128_desc(sbase + c * gchunk);
+        const uint64_t bl = sw128_desc(sbase + (2 + c) * gchunk);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            umma_bf16(d, ad + 2 * kk, bh + 2 * kk, idesc, (c | kk) != 0);
-            umma_bf16(d, ad + 2 * kk, bl + 2 * kk, idesc, 1);
-          }
+        for (int kk = 0; kk < 4; ++kk) {
+          umma_bf16_warp(d, ad + 2 * kk, bh + 2 * kk, idesc, (c | kk) != 0);
+          umma_bf16_warp(d, ad + 2 * kk, bl + 2 * kk, idesc, 1);
         }
-        umma_commit(&x_empty[s]);
-        umma_commit(&acc_full[a]);
       }
+      umma_commit_warp(&x_empty[s]);
+      umma_commit_warp(&acc_full[a]);
     }
   } else {
     pdl_wait();   // the workspace belongs to the preceding grid until then
@@ -556,7 +551,6 @@ __global__ void __launch_bounds__(kPtThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
-    __syncwarp();   // warp-collective: lane 0 ran the producer loop alone
     tc_fence_after();
     tmem_dealloc(tmem, tcols);
   }
