@@ -145,6 +145,15 @@ extern "C" int sdq_plan_create(const sdq_layer_desc* desc, const int8_t* had_sig
   p->geo = g;
   p->device = dev;
   p->sm_count = sms;
+  p->half_shift = g.n_b % 2 == 0;
+  for (int j = 0; j < g.n_b / 2 && p->half_shift; ++j)
+    for (int k = 0; k < g.block; ++k) {
+      const float lo = a_enc[(size_t)j * g.block + k], hi = a_enc[(size_t)(j + g.n_b / 2) * g.block + k];
+      if (hi != (k < g.block / 2 ? lo : -lo)) {
+        p->half_shift = 0;
+        break;
+      }
+    }
   if (cudaMalloc(&p->d_at, sizeof(float) * tab) != cudaSuccess ||
       cudaMalloc(&p->d_g32, sizeof(float) * tab) != cudaSuccess ||
       cudaMalloc(&p->d_g_hi, sizeof(uint16_t) * tab) != cudaSuccess ||

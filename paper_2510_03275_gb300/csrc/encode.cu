@@ -1,7 +1,11 @@
 // K1: row-parallel Sigma-Delta encoder (SDQ-LLM Algorithm 1, eqs. (3)-(8)),
 // and the per-block half of its GPTQ compensation.
 //
-// One warp owns 4 output rows.  For every block of B input columns it
+// Two kernels, the same codes bit for bit.  encode_tile_kernel (second half of
+// this file) takes the layers whose tables and sizes allow it; the row
+// encoder takes the others, alpha as a mean, and the GPTQ blocks.
+//
+// The row encoder: one warp owns 4 output rows.  For every block of B input columns it
 // rebuilds the upsampled block x_up = A_enc w (A_enc = U Had^T, the
 // Hadamard smoothing of eq. (13) fused with the Resample upsampler) with all
 // 32 lanes, each lane producing 4 of every 128 samples for the 4 rows, in
@@ -17,7 +21,10 @@
 // the warp rebuilds the block Q = alpha (c . G), forms E = W_F - Q and the
 // normalised error E~ = E U_FF^-1 (forward substitution over the block's
 // columns), which gptq_update_kernel then applies to the later columns.
+#include <algorithm>
+
 #include "encode.cuh"
+#include "encode_tile.cuh"
 
 namespace sdq {
 
@@ -268,11 +275,244 @@ __global__ void __launch_bounds__(32 * kMaxWarps) encode_kernel(EncodeParams p) 
   }
 }
 
+// ------------------------------------------------------------ tile encoder
+// The encoder for layers whose table has the half-shift symmetry (below) and
+// whose codes of a block fill whole words, MAXABS alpha (or alpha given).
+//
+// A_enc row j + n_b / 2 is row j shifted by half a block, and a shift by B / 2
+// of an index below B flips its top bit: in the Hadamard domain
+//   A[j + n_b / 2][k] = A[j][k] (k < B / 2),  -A[j][k] (k >= B / 2)
+// for every OSR (checked bit for bit at plan creation).  So samples j and j +
+// n_b / 2 share their sums over k < B / 2, and above that their products
+// p: one adds p, the other subtracts it.  320 rounded operations in place of
+// 512 per pair at B = 128, every sum in the canonical order.
+//
+// fp32 multiply / add issue bounds it, so the rest is arranged around that: a
+// warp owns 8 virtual rows (row, block) x all n_b samples, lane l the pairs j =
+// l + 32 q (q < PT), 8 PT x 2 sums in registers; per k one shared-memory word of
+// the table per pair (conflict-free) and two broadcast 16-byte loads of the 8
+// weights serve 8 PT x 2 or 3 operations.  The persistent CTA (one per SM) holds
+// half the table and works on groups of whole rows: where a group's virtual
+// rows fit in the CTA's tile (8 per warp), alpha and the scan both use the one
+// computation of x_up, else pass 0 takes the maxima and pass 1 recomputes.
+// The scan (eq. 8) of a tile runs with one lane per virtual row, 32 to a
+// warp, beside the other warps' next tile: blocks are independent, so 32
+// lanes of a warp scan where 4 did with a lane per row.
+// 11008 x 4096, OSR 2 (46 G rounded operations as two plain passes, 14 G so):
+// 6.24 ms with the row encoder, 0.95 ms.
+// warps at most: 16, or 8 where a thread needs more than 128 registers
+constexpr int tile_max_warps(int pt) { return pt <= 4 ? 16 : 8; }
+constexpr int kTMaxRows = 16;   // rows per group
+
+struct TileParams {
+  const float* W;
+  uint32_t* codes;
+  float* alpha;
+  const float* at;   // B x n_b
+  int n_out, k_in, B, n_b, nblk, wpr, quantizer, rows, given, only_alpha;
+  uint32_t pad0;     // first padding word of a row
+};
+
+template <int PT>
+__global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel(TileParams p) {
+  extern __shared__ __align__(16) float smem[];
+  __shared__ uint32_t s_amax[2][kTMaxRows];   // bit patterns of the rows' maxima (non-negative floats)
+  const int warp = warp_index(), lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+  const int np = p.n_b / 2, xs_stride = p.n_b + 1;
+  float* ts = smem;                                        // B x np
+  float* wt = ts + (size_t)p.B * np + (size_t)warp * tile_weight_floats(p.B);
+  float* xs0 = ts + (size_t)p.B * np + (size_t)nwarp * tile_weight_floats(p.B);
+  float* xs = xs0 + (size_t)warp * kTv * xs_stride;
+  tile_load_table(ts, p.at, p.B, p.n_b);
+  if (threadIdx.x < 2 * kTMaxRows) s_amax[threadIdx.x / kTMaxRows][threadIdx.x % kTMaxRows] = 0u;
+  __syncthreads();
+
+  const int tv = kTv * nwarp, ngroups = (p.n_out + p.rows - 1) / p.rows;
+  float acc[kTv][PT], acc2[kTv][PT];
+
+  // x_up of virtual rows v0 .. v0 + 7 of the group at row0 (nv in all) into
+  // acc (samples l + 32 q) and acc2 (the same + n_b / 2)
+  auto compute = [&](int row0, int v0, int nv) {
+    {
+      // the 8 x B weights, transposed to [k][8]: lane = (virtual row, float4)
+      const int v = v0 + (lane >> 2), r = min(v, nv - 1) / p.nblk, b = min(v, nv - 1) - r * p.nblk;
+      const float4* src = reinterpret_cast<const float4*>(p.W + (size_t)(row0 + r) * p.k_in + (size_t)b * p.B);
+      __syncwarp();
+      for (int k4 = lane & 3; k4 < p.B / 4; k4 += 4) {
+        const float4 w = v < nv ? __ldg(src + k4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float* d = wt + k4 * kWk4 + (lane >> 2);
+        d[0] = w.x; d[8] = w.y; d[16] = w.z; d[24] = w.w;
+      }
+      __syncwarp();
+    }
+    tile_upsample<PT>(ts + lane, np, np - lane, wt, p.B, acc, acc2);
+  };
+  // row maxima of the warp's 8 virtual rows (pairs past np hold zeros)
+  auto maxima = [&](int v0, int nv, uint32_t* am) {
+#pragma unroll
+    for (int v = 0; v < kTv; ++v) {
+      float m = 0.f;
+#pragma unroll
+      for (int q = 0; q < PT; ++q) m = fmaxf(m, fmaxf(fabsf(acc[v][q]), fabsf(acc2[v][q])));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0 && v0 + v < nv) atomicMax(&am[(v0 + v) / p.nblk], __float_as_uint(m));
+    }
+  };
+  auto store = [&]() {
+#pragma unroll
+    for (int v = 0; v < kTv; ++v)
+#pragma unroll
+      for (int q = 0; q < PT; ++q)
+        if (lane + 32 * q < np) {
+          xs[v * xs_stride + lane + 32 * q] = acc[v][q];
+          xs[v * xs_stride + np + lane + 32 * q] = acc2[v][q];
+        }
+  };
+  // Eq. (8) over virtual row `lv` of the tile: i = (i + x) - y_prev from 0,
+  // the codes packed into whole words.
+  auto scan = [&](int row, int b, int lv, float a) {
+    const float theta = 0.5f * a;
+    const float* x = xs0 + (size_t)lv * xs_stride;
+    uint32_t* out = p.codes + (size_t)row * p.wpr + (size_t)b * p.n_b * p.quantizer / 32;
+    float integ = 0.f, yp = 0.f;
+    if (p.quantizer == SDQ_TERNARY) {
+      for (int j = 0; j < p.n_b; j += 16) {
+        uint32_t cw = 0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) cw |= sd_step<true>(integ, yp, x[j + i], a, theta) << (2 * i);
+        out[j / 16] = cw;
+      }
+    } else {
+      for (int j = 0; j < p.n_b; j += 32) {
+        uint32_t cw = 0;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) cw |= sd_step<false>(integ, yp, x[j + i], a, theta) << i;
+        out[j / 32] = cw;
+      }
+    }
+    if (b == p.nblk - 1)   // the row's padding words
+      for (int w = (int)p.pad0; w < p.wpr; ++w) p.codes[(size_t)row * p.wpr + w] = 0u;
+  };
+
+  int turn = 0;   // scanning warps rotate over the warps
+  int buf = 0;
+  for (int g = blockIdx.x; g < ngroups; g += gridDim.x, buf ^= 1) {
+    const int row0 = g * p.rows, nv = min(p.rows, p.n_out - row0) * p.nblk;
+    const int tiles = (nv + tv - 1) / tv;
+    uint32_t* am = s_amax[buf];
+    const bool single = tiles == 1 && !p.given && !p.only_alpha;   // one computation for alpha and the scan
+    const int n0 = p.given || single ? 0 : tiles;                  // steps of pass 0
+    const int steps = n0 + (p.only_alpha ? 0 : tiles);
+    for (int step = 0; step < steps; ++step) {
+      const int t = step < n0 ? step : step - n0, v0 = t * tv + warp * kTv;
+      if (v0 < nv) {
+        compute(row0, v0, nv);
+        if (step < n0 || single) maxima(v0, nv, am);
+      }
+      if (step < n0) continue;
+      __syncthreads();   // the tile before is scanned; the maxima are in
+      if (t == 0 && threadIdx.x < kTMaxRows) s_amax[buf ^ 1][threadIdx.x] = 0u;
+      if (v0 < nv) store();
+      __syncthreads();
+      // 32 virtual rows per scanning warp
+      const int part = (warp - turn + nwarp) % nwarp;
+      const int lv = 32 * part + lane, v = t * tv + lv;
+      if (lv < tv && v < nv) {
+        const int r = v / p.nblk, b = v - r * p.nblk, row = row0 + r;
+        const float a = p.given ? p.alpha[row] : __uint_as_float(am[r]);
+        if (!p.given && b == 0) p.alpha[row] = a;
+        scan(row, b, lv, a);
+      }
+      turn = (turn + (tv + 31) / 32) % nwarp;
+    }
+    if (p.only_alpha) {
+      __syncthreads();
+      if (threadIdx.x < kTMaxRows) {
+        if ((int)threadIdx.x * p.nblk < nv) p.alpha[row0 + threadIdx.x] = __uint_as_float(am[threadIdx.x]);
+        s_amax[buf ^ 1][threadIdx.x] = 0u;
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// Warps and rows per group of the tile encoder, 0 warps where it does not
+// apply: the half-shift table, whole words of codes per block, at most 192
+// pairs, and half the table in shared memory beside at least 4 warps' buffers
+// (n_b / 2 x B words; 5 B + 8 (n_b + 1) words a warp).
+struct TileShape {
+  int warps, rows, pt;
+  size_t smem;
+};
+TileShape tile_shape(const sdq_plan_s* pl, bool given) {
+  const Geometry& g = pl->geo;
+  TileShape t{};
+  const int np = g.n_b / 2;
+  if (!pl->half_shift || g.block < 16 || np > 192 || (g.n_b * g.bits) % 32) return t;
+  const size_t table = sizeof(float) * (size_t)g.block * np;
+  const size_t per_warp = sizeof(float) * ((size_t)tile_weight_floats(g.block) + (size_t)kTv * (g.n_b + 1));
+  const size_t room = 226 * 1024;
+  if (table + 4 * per_warp > room) return t;
+  t.pt = (np + 31) / 32;
+  t.warps = (int)std::min<size_t>(tile_max_warps(t.pt), (room - table) / per_warp) & ~1;
+  t.smem = table + t.warps * per_warp;
+  const int tv = kTv * t.warps;
+  const int64_t sms = std::max(1, pl->sm_count);
+  // the row count whose groups take the fewest tile computations on the
+  // busiest SM; one tile serves both passes where the group fits in it
+  double best = 0;
+  for (int r = 1; r <= kTMaxRows; ++r) {
+    const int64_t groups = (g.n_out + r - 1) / r, waves = (groups + sms - 1) / sms;
+    const int64_t tiles = ((int64_t)r * g.nblk + tv - 1) / tv;
+    // work of the warps that have virtual rows in the tile, at least a scan
+    const double fill = tiles == 1 ? std::max(0.25, (double)((r * g.nblk + kTv - 1) / kTv) / t.warps) : 1.0;
+    const double c = (double)waves * (given || tiles == 1 ? tiles * fill : 2.0 * tiles);
+    if (r == 1 || c < best * 0.999) {
+      best = c;
+      t.rows = r;
+    }
+  }
+  return t;
+}
+
+cudaError_t launch_encode_tile(const sdq_plan_s* pl, const TileShape& t, const float* W, uint32_t* codes, float* alpha,
+                               cudaStream_t st, bool given, bool only_alpha) {
+  const Geometry& g = pl->geo;
+  TileParams p;
+  p.W = W; p.codes = codes; p.alpha = alpha; p.at = pl->d_at;
+  p.n_out = g.n_out; p.k_in = g.k_in; p.B = g.block; p.n_b = g.n_b; p.nblk = g.nblk;
+  p.wpr = g.words_per_row; p.quantizer = pl->desc.quantizer; p.rows = t.rows;
+  p.given = given; p.only_alpha = only_alpha;
+  p.pad0 = (uint32_t)(g.k_eff * g.bits / 32);
+  auto kern = t.pt <= 1 ? encode_tile_kernel<1> : t.pt == 2 ? encode_tile_kernel<2> : t.pt == 3 ? encode_tile_kernel<3>
+            : t.pt == 4 ? encode_tile_kernel<4> : t.pt == 5 ? encode_tile_kernel<5> : encode_tile_kernel<6>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+  if (e != cudaSuccess) return e;
+  const int groups = (g.n_out + t.rows - 1) / t.rows;
+  kern<<<std::min(groups, std::max(1, pl->sm_count)), 32 * t.warps, t.smem, st>>>(p);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_encode(const sdq_plan_s* pl, const float* W, uint32_t* codes, float* alpha,
                           cudaStream_t st) {
-  return launch_encode_range(pl, W, codes, alpha, st, 0, 2, 0, pl->geo.nblk, nullptr, nullptr);
+  const bool mean = pl->desc.alpha_mode == SDQ_ALPHA_MEANABS;   // alpha in sequence order: the row encoder's pass 0
+  const TileShape t = tile_shape(pl, mean);
+  if (!t.warps) return launch_encode_range(pl, W, codes, alpha, st, 0, 2, 0, pl->geo.nblk, nullptr, nullptr);
+  if (mean) {
+    const cudaError_t e = launch_encode_range(pl, W, codes, alpha, st, 0, 1, 0, pl->geo.nblk, nullptr, nullptr);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_encode_tile(pl, t, W, codes, alpha, st, mean, false);
+}
+
+cudaError_t launch_encode_alpha(const sdq_plan_s* pl, const float* W, uint32_t* codes, float* alpha, cudaStream_t st) {
+  const TileShape t = tile_shape(pl, false);
+  if (!t.warps || pl->desc.alpha_mode == SDQ_ALPHA_MEANABS)
+    return launch_encode_range(pl, W, codes, alpha, st, 0, 1, 0, pl->geo.nblk, nullptr, nullptr);
+  return launch_encode_tile(pl, t, W, codes, alpha, st, false, true);
 }
 
 cudaError_t launch_encode_range(const sdq_plan_s* pl, const float* W, uint32_t* codes, float* alpha,

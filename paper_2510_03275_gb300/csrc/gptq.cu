@@ -132,7 +132,7 @@ extern "C" int sdq_encode_rows_gptq(sdq_plan p, const float* W, const float* U, 
   float* et = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + align256(sizeof(float) * (size_t)g.n_out * g.k_in));
   cudaError_t e = cudaMemcpyAsync(wc, W, sizeof(float) * (size_t)g.n_out * g.k_in, cudaMemcpyDeviceToDevice, st);
   // alpha from the original weights (pass 0 over every block)
-  if (e == cudaSuccess) e = launch_encode_range(p, wc, codes_plain, alpha, st, 0, 1, 0, g.nblk, nullptr, nullptr);
+  if (e == cudaSuccess) e = launch_encode_alpha(p, wc, codes_plain, alpha, st);
   for (int b = 0; b < g.nblk && e == cudaSuccess; ++b) {
     e = launch_encode_range(p, wc, codes_plain, alpha, st, 1, 2, b, b + 1, U, et);
     if (e == cudaSuccess && b + 1 < g.nblk) e = launch_gptq_update(p, wc, et, U, b, st);
