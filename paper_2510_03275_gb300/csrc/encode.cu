@@ -299,10 +299,12 @@ __global__ void __launch_bounds__(32 * kMaxWarps) encode_kernel(EncodeParams p) 
 // warp, beside the other warps' next tile: blocks are independent, so 32
 // lanes of a warp scan where 4 did with a lane per row.
 // 11008 x 4096, OSR 2 (46 G rounded operations as two plain passes, 14 G so):
-// 6.24 ms with the row encoder, 0.95 ms.
+// 6.24 ms with the row encoder, 0.71 ms (0.95 with one
+// team per CTA, whose barriers had the other warps wait for the scan).
 // warps at most: 16, or 8 where a thread needs more than 128 registers
 constexpr int tile_max_warps(int pt) { return pt <= 4 ? 16 : 8; }
 constexpr int kTMaxRows = 16;   // rows per group
+constexpr int kTMaxTeams = 4;
 
 struct TileParams {
   const float* W;
@@ -310,24 +312,30 @@ struct TileParams {
   float* alpha;
   const float* at;   // B x n_b
   int n_out, k_in, B, n_b, nblk, wpr, quantizer, rows, given, only_alpha;
+  int gw;            // warps of a team
   uint32_t pad0;     // first padding word of a row
 };
 
 template <int PT>
 __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel(TileParams p) {
   extern __shared__ __align__(16) float smem[];
-  __shared__ uint32_t s_amax[2][kTMaxRows];   // bit patterns of the rows' maxima (non-negative floats)
+  __shared__ uint32_t s_amax[kTMaxTeams][2][kTMaxRows];   // bit patterns of the rows' maxima (non-negative floats)
   const int warp = warp_index(), lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+  // teams of gw warps work on row groups of their own and meet at their own
+  // barriers, so that one team's scan runs beside the others' products
+  const int team = warp / p.gw, tw = warp - team * p.gw, nteam = nwarp / p.gw, tt = 32 * tw + lane;
+  auto team_sync = [&]() { named_bar_sync(1 + team, 32 * p.gw); };
   const int np = p.n_b / 2, xs_stride = p.n_b + 1;
   float* ts = smem;                                        // B x np
   float* wt = ts + (size_t)p.B * np + (size_t)warp * tile_weight_floats(p.B);
-  float* xs0 = ts + (size_t)p.B * np + (size_t)nwarp * tile_weight_floats(p.B);
-  float* xs = xs0 + (size_t)warp * kTv * xs_stride;
+  float* xs0 = ts + (size_t)p.B * np + (size_t)nwarp * tile_weight_floats(p.B) +
+               (size_t)team * p.gw * kTv * xs_stride;   // the team's samples
+  float* xs = xs0 + (size_t)tw * kTv * xs_stride;
   tile_load_table(ts, p.at, p.B, p.n_b);
-  if (threadIdx.x < 2 * kTMaxRows) s_amax[threadIdx.x / kTMaxRows][threadIdx.x % kTMaxRows] = 0u;
+  for (int i = threadIdx.x; i < kTMaxTeams * 2 * kTMaxRows; i += blockDim.x) (&s_amax[0][0][0])[i] = 0u;
   __syncthreads();
 
-  const int tv = kTv * nwarp, ngroups = (p.n_out + p.rows - 1) / p.rows;
+  const int tv = kTv * p.gw, ngroups = (p.n_out + p.rows - 1) / p.rows;
   float acc[kTv][PT], acc2[kTv][PT];
 
   // x_up of virtual rows v0 .. v0 + 7 of the group at row0 (nv in all) into
@@ -395,28 +403,28 @@ __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel
       for (int w = (int)p.pad0; w < p.wpr; ++w) p.codes[(size_t)row * p.wpr + w] = 0u;
   };
 
-  int turn = 0;   // scanning warps rotate over the warps
+  int turn = 0;   // scanning warps rotate over the team
   int buf = 0;
-  for (int g = blockIdx.x; g < ngroups; g += gridDim.x, buf ^= 1) {
+  for (int g = blockIdx.x + team * gridDim.x; g < ngroups; g += gridDim.x * nteam, buf ^= 1) {
     const int row0 = g * p.rows, nv = min(p.rows, p.n_out - row0) * p.nblk;
     const int tiles = (nv + tv - 1) / tv;
-    uint32_t* am = s_amax[buf];
+    uint32_t *am = s_amax[team][buf], *am_next = s_amax[team][buf ^ 1];
     const bool single = tiles == 1 && !p.given && !p.only_alpha;   // one computation for alpha and the scan
     const int n0 = p.given || single ? 0 : tiles;                  // steps of pass 0
     const int steps = n0 + (p.only_alpha ? 0 : tiles);
     for (int step = 0; step < steps; ++step) {
-      const int t = step < n0 ? step : step - n0, v0 = t * tv + warp * kTv;
+      const int t = step < n0 ? step : step - n0, v0 = t * tv + tw * kTv;
       if (v0 < nv) {
         compute(row0, v0, nv);
         if (step < n0 || single) maxima(v0, nv, am);
       }
       if (step < n0) continue;
-      __syncthreads();   // the tile before is scanned; the maxima are in
-      if (t == 0 && threadIdx.x < kTMaxRows) s_amax[buf ^ 1][threadIdx.x] = 0u;
+      team_sync();   // the tile before is scanned; the maxima are in
+      if (t == 0 && tt < kTMaxRows) am_next[tt] = 0u;
       if (v0 < nv) store();
-      __syncthreads();
+      team_sync();
       // 32 virtual rows per scanning warp
-      const int part = (warp - turn + nwarp) % nwarp;
+      const int part = (tw - turn + p.gw) % p.gw;
       const int lv = 32 * part + lane, v = t * tv + lv;
       if (lv < tv && v < nv) {
         const int r = v / p.nblk, b = v - r * p.nblk, row = row0 + r;
@@ -424,25 +432,25 @@ __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel
         if (!p.given && b == 0) p.alpha[row] = a;
         scan(row, b, lv, a);
       }
-      turn = (turn + (tv + 31) / 32) % nwarp;
+      turn = (turn + (tv + 31) / 32) % p.gw;
     }
     if (p.only_alpha) {
-      __syncthreads();
-      if (threadIdx.x < kTMaxRows) {
-        if ((int)threadIdx.x * p.nblk < nv) p.alpha[row0 + threadIdx.x] = __uint_as_float(am[threadIdx.x]);
-        s_amax[buf ^ 1][threadIdx.x] = 0u;
+      team_sync();
+      if (tt < kTMaxRows) {
+        if (tt * p.nblk < nv) p.alpha[row0 + tt] = __uint_as_float(am[tt]);
+        am_next[tt] = 0u;
       }
-      __syncthreads();
+      team_sync();
     }
   }
 }
 
-// Warps and rows per group of the tile encoder, 0 warps where it does not
-// apply: the half-shift table, whole words of codes per block, at most 192
-// pairs, and half the table in shared memory beside at least 4 warps' buffers
-// (n_b / 2 x B words; 5 B + 8 (n_b + 1) words a warp).
+// Warps, warps per team and rows per group of the tile encoder, 0 warps where
+// it does not apply: the half-shift table, whole words of codes per block, at
+// most 192 pairs, and half the table in shared memory beside at least 4 warps'
+// buffers (n_b / 2 x B words; 10 B + 8 (n_b + 1) words a warp).
 struct TileShape {
-  int warps, rows, pt;
+  int warps, gw, rows, pt;
   size_t smem;
 };
 TileShape tile_shape(const sdq_plan_s* pl, bool given) {
@@ -455,24 +463,34 @@ TileShape tile_shape(const sdq_plan_s* pl, bool given) {
   const size_t room = 226 * 1024;
   if (table + 4 * per_warp > room) return t;
   t.pt = (np + 31) / 32;
-  t.warps = (int)std::min<size_t>(tile_max_warps(t.pt), (room - table) / per_warp) & ~1;
-  t.smem = table + t.warps * per_warp;
-  const int tv = kTv * t.warps;
+  const int most = (int)std::min<size_t>(tile_max_warps(t.pt), (room - table) / per_warp);
   const int64_t sms = std::max(1, pl->sm_count);
-  // the row count whose groups take the fewest tile computations on the
-  // busiest SM; one tile serves both passes where the group fits in it
+  // Teams of 4 warps or of all (most of them in whole teams), and the row
+  // count whose groups take the least time on the busiest SM: a tile's
+  // products on the warps that have virtual rows in it, twice where alpha
+  // and the scan need two computations, and a scan (a fifth of a full
+  // tile's products on 12 warps), which other teams' products hide.
   double best = 0;
-  for (int r = 1; r <= kTMaxRows; ++r) {
-    const int64_t groups = (g.n_out + r - 1) / r, waves = (groups + sms - 1) / sms;
-    const int64_t tiles = ((int64_t)r * g.nblk + tv - 1) / tv;
-    // work of the warps that have virtual rows in the tile, at least a scan
-    const double fill = tiles == 1 ? std::max(0.25, (double)((r * g.nblk + kTv - 1) / kTv) / t.warps) : 1.0;
-    const double c = (double)waves * (given || tiles == 1 ? tiles * fill : 2.0 * tiles);
-    if (r == 1 || c < best * 0.999) {
-      best = c;
-      t.rows = r;
+  const int widths[2] = {4, most & ~1};
+  for (int gw : widths) {
+    const int nteam = most / gw, tv = kTv * gw;
+    for (int r = 1; r <= kTMaxRows; ++r) {
+      const int64_t groups = (g.n_out + r - 1) / r;
+      const int64_t turns = (groups + sms * nteam - 1) / (sms * nteam);   // groups of the busiest team
+      const int64_t tiles = ((int64_t)r * g.nblk + tv - 1) / tv;
+      const double live = tiles == 1 ? (double)((r * g.nblk + kTv - 1) / kTv) : (double)gw;   // warps at work
+      // the SM's issue slots shared by its teams' warps, at least one warp per quadrant's own pace
+      const double products = tiles * std::max(live * nteam / 12.0, 0.35) * (given || tiles == 1 ? 1.0 : 2.0);
+      const double c = (double)turns * (products + (nteam > 1 ? 0.08 : 0.3) * tiles);
+      if (!t.warps || c < best * 0.999) {
+        best = c;
+        t.warps = gw * nteam;
+        t.gw = gw;
+        t.rows = r;
+      }
     }
   }
+  t.smem = table + t.warps * per_warp;
   return t;
 }
 
@@ -483,7 +501,7 @@ cudaError_t launch_encode_tile(const sdq_plan_s* pl, const TileShape& t, const f
   p.W = W; p.codes = codes; p.alpha = alpha; p.at = pl->d_at;
   p.n_out = g.n_out; p.k_in = g.k_in; p.B = g.block; p.n_b = g.n_b; p.nblk = g.nblk;
   p.wpr = g.words_per_row; p.quantizer = pl->desc.quantizer; p.rows = t.rows;
-  p.given = given; p.only_alpha = only_alpha;
+  p.given = given; p.only_alpha = only_alpha; p.gw = t.gw;
   p.pad0 = (uint32_t)(g.k_eff * g.bits / 32);
   auto kern = t.pt <= 1 ? encode_tile_kernel<1> : t.pt == 2 ? encode_tile_kernel<2> : t.pt == 3 ? encode_tile_kernel<3>
             : t.pt == 4 ? encode_tile_kernel<4> : t.pt == 5 ? encode_tile_kernel<5> : encode_tile_kernel<6>;
