@@ -331,6 +331,10 @@ PrefillShape prefill_shape(const sdq_plan_s* pl, int M) {
     }
   }
   s.smem = kFixedSmem + std::max(s.stages * s.bn * 128, s.split > 1 ? s.bn * kBM * 4 - kCodeSlots * kCSlot : 0);
+  // a grid that fits one CTA per SM asks for more than half an SM: launched
+  // early, CTAs would pair up on the first SMs that the prepare kernel leaves
+  // (4096 x 22016 codes at M = 65: 33 us against 22 spread out)
+  if (occ == 2 && tiles <= pl->pf_clusters[s.split]) s.smem = std::max(s.smem, kSmemSm / 2 + 4096);
   return s;
 }
 constexpr int kPfSmemLimit = kSmemSm - 1024;
@@ -372,27 +376,30 @@ cudaError_t prefill_smem_limit(int device) {
 
 // ------------------------------------------ prefill prepare, tensor cores
 // x_tilde = G x_b for every block b (section 3.5), as one GEMM: x viewed as
-// R = M nblk rows of B = 128 inputs (row r = block r mod nblk of batch row
-// r / nblk), x_tilde rows = x rows . G^T (128 x n_b), on tcgen05.mma
-// kind::f16 (M = 128 rows, N = n_b, K = 16 per instruction) with G split
-// into bf16 hi and lo parts accumulated into the same fp32 accumulator (the
-// pair carries G to ~2^-16; x is bf16, exact).  Persistent CTAs, one per SM,
-// over tiles of 128 rows:
-//   warp 0     TMEM allocation (two accumulators of n_b columns);
-//              loads G hi / lo once, then the x tiles into a 3-slot ring
-//              (TMA, 128-byte swizzle: the canonical K-major operand layout)
-//   warp 1     issues each tile's 16 MMAs into accumulator t mod 2
-//   warps 2-9  epilogue, two warps per TMEM lane quadrant (half of the n_b
+// R = M nblk rows of B inputs (row r = block r mod nblk of batch row r /
+// nblk), x_tilde rows = x rows . G^T (B x n_b), on tcgen05.mma kind::f16 (M =
+// 128 rows, N = ncol, K = 16 per instruction) with G split into bf16 hi and lo
+// parts accumulated into the same fp32 accumulator (the pair carries G to
+// ~2^-16; x is bf16, exact).  A CTA keeps the hi and lo parts of ncol of
+// the n_b columns (grid.y: which) and walks tiles of 128 rows (grid.x):
+//   warp 0     TMEM allocation (two accumulators of ncol columns); loads its
+//              part of G once, then the x tiles by 64-wide K chunks into a
+//              ring (TMA, 128-byte swizzle: the canonical K-major operand)
+//   warp 1     issues each tile's B / 8 MMAs into accumulator t mod 2
+//   warps 2-9  epilogue, two warps per TMEM lane quadrant (half of the ncol
 //              columns each): bf16 x_tilde (round to nearest even) in the
 //              prefill operand order (prefill_pos64) with 16-byte stores;
 //              the K padding of every batch row set to zero
-// Layers with n_b above 256 take one launch per 256 or fewer columns (x read
-// once per launch).  Bounded waits as in the contraction kernels.
+// Large batches write 2 M K_eff bytes and are bound by that (ncol as large as
+// fits); small ones by the chain of one tile, so they take ncol = 64: four
+// times the CTAs at OSR 2, each loading a quarter of G (M = 201 on 4096
+// inputs: 6.3 -> 4.6 us, M = 65: 6.2 -> 3.3).  Bounded waits as in the contraction kernels.
 constexpr int kPtEpiWarps = 8;
 constexpr int kPtThreads = 64 + 32 * kPtEpiWarps;
 constexpr int kPtRows = 128;
-constexpr int kPtXTile = kPtRows * 128 * 2;   // 32 KB: 128 rows x 128 bf16 (two 64-wide K chunks)
-constexpr int kPtSlots = 3;                   // x ring (with G hi / lo of n_b = 256: 225 KB)
+constexpr int kPtChunk = kPtRows * 64 * 2;    // 16 KB: 128 rows x 64 bf16
+constexpr int kPtMaxSlots = 6;
+constexpr int kPtSmem = 226 * 1024;
 
 struct PrepTcParams {
   uint16_t* xtb;
@@ -400,27 +407,26 @@ struct PrepTcParams {
   uint64_t call;
   int64_t R, k_eff, kpad;
   int M, nblk, n_b, ntile, ternary;
-  int j0, ncol;   // this launch's x_tilde columns j0 .. j0 + ncol - 1 of every block (ncol <= 256)
+  int ncol, nch, slots;   // columns per CTA, 64-wide K chunks (B / 64), ring slots
 };
 
 __global__ void __launch_bounds__(kPtThreads, 1)
     prep_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap ghmap,
                    const __grid_constant__ CUtensorMap glmap, PrepTcParams p) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t g_full, x_full[kPtSlots], x_empty[kPtSlots], acc_full[2], acc_empty[2];
+  __shared__ __align__(8) uint64_t g_full, x_full[kPtMaxSlots], x_empty[kPtMaxSlots], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base;
-  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31, j0 = (int)blockIdx.y * p.ncol;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (sbase - smem_u32(smem_raw));
   const uint32_t gchunk = (uint32_t)p.ncol * 128u;  // one 64-wide K chunk of G^T: ncol rows x 128 B
-  uint8_t* gh = base;                               // 2 chunks
-  uint8_t* gl = base + 2 * gchunk;                  // 2 chunks
-  uint8_t* xs = base + 4 * gchunk;                  // kPtSlots ring slots
+  uint8_t* gl = base + p.nch * gchunk;              // (hi chunks first)
+  const uint32_t xoff = 2u * p.nch * gchunk;        // then the ring
   const uint32_t tcols = p.ncol <= 64 ? 128u : (p.ncol <= 128 ? 256u : 512u);
 
   if (tid == 0) {
     mbar_init(&g_full, 1);
-    for (int s = 0; s < kPtSlots; ++s) {
+    for (int s = 0; s < kPtMaxSlots; ++s) {
       mbar_init(&x_full[s], 1);
       mbar_init(&x_empty[s], 1);
     }
@@ -443,71 +449,77 @@ __global__ void __launch_bounds__(kPtThreads, 1)
   if (warp == 0) {
     // G (the plan's table, never written by the stream) before the wait
     // for the preceding grid; x and the workspace after it
-    mbar_expect_tx_warp(&g_full, 4 * gchunk);
-    for (int c = 0; c < 2; ++c) {
-      tma_load_2d_warp(gh + c * gchunk, &ghmap, 64 * c, 0, &g_full);
-      tma_load_2d_warp(gl + c * gchunk, &glmap, 64 * c, 0, &g_full);
+    mbar_expect_tx_warp(&g_full, 2u * p.nch * gchunk);
+    for (int c = 0; c < p.nch; ++c) {
+      tma_load_2d_warp(base + c * gchunk, &ghmap, 64 * c, j0, &g_full);
+      tma_load_2d_warp(gl + c * gchunk, &glmap, 64 * c, j0, &g_full);
     }
     pdl_wait();
     pdl_launch_dependents();
-    int i = 0;
-    for (int t = blockIdx.x; t < p.ntile && ok; t += gridDim.x, ++i) {
-      const int s = i % kPtSlots, r = i / kPtSlots;
-      if (r > 0) ok = mbar_wait_warp(&x_empty[s], (r - 1) & 1);
-      if (!ok) break;
-      mbar_expect_tx_warp(&x_full[s], kPtXTile);
-      tma_load_2d_warp(xs + s * kPtXTile, &xmap, 0, t * kPtRows, &x_full[s]);
-      tma_load_2d_warp(xs + s * kPtXTile + kPtXTile / 2, &xmap, 64, t * kPtRows, &x_full[s]);
-    }
+    int s = 0, r = 0, n = 0;
+    for (int t = blockIdx.x; t < p.ntile && ok; t += gridDim.x)
+      for (int c = 0; c < p.nch && ok; ++c) {
+        if (r > 0) ok = mbar_wait_warp(&x_empty[s], (r - 1) & 1);
+        if (!ok) break;
+        mbar_expect_tx_warp(&x_full[s], kPtChunk);
+        tma_load_2d_warp(base + xoff + s * kPtChunk, &xmap, 64 * c, t * kPtRows, &x_full[s]);
+        ++n;
+        if (++s == p.slots) { s = 0; ++r; }
+      }
+    // every copy issued has landed before the CTA ends
+    if (!mbar_wait_warp(&g_full, 0)) ok = false;
+    for (int i = max(0, n - p.slots); i < n; ++i)
+      if (!mbar_wait_warp(&x_full[i % p.slots], (i / p.slots) & 1)) ok = false;
   } else if (warp == 1) {
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.ncol >> 3) << 17) |
                            ((uint32_t)(kPtRows >> 4) << 24);
     ok = mbar_wait_warp(&g_full, 0);
-    int i = 0;
+    const uint64_t gd = sw128_desc(sbase), xd = sw128_desc(sbase + xoff);
+    const uint32_t gstep = gchunk >> 4;
+    int i = 0, s = 0, r = 0;
     for (int t = blockIdx.x; t < p.ntile && ok; t += gridDim.x, ++i) {
-      const int s = i % kPtSlots, r = i / kPtSlots, a = i & 1, ra = i >> 1;
-      ok = mbar_wait_warp(&x_full[s], r & 1);
-      if (ok && ra > 0) ok = mbar_wait_warp(&acc_empty[a], (ra - 1) & 1);
-      if (!ok) break;
-      tc_fence_after();
+      const int a = i & 1, ra = i >> 1;
+      if (ra > 0) ok = mbar_wait_warp(&acc_empty[a], (ra - 1) & 1);
       const uint32_t d = tmem + (uint32_t)(a * p.ncol);
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const uint64_t ad = sw128_desc(sbase + 4 * gchunk + s * kPtXTile + c * (kPtXTile / 2));
-        const uint64_t bh = sw128_desc(sbase + c * gchunk);
-        const uint64_t bl = sw128_desc(sbase + (2 + c) * gchunk);
+      for (int c = 0; c < p.nch && ok; ++c) {
+        ok = mbar_wait_warp(&x_full[s], r & 1);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t ad = xd + (uint64_t)(s * (kPtChunk >> 4));
+        const uint64_t bh = gd + (uint64_t)(c * gstep), bl = gd + (uint64_t)((p.nch + c) * gstep);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           umma_bf16_warp(d, ad + 2 * kk, bh + 2 * kk, idesc, (c | kk) != 0);
           umma_bf16_warp(d, ad + 2 * kk, bl + 2 * kk, idesc, 1);
         }
+        umma_commit_warp(&x_empty[s]);
+        if (++s == p.slots) { s = 0; ++r; }
       }
-      umma_commit_warp(&x_empty[s]);
-      umma_commit_warp(&acc_full[a]);
+      if (ok) umma_commit_warp(&acc_full[a]);
     }
   } else {
     pdl_wait();   // the workspace belongs to the preceding grid until then
     const int et = tid - 64, q = warp & 3, half = (warp - 2) >> 2;
     // the K padding of every batch row (k_eff .. kpad, a multiple of 8; by
-    // the launch of the first columns)
-    if (p.j0 == 0)
-    for (int64_t z = (int64_t)blockIdx.x * (32 * kPtEpiWarps) + et; z < (int64_t)p.M * ((p.kpad - p.k_eff) / 8);
-         z += (int64_t)gridDim.x * (32 * kPtEpiWarps)) {
-      const int64_t per = (p.kpad - p.k_eff) / 8, m = z / per;
-      *reinterpret_cast<uint4*>(p.xtb + m * p.kpad + p.k_eff + 8 * (z - m * per)) = make_uint4(0, 0, 0, 0);
-    }
+    // the CTAs of the first columns)
+    if (j0 == 0)
+      for (int64_t z = (int64_t)blockIdx.x * (32 * kPtEpiWarps) + et; z < (int64_t)p.M * ((p.kpad - p.k_eff) / 8);
+           z += (int64_t)gridDim.x * (32 * kPtEpiWarps)) {
+        const int64_t per = (p.kpad - p.k_eff) / 8, m = z / per;
+        *reinterpret_cast<uint4*>(p.xtb + m * p.kpad + p.k_eff + 8 * (z - m * per)) = make_uint4(0, 0, 0, 0);
+      }
     const int cw = p.ncol / 2;                                  // this warp's columns
     const uint32_t lq = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(half * cw);
     int i = 0;
     for (int t = blockIdx.x; t < p.ntile && ok; t += gridDim.x, ++i) {
       const int s = i & 1, r = i >> 1;
-      ok = mbar_wait(&acc_full[s], r & 1);
+      ok = mbar_wait_warp(&acc_full[s], r & 1);
       if (!ok) break;
       tc_fence_after();
       const int64_t row = (int64_t)t * kPtRows + 32 * q + lane;
       const bool live = row < p.R;
       const int64_t m = live ? row / p.nblk : 0;
-      uint16_t* out = p.xtb + m * p.kpad + (live ? (row - m * p.nblk) * p.n_b : 0) + p.j0 + half * cw;
+      uint16_t* out = p.xtb + m * p.kpad + (live ? (row - m * p.nblk) * p.n_b : 0) + j0 + half * cw;
       const uint32_t acol = (uint32_t)(s * p.ncol);
       // 32 columns at a time: a ternary operand permutes within 16, a binary
       // one within 32 positions (prefill_pos64); physical pair (2k, 2k + 1)
@@ -531,11 +543,8 @@ __global__ void __launch_bounds__(kPtThreads, 1)
           }
         } else {
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const float lo = k < 16 ? __uint_as_float(a[15 - k]) : 0.f;
-            const float hi = __uint_as_float(b[15 - k]);
-            w[k] = pack_bf16x2(lo, hi);
-          }
+          for (int k = 0; k < 16; ++k)
+            w[k] = pack_bf16x2(__uint_as_float(a[15 - k]), __uint_as_float(b[15 - k]));
         }
         if (live) {
           uint4* o = reinterpret_cast<uint4*>(out + c0);
@@ -609,69 +618,58 @@ cudaError_t prefill_occupancy(sdq_plan_s* pl) {
   return e;
 }
 
-// The prefill prepare kernel on the tensor cores where it applies (B = 128,
-// n_b a multiple of 64, x 16-byte aligned), one launch per 256 or fewer of
-// the n_b columns; *used = false otherwise.
+// The prefill prepare kernel on the tensor cores where it applies (B = 64 ..
+// 512, n_b a multiple of 64, x 16-byte aligned); *used = false otherwise.
 cudaError_t launch_prep_tc(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws, cudaStream_t st,
                            bool* used) {
   const Geometry& g = pl->geo;
   *used = false;
-  if (g.block != 128 || g.n_b % 64 != 0 || (reinterpret_cast<uintptr_t>(x) & 15u)) return cudaSuccess;
+  if (g.block < 64 || g.block > 512 || g.n_b % 64 != 0 || (reinterpret_cast<uintptr_t>(x) & 15u)) return cudaSuccess;
   auto enc = encode_fn();
   if (!enc) return cudaSuccess;
   const WsLayout L = workspace_layout(pl, M);
   uint8_t* wbase = static_cast<uint8_t*>(ws);
   const int64_t R = (int64_t)M * g.nblk;
   if (R >= (int64_t(1) << 31) - kPtRows) return cudaSuccess;
-  const int nparts = (g.n_b + 255) / 256;
-  CUtensorMap xmap, ghmap[16], glmap[16];
-  if (nparts > 16) return cudaSuccess;
-  const cuuint32_t estr[2] = {1, 1};
-  {
-    const cuuint64_t dims[2] = {128, (cuuint64_t)R};
-    const cuuint64_t strides[1] = {256};
-    const cuuint32_t box[2] = {64, (cuuint32_t)kPtRows};
-    if (enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(x), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaSuccess;
-  }
-  int j0s[16], ncols[16];
-  for (int q = 0, j0 = 0; q < nparts; ++q) {
-    const int ncol = std::min(256, g.n_b - j0);
-    const cuuint64_t dims[2] = {128, (cuuint64_t)ncol};
-    const cuuint64_t strides[1] = {256};
-    const cuuint32_t box[2] = {64, (cuuint32_t)ncol};
-    if (enc(&ghmap[q], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, pl->d_g_hi + (size_t)j0 * 128, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-        enc(&glmap[q], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, pl->d_g_lo + (size_t)j0 * 128, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaSuccess;
-    j0s[q] = j0;
-    ncols[q] = ncol;
-    j0 += ncol;
-  }
   PrepTcParams p;   // (a timeout is recorded under this kernel's own call number)
   p.xtb = reinterpret_cast<uint16_t*>(wbase + L.xt);
   p.rec = reinterpret_cast<uint64_t*>(wbase + L.err);
+  p.call = call_tag(next_call_number());
   p.R = R; p.k_eff = g.k_eff; p.kpad = g.k_eff_pad;
   p.M = M; p.nblk = g.nblk; p.n_b = g.n_b; p.ternary = pl->desc.quantizer == SDQ_TERNARY;
   p.ntile = (int)((R + kPtRows - 1) / kPtRows);
-  const size_t smem_max = 1024 + 4 * (size_t)256 * 128 + kPtSlots * (size_t)kPtXTile;
-  cudaError_t e = cudaFuncSetAttribute(prep_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+  p.nch = g.block / 64;
+  // the most columns per CTA (64 .. 256, dividing n_b, with two ring slots
+  // beside them) that still give every SM a CTA, else 64
+  const int64_t sms = std::max(1, pl->sm_count);
+  p.ncol = 64;
+  for (int c = 128; c <= 256; c += 64)
+    if (g.n_b % c == 0 && 1024 + 256 * p.nch * c + 2 * kPtChunk <= kPtSmem && p.ntile * (int64_t)(g.n_b / c) >= sms)
+      p.ncol = c;
+  const int gbytes = 256 * p.nch * p.ncol;
+  // two CTAs per SM where their parts of G leave room
+  const bool two = 2 * (2048 + gbytes + 4 * kPtChunk) <= kPtSmem;
+  p.slots = two ? 4 : std::min(kPtMaxSlots, (kPtSmem - 1024 - gbytes) / kPtChunk);
+  const int parts = g.n_b / p.ncol;
+  CUtensorMap xmap, ghmap, glmap;
+  const cuuint32_t estr[2] = {1, 1};
+  const cuuint64_t strides[1] = {(cuuint64_t)g.block * 2};
+  auto map = [&](CUtensorMap* m, const uint16_t* ptr, int64_t rows, int box_rows) {
+    const cuuint64_t dims[2] = {(cuuint64_t)g.block, (cuuint64_t)rows};
+    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(ptr), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  if (!map(&xmap, x, R, kPtRows) || !map(&ghmap, pl->d_g_hi, g.n_b, p.ncol) || !map(&glmap, pl->d_g_lo, g.n_b, p.ncol))
+    return cudaSuccess;
+  static std::atomic<int> smem_set[64];
+  cudaError_t e = smem_limit_once(prep_tc_kernel, kPtSmem, pl->device, smem_set);
   if (e != cudaSuccess) return e;
-  const int grid = std::min(p.ntile, std::max(1, pl->sm_count));
   *used = true;
-  for (int q = 0; q < nparts; ++q) {
-    p.call = call_tag(next_call_number());
-    p.j0 = j0s[q];
-    p.ncol = ncols[q];
-    const size_t smem = 1024 + 4 * (size_t)p.ncol * 128 + kPtSlots * (size_t)kPtXTile;
-    e = launch_pdl(prep_tc_kernel, dim3(grid), dim3(kPtThreads), smem, st, xmap, ghmap[q], glmap[q], p);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  const int64_t ctas = sms * (two ? 2 : 1);
+  const int gx = (int)std::min<int64_t>(p.ntile, std::max<int64_t>(1, (ctas + parts - 1) / parts));
+  return launch_pdl(prep_tc_kernel, dim3(gx, parts), dim3(kPtThreads),
+                    (size_t)(1024 + gbytes + p.slots * kPtChunk), st, xmap, ghmap, glmap, p);
 }
 }  // namespace sdq
