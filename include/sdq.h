@@ -153,7 +153,8 @@ int sdq_build_gptq_table(const sdq_layer_desc* desc, const int8_t* had_signs, fl
 
 /* Host-only (no GPU needed): the launch shape the decode contraction takes
  * at batch M (1..64) on a device with `sm_count` SMs, as sdq_plan_create
- * chooses it.  Writes 16 int64 values to `out_host`: T (e2m1 terms per
+ * chooses it (its 4-bit kernel; the larger of these batches contract with the
+ * prefill kernel, see sdq_contract).  Writes 16 int64 values to `out_host`: T (e2m1 terms per
  * activation), NP (MMA N), S (k chunks), P (CTAs per chunk), CB (128-code
  * blocks per chunk), ring (stages in the shared-memory ring), sb (blocks per
  * stage), nbuf (accumulators per pipeline), dynamic shared memory bytes,
@@ -239,8 +240,8 @@ int sdq_unpack_base3(sdq_plan plan, const uint8_t* codes_base3, uint32_t* codes_
 /* x_tilde = G x_b for every block b of every row of x (device, bf16 bits,
  * M x k_in row-major), written into the workspace `ws` for sdq_contract.
  * M <= 64: x_tilde is written in fp32 (M x K_pad, K_pad = 128
- * ceil(K_eff / 128), padding 0); the decode kernel forms its tensor-core B
- * operand from it.  M > 64: x_tilde is written in bf16 in the permuted K
+ * ceil(K_eff / 128), padding 0), with the operand that the contraction of
+ * this batch size reads.  M > 64: x_tilde is written in bf16 in the permuted K
  * order the prefill kernel reads.  Kernels are launched with programmatic
  * dependent launch.  Errors: INVALID_ARG (also when the current device is
  * not the plan's), WORKSPACE, CUDA. */
@@ -259,7 +260,10 @@ int sdq_prep_activations(sdq_plan plan, const uint16_t* x, int32_t M,
  * thread blocks with a deterministic last-block reduction: results are
  * bit-for-bit reproducible for a given plan, M and device; the launch shape
  * is chosen per batch size at plan creation and can be queried with
- * sdq_decode_launch_shape).  M > 64: tcgen05 bf16 prefill kernel.  Errors as
+ * sdq_decode_launch_shape).  M > 64, and below that from M = 24, 40 or 56 on
+ * (by the layer's size, where B is 64 .. 512 and n_b a multiple of 64): tcgen05
+ * bf16 prefill kernel, x_tilde in bf16, K split over a cluster's thread
+ * blocks whose sums are added in a fixed order.  Errors as
  * sdq_prep_activations, and UNSUPPORTED when no launch shape fits. */
 int sdq_contract(sdq_plan plan, const uint32_t* codes_tiled, const float* alpha, int32_t M,
                  float* y, void* ws, size_t ws_bytes, void* stream);
@@ -295,7 +299,7 @@ int sdq_linear_forward(sdq_plan plan, const uint32_t* codes_tiled, const float* 
 int sdq_forward_kernels(sdq_plan plan, int32_t M, const uint16_t* x);
 
 /* The route sdq_linear_forward takes for this plan and batch M: 1 decode
- * (M <= 64: prepare kernel, tcgen05 block-scaled 4-bit contraction); 2
+ * (M <= 64: prepare kernel and contraction, see sdq_contract); 2
  * prefill in the code domain (x_tilde = G x in bf16, tcgen05 bf16
  * contraction with the codes); 3 dense (M >= 768 where the plan allows it:
  * B = 128, n_b a multiple of 64 up to 384: the kernel rebuilds the weights

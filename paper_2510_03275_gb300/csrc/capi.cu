@@ -61,6 +61,8 @@ uint64_t call_tag(uint64_t n) {
   return v | (1ull << 47);
 }
 
+bool prefill_route(const sdq_plan_s* p, int M) { return M >= p->wide_min; }
+
 WsLayout workspace_layout(const sdq_plan_s* pl, int M) {
   const Geometry& g = pl->geo;
   WsLayout L{};
@@ -80,12 +82,23 @@ WsLayout workspace_layout(const sdq_plan_s* pl, int M) {
     off = align_up(off + sizeof(uint64_t) * (size_t)g.ntiles, 256);
     L.err = off;                                   // call record
     off = align_up(off + 2 * sizeof(uint64_t), 256);
+    L.least = off;
+    if (prefill_route(pl, M)) {
+      // call record, bf16 x_tilde, then (sdq_prep_activations alone) fp32
+      // x_tilde; a forward call needs the first two, less than the above
+      L.err = 0;
+      L.xtb = 256;
+      L.xt = L.xtb + align_up(sizeof(uint16_t) * (size_t)M * g.k_eff_pad, 256);
+      off = std::max(off, L.xt + align_up(sizeof(float) * (size_t)M * g.k_eff_pad, 256));
+    }
   } else {
+    L.xtb = off;
     off = align_up(off + sizeof(uint16_t) * (size_t)M * g.k_eff_pad, 256);
     L.what = off;                                  // dense route: W', n_out x k_in bf16
     if (dense_route_applies(pl, M)) off = align_up(off + sizeof(uint16_t) * (size_t)g.n_out * g.k_in, 256);
     L.bimg = L.sfbw = L.part = L.cnt = L.err = off;   // call record only
     off = align_up(off + 2 * sizeof(uint64_t), 256);
+    L.least = off;
   }
   L.total = off;
   return L;
@@ -182,6 +195,7 @@ extern "C" int sdq_plan_create(const sdq_layer_desc* desc, const int8_t* had_sig
     sdq_plan_destroy(p);
     return SDQ_ERR_CUDA;
   }
+  p->wide_min = wide_min_batch(p);
   for (int M = 1; M <= kMaxDecodeM; ++M) p->dcfg[M] = decode_config_search(p, M);
   *out = p;
   return SDQ_OK;
@@ -223,13 +237,14 @@ extern "C" int sdq_unpack(sdq_plan p, const uint32_t* tiled, uint32_t* plain, ui
   return cuda_status(launch_unpack(p, tiled, plain, bad_count, (cudaStream_t)stream));
 }
 
-static int check_ws(sdq_plan p, int32_t M, const void* ws, size_t ws_bytes) {
+// `forward`: the workspace of sdq_linear_forward, which may be smaller.
+static int check_ws(sdq_plan p, int32_t M, const void* ws, size_t ws_bytes, bool forward = false) {
   if (!p || M < 1 || M > 65535) return SDQ_ERR_INVALID_ARG;
   const int dv = sdq_check_device(p);
   if (dv != SDQ_OK) return dv;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SDQ_ERR_INVALID_ARG;
-  if (ws_bytes < workspace_layout(p, M).total) return SDQ_ERR_WORKSPACE;
-  return SDQ_OK;
+  const WsLayout L = workspace_layout(p, M);
+  return ws_bytes < (forward ? L.least : L.total) ? SDQ_ERR_WORKSPACE : SDQ_OK;
 }
 
 extern "C" int sdq_prep_activations(sdq_plan p, const uint16_t* x, int32_t M, void* ws,
@@ -242,12 +257,12 @@ extern "C" int sdq_prep_activations(sdq_plan p, const uint16_t* x, int32_t M, vo
 
 static int contract(sdq_plan p, const uint32_t* codes_tiled, const float* alpha, int32_t M, float* y,
                     void* ws, size_t ws_bytes, void* stream, int early, int y_mode) {
-  int st = check_ws(p, M, ws, ws_bytes);
+  int st = check_ws(p, M, ws, ws_bytes, early != 0);   // (early: behind this call's own prepare kernel)
   if (st != SDQ_OK) return st;
   if (!codes_tiled || !alpha || !y || !aligned16(codes_tiled) || !aligned16(y)) return SDQ_ERR_INVALID_ARG;
-  cudaError_t e = M <= kMaxDecodeM
-                      ? launch_decode(p, codes_tiled, alpha, M, y, ws, (cudaStream_t)stream, early, y_mode)
-                      : launch_prefill(p, codes_tiled, alpha, M, y, ws, (cudaStream_t)stream, early);
+  cudaError_t e = prefill_route(p, M)
+                      ? launch_prefill(p, codes_tiled, alpha, M, y, ws, (cudaStream_t)stream, early, y_mode)
+                      : launch_decode(p, codes_tiled, alpha, M, y, ws, (cudaStream_t)stream, early, y_mode);
   if (e == cudaErrorNotSupported) return SDQ_ERR_UNSUPPORTED;
   return cuda_status(e);
 }
@@ -272,8 +287,8 @@ extern "C" int sdq_linear_forward(sdq_plan p, const uint32_t* codes_tiled, const
                                   void* stream) {
   // Decode batches: the prepare kernel also clears y, and the decode kernel
   // adds its split-K partial sums into it with float atomics.
-  const bool zero_y = p && M >= 1 && M <= kMaxDecodeM && decode_config(p, M).S > 1;
-  int st = check_ws(p, M, ws, ws_bytes);
+  const bool zero_y = p && M >= 1 && M <= kMaxDecodeM && !prefill_route(p, M) && decode_config(p, M).S > 1;
+  int st = check_ws(p, M, ws, ws_bytes, true);
   if (st != SDQ_OK) return st;
   if (!x || !aligned16(x) || !y || !aligned16(y)) return SDQ_ERR_INVALID_ARG;
   if (M > kMaxDecodeM && dense_route_applies(p, M)) {
@@ -282,7 +297,7 @@ extern "C" int sdq_linear_forward(sdq_plan p, const uint32_t* codes_tiled, const
     const cudaError_t e = launch_dense_forward(p, codes_tiled, alpha, x, M, y, ws, (cudaStream_t)stream);
     if (e != cudaErrorNotSupported) return cuda_status(e);
   }
-  st = cuda_status(launch_prep(p, x, M, ws, (cudaStream_t)stream, zero_y ? y : nullptr));
+  st = cuda_status(launch_prep(p, x, M, ws, (cudaStream_t)stream, zero_y ? y : nullptr, /*forward=*/true));
   if (st != SDQ_OK) return st;
   return contract(p, codes_tiled, alpha, M, y, ws, ws_bytes, stream, 1, zero_y ? kYZeroed : kYStore);
 }

@@ -19,9 +19,14 @@ inline const DecodeConfig& decode_config(const sdq_plan_s* plan, int M) { return
 // tile; err: the call record (two 64-bit words, see call_record_*).
 struct WsLayout {
   size_t xt, bimg, sfbw, part, cnt, err, total;
+  size_t xtb;    // bf16 x_tilde of the prefill contraction (prefill_route)
+  size_t least;  // bytes that sdq_linear_forward needs
   size_t what;   // rebuilt weights W' (n_out x k_in bf16) of the dense large-batch route
 };
 WsLayout workspace_layout(const sdq_plan_s* plan, int M);
+// Whether batch M contracts with the prefill kernel (M > 64, and the decode
+// batches for which it is the faster one).
+bool prefill_route(const sdq_plan_s* plan, int M);
 // SDQ_OK when the current device is the plan's, else SDQ_ERR_INVALID_ARG (or
 // SDQ_ERR_CUDA).
 int sdq_check_device(const sdq_plan_s* p);
@@ -42,8 +47,13 @@ cudaError_t launch_pack(const sdq_plan_s* p, const uint32_t* plain, uint32_t* ti
 cudaError_t launch_unpack(const sdq_plan_s* p, const uint32_t* tiled, uint32_t* plain,
                           uint32_t* bad, cudaStream_t st);
 // y_zero (M x n_out, may be null): cleared by the decode prepare kernel.
+// forward: only what this call's contraction reads (else also the fp32 x_tilde
+// of a decode batch that contracts with the prefill kernel).
 cudaError_t launch_prep(const sdq_plan_s* p, const uint16_t* x, int M, void* ws, cudaStream_t st,
-                        float* y_zero = nullptr);
+                        float* y_zero = nullptr, bool forward = false);
+// Decode batches from here on contract with the prefill kernel (kMaxDecodeM +
+// 1: none do).
+int wide_min_batch(const sdq_plan_s* p);
 // The dense large-batch route (rebuild W' = 2 C G, then y = alpha / 2 W' x):
 // whether it applies to plan p at batch M, and its two launches.
 bool dense_route_applies(const sdq_plan_s* p, int M);
@@ -69,7 +79,7 @@ cudaError_t launch_decode(const sdq_plan_s* p, const uint32_t* codes, const floa
 // multiple of 64), so that each decode CTA copies its chunk's part.
 bool decode_image(const sdq_plan_s* p);
 cudaError_t launch_prefill(const sdq_plan_s* p, const uint32_t* codes, const float* alpha, int M,
-                           float* y, void* ws, cudaStream_t st, int early);
+                           float* y, void* ws, cudaStream_t st, int early, int y_mode);
 // Fills the plan's pf_clusters (launch-shape facts of the device).
 cudaError_t prefill_occupancy(sdq_plan_s* p);
 cudaError_t launch_read_prep(const sdq_plan_s* p, int M, const void* ws, float* out, cudaStream_t st);

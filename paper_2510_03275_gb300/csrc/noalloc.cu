@@ -51,8 +51,7 @@ int noalloc_scratch(sdq_plan p, int32_t M, void** ws) {
   if (!p || M < 1 || M > sdq::kMaxDecodeM) return SDQ_ERR_INVALID_ARG;
   int st = sdq::sdq_check_device(p);
   if (st != SDQ_OK) return st;
-  const size_t need = sdq_workspace_bytes(p, M);
-  if (need == 0) return SDQ_ERR_INVALID_ARG;
+  const size_t need = sdq::workspace_layout(p, M).least;
   if (need > kNoAllocScratchBytes) return SDQ_ERR_WORKSPACE;
   return scratch_for_current_device(ws);
 }

@@ -1,4 +1,4 @@
-// K5: prefill contraction (M > 64) on the 5th-generation tensor cores.
+// K5: prefill contraction (M > 64, and the larger decode batches) on the 5th-generation tensor cores.
 //
 //   y[m, r] = alpha_r * sum_j c[r, j] * x_tilde[m, j]        (section 3.5, eq. 12)
 //
@@ -73,7 +73,7 @@ struct PrefillParams {
   uint64_t* rec;       // call record
   uint64_t call;
   int M, N, ngroups, wpg, nks, quantizer;
-  int bn, stages, split, early;
+  int bn, stages, split, early, add;   // add: y += the result
 };
 
 __device__ __forceinline__ void cluster_sync() {
@@ -250,7 +250,11 @@ __global__ void __launch_bounds__(kThreads, 2)
         } else if (row < p.N) {
 #pragma unroll
           for (int i = 0; i < 16; ++i)
-            if (c0 + i < c1) p.y[(size_t)(m0 + c0 + i) * p.N + row] = __uint_as_float(a[i]) * sa;
+            if (c0 + i < c1) {
+              float* o = p.y + (size_t)(m0 + c0 + i) * p.N + row;
+              if (p.add) red_add_f32(o, __uint_as_float(a[i]) * sa);
+              else *o = __uint_as_float(a[i]) * sa;
+            }
         }
       }
     }
@@ -283,13 +287,17 @@ __global__ void __launch_bounds__(kThreads, 2)
       for (int i = 1; i < kMaxSplit; ++i)
         if (i < p.split) { t.x += v[i].x; t.y += v[i].y; t.z += v[i].z; t.w += v[i].w; }
       float* o = p.y + (size_t)(m0 + c) * p.N + row;
-      if (vec) {
-        *reinterpret_cast<float4*>(o) = make_float4(t.x * al[0], t.y * al[1], t.z * al[2], t.w * al[3]);
+      t = make_float4(t.x * al[0], t.y * al[1], t.z * al[2], t.w * al[3]);
+      if (vec && !p.add) {
+        *reinterpret_cast<float4*>(o) = t;
       } else {
-        if (row < p.N) o[0] = t.x * al[0];
-        if (row + 1 < p.N) o[1] = t.y * al[1];
-        if (row + 2 < p.N) o[2] = t.z * al[2];
-        if (row + 3 < p.N) o[3] = t.w * al[3];
+        const float tv[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (row + i < p.N) {
+            if (p.add) red_add_f32(o + i, tv[i]);
+            else o[i] = tv[i];
+          }
       }
     }
   }
@@ -570,7 +578,7 @@ __global__ void __launch_bounds__(kPtThreads, 1)
 void* tensor_map_encoder() { return reinterpret_cast<void*>(encode_fn()); }
 
 cudaError_t launch_prefill(const sdq_plan_s* pl, const uint32_t* codes, const float* alpha, int M,
-                           float* y, void* ws, cudaStream_t st, int early) {
+                           float* y, void* ws, cudaStream_t st, int early, int y_mode) {
   const Geometry& g = pl->geo;
   const WsLayout L = workspace_layout(pl, M);
   uint8_t* wbase = static_cast<uint8_t*>(ws);
@@ -582,7 +590,7 @@ cudaError_t launch_prefill(const sdq_plan_s* pl, const uint32_t* codes, const fl
   const cuuint64_t strides[1] = {(cuuint64_t)g.k_eff_pad * 2};
   const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)sh.bn};
   const cuuint32_t estr[2] = {1, 1};
-  CUresult cr = enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, wbase + L.xt, dims, strides, box, estr,
+  CUresult cr = enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, wbase + L.xtb, dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) return cudaErrorInvalidValue;
@@ -593,7 +601,7 @@ cudaError_t launch_prefill(const sdq_plan_s* pl, const uint32_t* codes, const fl
   p.M = M; p.N = g.n_out; p.ngroups = g.ngroups; p.wpg = g.wpg;
   p.nks = (int)(g.k_eff_pad / kBK);
   p.quantizer = pl->desc.quantizer;
-  p.bn = sh.bn; p.stages = sh.stages; p.split = sh.split; p.early = early;
+  p.bn = sh.bn; p.stages = sh.stages; p.split = sh.split; p.early = early; p.add = y_mode == kYAdd;
   cudaError_t e = prefill_smem_limit(pl->device);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
@@ -618,13 +626,27 @@ cudaError_t prefill_occupancy(sdq_plan_s* pl) {
   return e;
 }
 
+static bool prep_tc_takes(const Geometry& g) { return g.block >= 64 && g.block <= 512 && g.n_b % 64 == 0; }
+// The crossings of the two contractions per layer size (us a forward call at
+// OSR 2, 4-bit decode kernel / this one): 4096 x 4096 M = 24 16.1 / 13.4;
+// 22016 x 4096 M = 24 32.5 / 34.7, M = 40 42.8 / 37.0; 57344 x 8192 M = 48
+// 116 / 122, M = 64 136 / 124.  This one's time is nearly flat in M: the
+// expanded codes' stores into tensor memory (16 KB per 2 KB of codes) bound
+// it, about 290 cycles a stage and SM.
+int wide_min_batch(const sdq_plan_s* pl) {
+  const Geometry& g = pl->geo;
+  if (!prep_tc_takes(g) || !encode_fn()) return kMaxDecodeM + 1;
+  const int64_t codes = (int64_t)g.n_out * g.k_eff;
+  return codes <= 40000000 ? 24 : (codes <= 200000000 ? 40 : 56);
+}
+
 // The prefill prepare kernel on the tensor cores where it applies (B = 64 ..
 // 512, n_b a multiple of 64, x 16-byte aligned); *used = false otherwise.
 cudaError_t launch_prep_tc(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws, cudaStream_t st,
                            bool* used) {
   const Geometry& g = pl->geo;
   *used = false;
-  if (g.block < 64 || g.block > 512 || g.n_b % 64 != 0 || (reinterpret_cast<uintptr_t>(x) & 15u)) return cudaSuccess;
+  if (!prep_tc_takes(g) || (reinterpret_cast<uintptr_t>(x) & 15u)) return cudaSuccess;
   auto enc = encode_fn();
   if (!enc) return cudaSuccess;
   const WsLayout L = workspace_layout(pl, M);
@@ -632,7 +654,7 @@ cudaError_t launch_prep_tc(const sdq_plan_s* pl, const uint16_t* x, int M, void*
   const int64_t R = (int64_t)M * g.nblk;
   if (R >= (int64_t(1) << 31) - kPtRows) return cudaSuccess;
   PrepTcParams p;   // (a timeout is recorded under this kernel's own call number)
-  p.xtb = reinterpret_cast<uint16_t*>(wbase + L.xt);
+  p.xtb = reinterpret_cast<uint16_t*>(wbase + L.xtb);
   p.rec = reinterpret_cast<uint64_t*>(wbase + L.err);
   p.call = call_tag(next_call_number());
   p.R = R; p.k_eff = g.k_eff; p.kpad = g.k_eff_pad;

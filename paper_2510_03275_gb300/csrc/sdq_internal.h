@@ -92,6 +92,7 @@ struct sdq_plan_s {
   uint16_t* d_gt_lo;   // code expansion's K order (prefill_pos64); null where the dense
                        // large-batch route does not apply (B != 128, n_b not a multiple
                        // of 64 or above kDenseMaxNb)
+  int wide_min;        // batches from here on contract with the prefill kernel (csrc/prefill.cu)
   int half_shift;      // A_enc[j + n_b / 2][k] = +-A_enc[j][k] (- for k >= B / 2), every bit (csrc/encode.cu)
   int pf_clusters[9];  // prefill kernel: clusters of S CTAs held at once with one CTA per SM
   sdq::DecodeConfig dcfg[sdq::kMaxDecodeM + 1];  // decode launch shape per batch size
