@@ -808,13 +808,14 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
 
 // Launch shape for batch M: the pipelines, TMEM slots, accumulators, stage
 // size and (S, P) grid of at most one CTA per SM (more only where nothing
-// else fits) that minimise a time model fitted to per-stage timestamps of
-// the kernel: per CTA the stage rate of its MMA pipelines (about 150 cycles
-// per MMA and 550 per stage on an issuing thread, the pipelines side by
-// side) and of its 4 expander sets (a set waits for the MMAs of its
-// previous stage when it owns one TMEM slot), against the HBM time of the
-// codes (the bytes in flight capped by the CTAs' code rings, at a loaded
-// latency), plus the prologue (B operand and scales) and the split-K tail.
+// else fits) that minimise a time model fitted to forced shapes of 9 layer
+// sizes at M = 1 .. 32: per CTA the stage rate of the tensor core (55 + 0.65 NP
+// cycles per MMA) and of its 4 expander sets (1600 cycles per stage and 300
+// per block), against the HBM time of the codes (the bytes in flight capped
+// by the CTAs' code rings, at a loaded latency), plus the prologue (B operand
+// and scales) and the split-K tail.  Large stages matter most: with two
+// pipelines' accumulators TMEM holds stages of 4 blocks up to M = 8, with four
+// only 2 (57344 x 16384 codes at M = 8: 52.7 us against 39.7).
 // TMEM holds, from column 0: ns A slots of sb blocks (16 sb columns each),
 // the A scales (4 columns), per slot the B scales of its sb blocks (a set of
 // ss = 4 ceil(ceil(NP / 32) / 4) columns per block: scale columns start on a
@@ -832,11 +833,11 @@ DecodeConfig decode_config_search(const sdq_plan_s* pl, int M) {
   const int sms = std::max(1, pl->sm_count);
   const int blk_bytes = kTileRows * kBlk * g.bits / 8;
   const double clk = 1.9e9;
-  const double hbm = 6.0e12, cta_bw = 30e9;                    // bytes/s: HBM, one CTA's copy ring
-  const double l2_bw = 20e12;                                  // bytes/s: L2 reads of streamed B rows
-  const double t_tail = 2.0e-6, ring_latency = 4.0e-6;   // a ring slot's round trip under load
-  const double c_mma = 150.0 + 0.5 * best.NP, c_stage = 550.0;   // issuing thread, cycles
-  const double c_xblk = 200.0, c_xstage = 600.0;                 // expander set, cycles
+  const double hbm = 6.4e12, cta_bw = 45e9;              // bytes/s: HBM, one CTA's copy ring
+  const double l2_bw = 20e12;                            // bytes/s: L2 reads of streamed B rows
+  const double t_tail = 2.8e-6, ring_latency = 2.2e-6;   // a ring slot's round trip under load
+  const double c_mma = 55.0 + 0.65 * best.NP, c_stage = 250.0;   // tensor core and issuing warp, cycles
+  const double c_xblk = 300.0, c_xstage = 1600.0;                // expander set, cycles
   double best_t = 1e30;
   const int pipes[3] = {4, 2, 1};
   const int MT = M * best.T;
@@ -886,10 +887,12 @@ DecodeConfig decode_config_search(const sdq_plan_s* pl, int M) {
           const int spu = bs ? std::max((2 * npr + sb - 1) / sb, std::min(2, npr))
                              : std::max((CB + sb - 1) / sb, std::min(2, CB));
           if (spu > kMaxSpu) continue;
-          const double issue = 2.0 * sb * c_mma + c_stage;        // cycles per stage, one pipeline
-          const double expand = c_xstage + c_xblk * sb;           // cycles per stage, one set
-          const double set_cyc = ns == 4 ? std::max(expand, issue * 4.0 / np + 300.0) : std::max(expand, issue * 2.0 / np);
-          const double mma_rate = std::min(np / issue, kExpSets / set_cyc) * clk;   // stages per second per CTA
+          // cycles per stage: the tensor core, which the pipelines share, and
+          // the issuing warps; an expander set (its one TMEM slot of four
+          // included: it waits for the slot's MMAs)
+          const double mma = std::max(2.0 * sb * c_mma, (2.0 * sb * c_mma + c_stage) / np);
+          const double set_cyc = c_xstage + c_xblk * sb;
+          const double mma_rate = std::min(1.0 / mma, kExpSets / set_cyc) * clk;   // stages per second per CTA
           // the prologue: the wait for the prepare kernel, the B operand (image
           // copy or terms formed in the CTA)
           const double t_build = bs ? 2.0e-6 : 2.0e-6 + (b_bytes + sfb_bytes) / 25e9 + CB * M * best.T * 2.0e-9;
@@ -902,9 +905,9 @@ DecodeConfig decode_config_search(const sdq_plan_s* pl, int M) {
             // share of HBM bandwidth, and the rate its MMA pipelines and
             // expander sets sustain (and, streaming B, its share of the L2's
             // bandwidth for the B rows); every row tile adds a cost that grows
-            // with the k chunks adding into the same rows of y (accumulator
-            // hand-off, epilogue, split-K contention: fitted to measured
-            // calls), every call a prologue and a tail.
+            // with the pipelines whose accumulators its epilogue adds and
+            // with the k chunks adding into the same rows of y (fitted to
+            // measured calls), every call a prologue and a tail.
             const double tile_bytes = (double)CB * blk_bytes;
             double rate = std::min({cta_bw, hbm / std::min(grid, sms), mma_rate * code_slot,
                                     (double)ring * code_slot / ring_latency});
@@ -914,7 +917,7 @@ DecodeConfig decode_config_search(const sdq_plan_s* pl, int M) {
             // beside the next tile's MMAs with two accumulators, else between
             const double t_stream = tile_bytes / rate;
             const double t_tile = nbuf == 2 ? std::max(t_stream, t_epi[pi]) : t_stream + t_epi[pi];
-            const double t_cta = units * (t_tile + 0.8e-6 + 0.15e-6 * S);
+            const double t_cta = units * (t_tile + 0.3e-6 + 0.1e-6 * np + 0.1e-6 * S);
             const double t = waves * t_cta + t_build + t_tail;
             if (t < best_t * 0.999) {
               best_t = t;
