@@ -62,9 +62,10 @@ cudaError_t launch_dense_forward(const sdq_plan_s* p, const uint32_t* codes, con
 // cuTensorMapEncodeTiled from the driver (null if unavailable), as void*.
 void* tensor_map_encoder();
 // Prefill prepare (M > 64) on the tensor cores where the layer allows it;
-// *used = false (nothing launched) otherwise.
+// *used = false (nothing launched) otherwise.  fp32_too: x_tilde also in fp32
+// (the decode layout's xt region).
 cudaError_t launch_prep_tc(const sdq_plan_s* p, const uint16_t* x, int M, void* ws, cudaStream_t st,
-                           bool* used);
+                           bool* used, bool fp32_too);
 // early = 1: the decode kernel starts streaming codes before waiting for the
 // preceding grid (valid only behind this library's own prep kernels).
 // y_mode: kYStore: y = the result (split-K by the deterministic ticket

@@ -411,6 +411,7 @@ constexpr int kPtSmem = 226 * 1024;
 
 struct PrepTcParams {
   uint16_t* xtb;
+  float* xt;         // x_tilde in fp32 too, natural order (null: not)
   uint64_t* rec;
   uint64_t call;
   int64_t R, k_eff, kpad;
@@ -514,7 +515,12 @@ __global__ void __launch_bounds__(kPtThreads, 1)
       for (int64_t z = (int64_t)blockIdx.x * (32 * kPtEpiWarps) + et; z < (int64_t)p.M * ((p.kpad - p.k_eff) / 8);
            z += (int64_t)gridDim.x * (32 * kPtEpiWarps)) {
         const int64_t per = (p.kpad - p.k_eff) / 8, m = z / per;
-        *reinterpret_cast<uint4*>(p.xtb + m * p.kpad + p.k_eff + 8 * (z - m * per)) = make_uint4(0, 0, 0, 0);
+        const int64_t at = m * p.kpad + p.k_eff + 8 * (z - m * per);
+        *reinterpret_cast<uint4*>(p.xtb + at) = make_uint4(0, 0, 0, 0);
+        if (p.xt) {
+          *reinterpret_cast<uint4*>(p.xt + at) = make_uint4(0, 0, 0, 0);
+          *reinterpret_cast<uint4*>(p.xt + at + 4) = make_uint4(0, 0, 0, 0);
+        }
       }
     const int cw = p.ncol / 2;                                  // this warp's columns
     const uint32_t lq = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(half * cw);
@@ -527,7 +533,8 @@ __global__ void __launch_bounds__(kPtThreads, 1)
       const int64_t row = (int64_t)t * kPtRows + 32 * q + lane;
       const bool live = row < p.R;
       const int64_t m = live ? row / p.nblk : 0;
-      uint16_t* out = p.xtb + m * p.kpad + (live ? (row - m * p.nblk) * p.n_b : 0) + j0 + half * cw;
+      const int64_t at = m * p.kpad + (live ? (row - m * p.nblk) * p.n_b : 0) + j0 + half * cw;
+      uint16_t* out = p.xtb + at;
       const uint32_t acol = (uint32_t)(s * p.ncol);
       // 32 columns at a time: a ternary operand permutes within 16, a binary
       // one within 32 positions (prefill_pos64); physical pair (2k, 2k + 1)
@@ -560,6 +567,14 @@ __global__ void __launch_bounds__(kPtThreads, 1)
           o[1] = make_uint4(w[4], w[5], w[6], w[7]);
           o[2] = make_uint4(w[8], w[9], w[10], w[11]);
           o[3] = make_uint4(w[12], w[13], w[14], w[15]);
+          if (p.xt) {
+            uint4* f = reinterpret_cast<uint4*>(p.xt + at + c0);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              f[k] = make_uint4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
+              f[4 + k] = make_uint4(b[4 * k], b[4 * k + 1], b[4 * k + 2], b[4 * k + 3]);
+            }
+          }
         }
       }
     }
@@ -643,7 +658,7 @@ int wide_min_batch(const sdq_plan_s* pl) {
 // The prefill prepare kernel on the tensor cores where it applies (B = 64 ..
 // 512, n_b a multiple of 64, x 16-byte aligned); *used = false otherwise.
 cudaError_t launch_prep_tc(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws, cudaStream_t st,
-                           bool* used) {
+                           bool* used, bool fp32_too) {
   const Geometry& g = pl->geo;
   *used = false;
   if (!prep_tc_takes(g) || (reinterpret_cast<uintptr_t>(x) & 15u)) return cudaSuccess;
@@ -655,6 +670,7 @@ cudaError_t launch_prep_tc(const sdq_plan_s* pl, const uint16_t* x, int M, void*
   if (R >= (int64_t(1) << 31) - kPtRows) return cudaSuccess;
   PrepTcParams p;   // (a timeout is recorded under this kernel's own call number)
   p.xtb = reinterpret_cast<uint16_t*>(wbase + L.xtb);
+  p.xt = fp32_too ? reinterpret_cast<float*>(wbase + L.xt) : nullptr;
   p.rec = reinterpret_cast<uint64_t*>(wbase + L.err);
   p.call = call_tag(next_call_number());
   p.R = R; p.k_eff = g.k_eff; p.kpad = g.k_eff_pad;

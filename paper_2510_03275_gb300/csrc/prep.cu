@@ -329,13 +329,12 @@ cudaError_t launch_prep(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws
   const WsLayout L = workspace_layout(pl, M);
   uint8_t* base = static_cast<uint8_t*>(ws);
   const int vec = (g.block % 32 == 0) && ((reinterpret_cast<uintptr_t>(x) & 15u) == 0);
-  const bool prefill = prefill_route(pl, M);
-  if (M <= kMaxDecodeM && !(prefill && forward)) {
+  if (!prefill_route(pl, M)) {
     const DecodeConfig& dc = decode_config(pl, M);
     DecPrepParams p;
     p.x = x; p.g_hi = pl->d_g_hi; p.g_lo = pl->d_g_lo;
     p.xt = reinterpret_cast<float*>(base + L.xt);
-    p.bimg = decode_image(pl) && !prefill ? base + L.bimg : nullptr;
+    p.bimg = decode_image(pl) ? base + L.bimg : nullptr;
     p.sfbw = base + L.sfbw;
     p.T = dc.T; p.NP = dc.NP;
     p.y_zero = y_zero;
@@ -351,11 +350,10 @@ cudaError_t launch_prep(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws
                                     pl->device, smem_set);
     if (e != cudaSuccess) return e;
     dim3 grid((g.n_b + 63) / 64, (g.nblk + 15) / 16, M);
-    e = launch_pdl(prep_decode_kernel, grid, dim3(128), smem, st, p);
-    if (e != cudaSuccess || !prefill) return e;
+    return launch_pdl(prep_decode_kernel, grid, dim3(128), smem, st, p);
   }
   bool used = false;
-  cudaError_t et = launch_prep_tc(pl, x, M, ws, st, &used);
+  cudaError_t et = launch_prep_tc(pl, x, M, ws, st, &used, M <= kMaxDecodeM && !forward);
   if (et != cudaSuccess || used) return et;
   PrepParams p;
   p.x = x; p.g_hi = pl->d_g_hi; p.g_lo = pl->d_g_lo;
