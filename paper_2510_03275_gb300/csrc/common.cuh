@@ -369,6 +369,20 @@ __device__ __forceinline__ void bulk_g2s_hint_warp(void* dst, const void* src, u
                "l"(policy) : "memory");
 }
 
+// TMA store of a shared-memory tile (one thread; its groups complete in
+// order): the tile may be rewritten after bulk_store_wait_read (at most N
+// stores still reading), and is in memory after bulk_store_wait_all.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];\n"
+               "cp.async.bulk.commit_group;\n" ::"l"(reinterpret_cast<uint64_t>(map)),
+               "r"(smem_u32(src)), "r"(c0), "r"(c1) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void bulk_store_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;\n" :: "n"(N) : "memory");
+}
+__device__ __forceinline__ void bulk_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
+
 // Two fp32 values to a byte of e2m1 codes (round to nearest even, saturating
 // at +-6): `lo` in bits 0-3, `hi` in bits 4-7; `q` receives the two values
 // the codes stand for (exact).

@@ -51,6 +51,7 @@ __host__ __device__ constexpr uint32_t f16_idesc(int n) {
 constexpr int kRbStages = 6;
 constexpr int kRbEpiWarp0 = 10;
 constexpr int kRbThreads = 32 * 14;
+constexpr int kRbHalf = 128 * 128;          // epilogue buffer: 128 rows x 64 columns of bf16 W'
 constexpr int kRbCTile = 128 * 16;          // code slab of a stage: 128 rows x 64 codes, at most 2 KB
 constexpr uint32_t kRbAcc = 128;            // accumulator columns (128 outputs k of a block)
 constexpr uint32_t kRbAcol = 2 * kRbAcc;    // first A slot column
@@ -58,15 +59,15 @@ constexpr uint32_t kRbAslot = kBK / 2;
 
 struct ReconParams {
   const uint32_t* codes;
-  uint16_t* w;          // W', n_out x k_in bf16 row-major (rows past n_out not written)
   uint64_t* rec;
   uint64_t call;
-  int n_out, k_in, nblk, n_b, ntiles, ngroups, wpg, quantizer, nitems;
+  int nblk, n_b, ngroups, wpg, quantizer, nitems;
+  int nstage;           // epilogue buffers (1 or 2)
 };
 
 __global__ void __launch_bounds__(kRbThreads, 1)
     recon_kernel(const __grid_constant__ CUtensorMap ghmap, const __grid_constant__ CUtensorMap glmap,
-                 ReconParams p) {
+                 const __grid_constant__ CUtensorMap wmap, ReconParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t g_full, full[kRbStages], empty[kRbStages], a_full[kRbStages],
       acc_full[2], acc_empty[2];
@@ -184,46 +185,55 @@ __global__ void __launch_bounds__(kRbThreads, 1)
       if (lane == 0) mbar_arrive(&a_full[s]);
     }
   } else {
-    // Epilogue: item it's accumulator -> W'[row, b B .. b B + 127] as bf16.
-    const int q = warp & 3, rr = 32 * q + lane;
+    // Epilogue: item it's accumulator -> W'[row, b B .. b B + 127] as bf16,
+    // 64 columns at a time through a shared-memory tile (128-byte rows and
+    // swizzle: no bank conflicts) and a TMA store of it (rows past n_out are
+    // clipped).  Stored from registers, a lane's row at a time, every 16 bytes
+    // were half a sector of their own, as long to issue as the item's MMAs.
+    const int q = warp & 3, rr = 32 * q + lane, et = tid - 32 * kRbEpiWarp0;
     const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16);
+    uint8_t* stage = c_tiles + kRbStages * kRbCTile;
+    int n = 0;   // halves stored
     for (int it = 0; it < nmine && ok; ++it) {
       const int a = it & 1;
-      ok = mbar_wait(&acc_full[a], (it >> 1) & 1);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = mbar_wait_warp(&acc_full[a], (it >> 1) & 1);
       if (!ok) break;
       tc_fence_after();
       const int item = (int)blockIdx.x + it * (int)gridDim.x;
       const int tile = item / p.nblk, b = item - tile * p.nblk;
-      const int row = tile * kTileRows + rr;
-      uint16_t* out = p.w + (size_t)row * p.k_in + (size_t)b * 128;
-      for (int c0 = 0; c0 < 128; c0 += 32) {
-        uint32_t u0[16], u1[16];
-        tmem_ld16(lane_addr + (uint32_t)a * kRbAcc + (uint32_t)c0, u0);
-        tmem_ld16(lane_addr + (uint32_t)a * kRbAcc + (uint32_t)c0 + 16, u1);
-        tmem_ld_wait();
-        if (c0 + 32 >= 128) {
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h, ++n) {
+        uint32_t w[32];   // 64 columns as bf16 pairs
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t u[16];
+          tmem_ld16(lane_addr + (uint32_t)a * kRbAcc + (uint32_t)(64 * h + 16 * c), u);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) w[8 * c + i] = pack_bf16x2(__uint_as_float(u[2 * i]), __uint_as_float(u[2 * i + 1]));
+        }
+        if (h == 1) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&acc_empty[a]);
         }
-        if (row < p.n_out) {
-          uint4* o = reinterpret_cast<uint4*>(out + c0);
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t* u = h ? u1 : u0;
-            o[2 * h] = make_uint4(pack_bf16x2(__uint_as_float(u[0]), __uint_as_float(u[1])),
-                                  pack_bf16x2(__uint_as_float(u[2]), __uint_as_float(u[3])),
-                                  pack_bf16x2(__uint_as_float(u[4]), __uint_as_float(u[5])),
-                                  pack_bf16x2(__uint_as_float(u[6]), __uint_as_float(u[7])));
-            o[2 * h + 1] = make_uint4(pack_bf16x2(__uint_as_float(u[8]), __uint_as_float(u[9])),
-                                      pack_bf16x2(__uint_as_float(u[10]), __uint_as_float(u[11])),
-                                      pack_bf16x2(__uint_as_float(u[12]), __uint_as_float(u[13])),
-                                      pack_bf16x2(__uint_as_float(u[14]), __uint_as_float(u[15])));
-          }
+        if (et == 0) {   // the store that last read this buffer is done with it
+          if (p.nstage == 2) bulk_store_wait_read<1>();
+          else bulk_store_wait_read<0>();
         }
+        named_bar_sync(1, 128);
+        uint8_t* sb = stage + (p.nstage == 2 ? (n & 1) * kRbHalf : 0) + rr * 128;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          *reinterpret_cast<uint4*>(sb + ((j ^ (rr & 7)) << 4)) =
+              make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+        fence_proxy_async_smem();
+        named_bar_sync(1, 128);
+        if (et == 0)
+          tma_store_2d(&wmap, sb - rr * 128, b * 128 + 64 * h, tile * kTileRows);
       }
     }
+    if (et == 0) bulk_store_wait_all();   // written before the CTA ends
   }
   if (!ok) call_record_fail(p.rec, p.call);
   tc_fence_before();
@@ -235,11 +245,12 @@ __global__ void __launch_bounds__(kRbThreads, 1)
 }
 
 // ------------------------------------------------------------ K7 dense GEMM
-// WT = 1 or 2 weight tiles of 128 rows per CTA against one 256-row batch
-// tile: with two, the x tile in shared memory serves two MMAs per K step
-// (shared-memory traffic per MMA 136 instead of 163 bytes per cycle of tensor
-// work), where the grid still fills the SMs.
-constexpr int kDnBN = 256;
+// WT = 1 or 2 weight tiles of 128 rows per CTA against one tile of `bn` batch
+// rows (a multiple of 16 up to 256): with two, the x tile in shared memory
+// serves two MMAs per K step (shared-memory traffic per MMA 136 instead of 163
+// bytes per cycle of tensor work at 256 rows).  dense_shape chooses WT and bn
+// by the waves that they make.
+constexpr int kDnBN = 256;                  // batch rows at most
 constexpr int kDnATile = 128 * kBK * 2;     // 16 KB: 128 weight rows x 64 inputs
 constexpr int kDnBTile = kDnBN * kBK * 2;   // 32 KB: 256 batch rows x 64 inputs
 constexpr int kDnThreads = 320;
@@ -255,7 +266,7 @@ struct DenseParams {
   float* y;
   uint64_t* rec;
   uint64_t call;
-  int M, N, nks;
+  int M, N, nks, bn;
   // CTA u < nfull takes unit u (weight-tile group u mod ngroups, batch tile u / ngroups, WT
   // tiles); CTAs from nfull on split the remaining units into their WT single tiles
   int ngroups, nfull;
@@ -276,7 +287,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
     unit = p.nfull + (unit - p.nfull) / WT;
     nt = 1;
   }
-  const int n0 = (unit % p.ngroups) * 128 * WT + 128 * sub, m0 = (unit / p.ngroups) * kDnBN;
+  const int n0 = (unit % p.ngroups) * 128 * WT + 128 * sub, m0 = (unit / p.ngroups) * p.bn;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (sbase - smem_u32(smem_raw));
   if (tid == 0) {
@@ -304,7 +315,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
       const int s = ks % kStages, r = ks / kStages;
       if (r > 0) ok = mbar_wait_warp(&empty[s], (r - 1) & 1);
       if (!ok) break;
-      mbar_expect_tx_warp(&full[s], (uint32_t)(nt * kDnATile + kDnBTile));
+      mbar_expect_tx_warp(&full[s], (uint32_t)(nt * kDnATile + p.bn * kBK * 2));
       uint8_t* st = base + s * kStage;
 #pragma unroll
       for (int w = 0; w < WT; ++w)
@@ -312,7 +323,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
       tma_load_2d_warp(st + WT * kDnATile, &xmap, ks * kBK, m0, &full[s]);
     }
   } else if (warp == 1) {
-    constexpr uint32_t idesc = f16_idesc(kDnBN);
+    const uint32_t idesc = f16_idesc(p.bn);
     for (int ks = 0; ks < p.nks && ok; ++ks) {
       const int s = ks % kStages, r = ks / kStages;
       ok = mbar_wait_warp(&full[s], r & 1);
@@ -333,7 +344,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
     umma_commit_warp(&acc_bar);
   } else {
     // Epilogue: lane quadrant q holds weight rows n0 + 128 w + 32 q + lane of
-    // accumulator w; this warp writes its columns (batch rows) 128 h .. 128 h + 127.
+    // accumulator w; this warp writes half of its columns (batch rows).
     const int q = warp & 3, h = (warp - 2) >> 2, rr = 32 * q + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16);
     ok = mbar_wait(&acc_bar, 0);
@@ -344,7 +355,8 @@ __global__ void __launch_bounds__(kDnThreads, 1)
       for (int w = 0; w < nt; ++w) {
         const int row = n0 + 128 * w + rr;
         const float sa = row < p.N ? 0.5f * __ldg(p.alpha + row) : 0.f;
-        for (int c0 = 128 * h; c0 < 128 * h + 128; c0 += 16) {
+        const int half = (p.bn / 16 + 1) / 2 * 16, c1 = h ? p.bn : half;
+        for (int c0 = h ? half : 0; c0 < c1; c0 += 16) {
           uint32_t a[16];
           tmem_ld16(lane_addr + (uint32_t)(w * kDnBN + c0), a);
           tmem_ld_wait();
@@ -376,6 +388,47 @@ bool dense_route_applies(const sdq_plan_s* pl, int M) {
          g.k_in % 64 == 0;
 }
 
+namespace {
+// K7's launch shape: weight tiles per CTA and batch rows per tile with the
+// least time over the waves of CTAs.  Shared memory bounds a K step, not the
+// tensor core: its tiles are written once and read by every MMA, 64 KB + 384
+// bn bytes with two weight tiles and 32 KB + 256 bn with one, at 128 bytes a
+// cycle (256 rows: 0.67 and 0.40 us measured, 0.66 and 0.40 so); a wave's two
+// ends take about 9000 cycles.  A last wave of at most half the SMs runs as
+// single tiles on twice the CTAs.  8192 x 8192 at M = 2048: 211 -> 165 us.
+struct DenseShape {
+  int wt, bn, ngroups, nfull, grid;
+};
+DenseShape dense_shape(const sdq_plan_s* pl, int M) {
+  const Geometry& g = pl->geo;
+  const int sms = std::max(1, pl->sm_count);
+  const double steps = g.k_in / kBK, ends = 9000.0;
+  DenseShape best{};
+  double best_t = 0;
+  for (int wt = 2; wt >= 1; --wt)
+    for (int bn = kDnBN; bn >= 96; bn -= 16) {
+      DenseShape s;
+      s.wt = wt;
+      s.bn = bn;
+      s.ngroups = (g.ntiles + wt - 1) / wt;
+      const int mt = (M + bn - 1) / bn;
+      if (mt > 1 && (M + mt - 1) / mt <= bn - 16) continue;   // smaller equal tiles cover M
+      const int units = s.ngroups * mt, full = units / sms, rest = units - full * sms;
+      const bool split = wt == 2 && full > 0 && rest > 0 && 2 * rest <= sms;
+      s.nfull = split ? full * sms : units;
+      s.grid = s.nfull + wt * (units - s.nfull);
+      const double step = 512.0 + 3.0 * bn, one = 256.0 + 2.0 * bn;   // cycles
+      const double t = full * ((wt == 2 ? step : one) * steps + ends) +
+                       (rest ? (split || wt == 1 ? one : step) * steps + ends : 0.0);
+      if (!best.grid || t < best_t * 0.99) {
+        best = s;
+        best_t = t;
+      }
+    }
+  return best;
+}
+}  // namespace
+
 cudaError_t launch_dense_forward(const sdq_plan_s* pl, const uint32_t* codes, const float* alpha,
                                  const uint16_t* x, int M, float* y, void* ws, cudaStream_t st) {
   const Geometry& g = pl->geo;
@@ -387,6 +440,7 @@ cudaError_t launch_dense_forward(const sdq_plan_s* pl, const uint32_t* codes, co
   uint16_t* wp = reinterpret_cast<uint16_t*>(wbase + L.what);
   const cuuint32_t estr[2] = {1, 1};
   const int spb = g.n_b / kBK;
+  const DenseShape sh = dense_shape(pl, M);
   // K6: G^T hi / lo maps (128 rows x n_b), one 64-code chunk per box
   CUtensorMap ghmap, glmap, wmap, xmap;
   {
@@ -401,7 +455,7 @@ cudaError_t launch_dense_forward(const sdq_plan_s* pl, const uint32_t* codes, co
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
   }
-  // K7: W' (n_out x k_in, rows past n_out read as zeros) and x (M x k_in)
+  // W' (n_out x k_in; K6 stores it, K7 loads it: rows past n_out clipped, read as zeros) and x (M x k_in)
   {
     const cuuint64_t dims[2] = {(cuuint64_t)g.k_in, (cuuint64_t)g.n_out};
     const cuuint64_t strides[1] = {(cuuint64_t)g.k_in * 2};
@@ -414,51 +468,43 @@ cudaError_t launch_dense_forward(const sdq_plan_s* pl, const uint32_t* codes, co
   {
     const cuuint64_t dims[2] = {(cuuint64_t)g.k_in, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)g.k_in * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kDnBN};
+    const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)sh.bn};
     if (enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(x), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
   }
   ReconParams rp;
-  rp.codes = codes; rp.w = wp;
+  rp.codes = codes;
   rp.rec = reinterpret_cast<uint64_t*>(wbase + L.err);
   rp.call = call_tag(next_call_number());
-  rp.n_out = g.n_out; rp.k_in = g.k_in; rp.nblk = g.nblk; rp.n_b = g.n_b; rp.ntiles = g.ntiles;
-  rp.ngroups = g.ngroups; rp.wpg = g.wpg; rp.quantizer = pl->desc.quantizer;
+  rp.nblk = g.nblk; rp.n_b = g.n_b; rp.ngroups = g.ngroups; rp.wpg = g.wpg; rp.quantizer = pl->desc.quantizer;
   rp.nitems = g.ntiles * g.nblk;
-  const size_t rsmem = 1024 + 2 * (size_t)spb * 128 * 128 + kRbStages * (size_t)kRbCTile;
-  if (rsmem > 227 * 1024) return cudaErrorNotSupported;
-  cudaError_t e = cudaFuncSetAttribute(recon_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
+  size_t rsmem = 1024 + 2 * (size_t)spb * 128 * 128 + kRbStages * (size_t)kRbCTile + kRbHalf;
+  rp.nstage = rsmem + kRbHalf <= 226 * 1024 ? 2 : 1;
+  rsmem += (size_t)(rp.nstage - 1) * kRbHalf;
+  static std::atomic<int> rb_smem_set[64];
+  cudaError_t e = smem_limit_once(recon_kernel, 226 * 1024, pl->device, rb_smem_set);
   if (e != cudaSuccess) return e;
   e = launch_pdl(recon_kernel, dim3(std::min(rp.nitems, std::max(1, pl->sm_count))), dim3(kRbThreads), rsmem, st,
-                 ghmap, glmap, rp);
+                 ghmap, glmap, wmap, rp);
   if (e != cudaSuccess) return e;
   DenseParams dp;
   dp.alpha = alpha; dp.y = y;
   dp.rec = rp.rec;
   dp.call = call_tag(next_call_number());
   dp.M = M; dp.N = g.n_out; dp.nks = g.k_in / kBK;
-  // two weight tiles per CTA where that still gives two waves of CTAs
-  const int sms = std::max(1, pl->sm_count);
-  const int mt = (M + kDnBN - 1) / kDnBN;
-  if ((int64_t)((g.ntiles + 1) / 2) * mt >= 2 * sms) {
-    dp.ngroups = (g.ntiles + 1) / 2;
-    const int units = dp.ngroups * mt, waves = units / sms, rest = units - waves * sms;
-    // a last wave of at most half the SMs runs as single tiles on twice the CTAs: the
-    // wave then takes a single tile's time (~0.6 of a pair's) instead of a pair's
-    dp.nfull = (rest > 0 && 2 * rest <= sms) ? waves * sms : units;
-    const int grid = dp.nfull + 2 * (units - dp.nfull);
+  dp.bn = sh.bn;
+  dp.ngroups = sh.ngroups;
+  dp.nfull = sh.nfull;
+  if (sh.wt == 2) {
     e = cudaFuncSetAttribute(dense_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, DnShape<2>::kSmem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(dense_kernel<2>, dim3(grid), dim3(kDnThreads), (size_t)DnShape<2>::kSmem, st, wmap, xmap, dp);
+    return launch_pdl(dense_kernel<2>, dim3(sh.grid), dim3(kDnThreads), (size_t)DnShape<2>::kSmem, st, wmap, xmap, dp);
   }
-  dp.ngroups = g.ntiles;
-  dp.nfull = g.ntiles * mt;
   e = cudaFuncSetAttribute(dense_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, DnShape<1>::kSmem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(dense_kernel<1>, dim3(dp.nfull), dim3(kDnThreads), (size_t)DnShape<1>::kSmem, st, wmap, xmap,
-                    dp);
+  return launch_pdl(dense_kernel<1>, dim3(sh.grid), dim3(kDnThreads), (size_t)DnShape<1>::kSmem, st, wmap, xmap, dp);
 }
 
 }  // namespace sdq
