@@ -369,6 +369,54 @@ __device__ __forceinline__ void bulk_g2s_hint_warp(void* dst, const void* src, u
                "l"(policy) : "memory");
 }
 
+// The cluster's barrier (all threads of all its CTAs), and this CTA's rank.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+  return r;
+}
+// Address of the same shared-memory location in the cluster's CTA `rank`.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+  return r;
+}
+
+// CTA pairs (cta_group::2, ranks 0 and 1 of a cluster of two): one MMA of M =
+// 256 over both, each CTA holding its 128 rows of A, its half of B's rows and
+// its 128 rows of D; issued by rank 0.  Allocation and release by a warp of
+// each.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n"
+               "tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::"r"(smem_u32(dst)),
+               "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void umma_bf16_pair_warp(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                                    uint32_t accumulate) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n" SDQ_ELECT
+               "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n}\n" ::"r"(d_tmem),
+               "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// Arrives on `bar` of both CTAs once the pair's MMAs so far are done.
+__device__ __forceinline__ void umma_commit_pair_warp(uint64_t* bar) {
+  asm volatile(SDQ_ELECT "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+               " [%0], %1;\n}\n" ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
+// TMA load into this CTA's shared memory whose bytes count on a barrier of
+// either CTA of the pair (`bar`: cluster address).
+__device__ __forceinline__ void tma_load_2d_pair_warp(void* dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
+  asm volatile(SDQ_ELECT
+               "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+               " [%0], [%1, {%2, %3}], [%4];\n}\n" ::"r"(smem_u32(dst)),
+               "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar) : "memory");
+}
+
 // TMA store of a shared-memory tile (one thread; its groups complete in
 // order): the tile may be rewritten after bulk_store_wait_read (at most N
 // stores still reading), and is in memory after bulk_store_wait_all.

@@ -22,9 +22,9 @@
 //   warp 1     8 MMAs per 64 codes (4 K steps x hi / lo)
 //   warps 2-9  two expander sets (stages of one parity each)
 //   warps 10-13 epilogue
-// K7: a plain tcgen05 GEMM, D[r, m] = W' x^T per CTA tile of 128 (or 2 x 128)
-// weight rows x 256 batch rows, both operands TMA-loaded (128-byte swizzle),
-// 4 (3) stages; epilogue as K5's.
+// K7: a plain tcgen05 GEMM on CTA pairs, D[r, m] = W' x^T per pair tile of 256
+// (or 2 x 256) weight rows x up to 256 batch rows, both operands TMA-loaded
+// (128-byte swizzle), 6 (4) stages; epilogue as K5's.
 // Every wait on an mbarrier is bounded (about 2 s); a timeout writes the call
 // number into the workspace's call record and the CTA finishes without
 // further waits.
@@ -245,17 +245,21 @@ __global__ void __launch_bounds__(kRbThreads, 1)
 }
 
 // ------------------------------------------------------------ K7 dense GEMM
-// WT = 1 or 2 weight tiles of 128 rows per CTA against one tile of `bn` batch
-// rows (a multiple of 16 up to 256): with two, the x tile in shared memory
-// serves two MMAs per K step (shared-memory traffic per MMA 136 instead of 163
-// bytes per cycle of tensor work at 256 rows).  dense_shape chooses WT and bn
-// by the waves that they make.
+// A pair of CTAs (cta_group::2) takes WT = 1 or 2 weight tiles of 256 rows (128
+// of each in either CTA) against one tile of `bn` batch rows (a multiple of 32
+// up to 256, half of them in either CTA's shared memory).  Each CTA loads its
+// rows and signals rank 0's barriers; rank 0 issues the pair's MMAs and
+// commits to both CTAs' barriers.  On single CTAs every MMA read all 256 batch
+// rows from its own shared memory, and that memory, at 128 bytes a cycle,
+// bound the steps: 160 KB per K step of two 128-row tiles against 1024 cycles
+// of tensor work, 0.67 us; a pair reads half of that from each.  8192 x 8192 at
+// M = 4096: 325 -> 301 us (1.83 PFLOP/s).
 constexpr int kDnBN = 256;                  // batch rows at most
 constexpr int kDnATile = 128 * kBK * 2;     // 16 KB: 128 weight rows x 64 inputs
-constexpr int kDnBTile = kDnBN * kBK * 2;   // 32 KB: 256 batch rows x 64 inputs
+constexpr int kDnBTile = kDnBN / 2 * kBK * 2;   // 16 KB: a CTA's half of the batch rows x 64 inputs
 constexpr int kDnThreads = 320;
 template <int WT> struct DnShape {
-  static constexpr int kStages = WT == 1 ? 4 : 3;
+  static constexpr int kStages = WT == 1 ? 6 : 4;
   static constexpr int kStage = WT * kDnATile + kDnBTile;
   static constexpr int kSmem = kStages * kStage + 1024;
   static constexpr uint32_t kCols = WT == 1 ? 256u : 512u;
@@ -267,13 +271,13 @@ struct DenseParams {
   uint64_t* rec;
   uint64_t call;
   int M, N, nks, bn;
-  // CTA u < nfull takes unit u (weight-tile group u mod ngroups, batch tile u / ngroups, WT
-  // tiles); CTAs from nfull on split the remaining units into their WT single tiles
+  // Pair u < nfull takes unit u (weight-tile group u mod ngroups, batch tile u / ngroups, WT
+  // tiles); pairs from nfull on split the remaining units into their WT single tiles
   int ngroups, nfull;
 };
 
 template <int WT>
-__global__ void __launch_bounds__(kDnThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kDnThreads, 1)
     dense_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap,
                  DenseParams p) {
   constexpr int kStages = DnShape<WT>::kStages, kStage = DnShape<WT>::kStage;
@@ -281,13 +285,15 @@ __global__ void __launch_bounds__(kDnThreads, 1)
   __shared__ __align__(8) uint64_t full[kStages], empty[kStages], acc_bar;
   __shared__ uint32_t tmem_base;
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
-  int unit = blockIdx.x, nt = WT, sub = 0;
+  const int rank = (int)cluster_rank();
+  int unit = blockIdx.x >> 1, nt = WT, sub = 0;
   if (unit >= p.nfull) {
     sub = (unit - p.nfull) % WT;
     unit = p.nfull + (unit - p.nfull) / WT;
     nt = 1;
   }
-  const int n0 = (unit % p.ngroups) * 128 * WT + 128 * sub, m0 = (unit / p.ngroups) * p.bn;
+  // this CTA's rows of weight tile w: n0 + 256 w ..; the pair's batch rows m0 ..
+  const int n0 = (unit % p.ngroups) * 256 * WT + 256 * sub + 128 * rank, m0 = (unit / p.ngroups) * p.bn;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (sbase - smem_u32(smem_raw));
   if (tid == 0) {
@@ -298,65 +304,72 @@ __global__ void __launch_bounds__(kDnThreads, 1)
     mbar_init(&acc_bar, 1);
     fence_mbar_init();
   }
-  if (warp == 0) {
-    tmem_alloc(&tmem_base, DnShape<WT>::kCols);
-    tmem_relinquish();
-  }
+  if (warp == 0) tmem_alloc_pair(&tmem_base, DnShape<WT>::kCols);
   tc_fence_before();
-  __syncthreads();
+  cluster_sync();   // both CTAs' barriers and tensor memory are set up
   tc_fence_after();
   pdl_wait();
   pdl_launch_dependents();
-  call_record_start(p.rec, p.call, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0);
+  call_record_start(p.rec, p.call, blockIdx.x == 0 && threadIdx.x == 0);
   const uint32_t tmem = tmem_base;
   bool ok = true;
   if (warp == 0) {
-    for (int ks = 0; ks < p.nks && ok; ++ks) {
+    const uint32_t bytes = (uint32_t)(nt * kDnATile + p.bn * kBK);   // of each CTA
+    int ks = 0;
+    for (; ks < p.nks; ++ks) {
       const int s = ks % kStages, r = ks / kStages;
       if (r > 0) ok = mbar_wait_warp(&empty[s], (r - 1) & 1);
       if (!ok) break;
-      mbar_expect_tx_warp(&full[s], (uint32_t)(nt * kDnATile + p.bn * kBK * 2));
+      if (rank == 0) mbar_expect_tx_warp(&full[s], 2 * bytes);
+      const uint32_t bar = cluster_addr(&full[s], 0);
       uint8_t* st = base + s * kStage;
 #pragma unroll
       for (int w = 0; w < WT; ++w)
-        if (w < nt) tma_load_2d_warp(st + w * kDnATile, &wmap, ks * kBK, n0 + 128 * w, &full[s]);
-      tma_load_2d_warp(st + WT * kDnATile, &xmap, ks * kBK, m0, &full[s]);
+        if (w < nt) tma_load_2d_pair_warp(st + w * kDnATile, &wmap, ks * kBK, n0 + 256 * w, bar);
+      tma_load_2d_pair_warp(st + WT * kDnATile, &xmap, ks * kBK, m0 + rank * (p.bn / 2), bar);
     }
+    // the pair's copies have landed before either CTA ends
+    if (rank == 0)
+      for (int j = max(0, ks - kStages); j < ks; ++j)
+        if (!mbar_wait_warp(&full[j % kStages], (j / kStages) & 1)) ok = false;
   } else if (warp == 1) {
-    const uint32_t idesc = f16_idesc(p.bn);
-    for (int ks = 0; ks < p.nks && ok; ++ks) {
-      const int s = ks % kStages, r = ks / kStages;
-      ok = mbar_wait_warp(&full[s], r & 1);
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t st = sbase + s * kStage;
-      const uint64_t bd = sw128_desc(st + WT * kDnATile);
+    if (rank == 0) {
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.bn >> 3) << 17) |
+                             ((uint32_t)(256 >> 4) << 24);   // D fp32, A and B bf16, both K-major, M = 256
+      const uint64_t d0 = sw128_desc(sbase);
+      for (int ks = 0; ks < p.nks; ++ks) {
+        const int s = ks % kStages, r = ks / kStages;
+        ok = mbar_wait_warp(&full[s], r & 1);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t st = d0 + (uint64_t)(s * (kStage >> 4)), bd = st + (uint64_t)(WT * (kDnATile >> 4));
 #pragma unroll
-      for (int w = 0; w < WT; ++w) {
-        if (w >= nt) break;
-        const uint64_t ad = sw128_desc(st + w * kDnATile);
+        for (int w = 0; w < WT; ++w) {
+          if (w >= nt) break;
+          const uint64_t ad = st + (uint64_t)(w * (kDnATile >> 4));
 #pragma unroll
-        for (int kk = 0; kk < kBK / 16; ++kk)
-          umma_bf16_warp(tmem + (uint32_t)(w * kDnBN), ad + 2 * kk, bd + 2 * kk, idesc, (ks | kk) != 0);
+          for (int kk = 0; kk < kBK / 16; ++kk)
+            umma_bf16_pair_warp(tmem + (uint32_t)(w * kDnBN), ad + 2 * kk, bd + 2 * kk, idesc, (ks | kk) != 0);
+        }
+        umma_commit_pair_warp(&empty[s]);
       }
-      umma_commit_warp(&empty[s]);
+      umma_commit_pair_warp(&acc_bar);
     }
-    umma_commit_warp(&acc_bar);
+    if (!mbar_wait_warp(&acc_bar, 0)) ok = false;   // every MMA of the pair is done
   } else {
-    // Epilogue: lane quadrant q holds weight rows n0 + 128 w + 32 q + lane of
+    // Epilogue: lane quadrant q holds weight rows n0 + 256 w + 32 q + lane of
     // accumulator w; this warp writes half of its columns (batch rows).
     const int q = warp & 3, h = (warp - 2) >> 2, rr = 32 * q + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16);
-    ok = mbar_wait(&acc_bar, 0);
-    ok = __all_sync(0xffffffffu, ok);
+    ok = mbar_wait_warp(&acc_bar, 0);
     tc_fence_after();
     if (ok) {
 #pragma unroll 1
       for (int w = 0; w < nt; ++w) {
-        const int row = n0 + 128 * w + rr;
+        const int row = n0 + 256 * w + rr;
         const float sa = row < p.N ? 0.5f * __ldg(p.alpha + row) : 0.f;
-        const int half = (p.bn / 16 + 1) / 2 * 16, c1 = h ? p.bn : half;
-        for (int c0 = h ? half : 0; c0 < c1; c0 += 16) {
+        const int half = p.bn / 2;
+        for (int c0 = h ? half : 0; c0 < (h ? p.bn : half); c0 += 16) {
           uint32_t a[16];
           tmem_ld16(lane_addr + (uint32_t)(w * kDnBN + c0), a);
           tmem_ld_wait();
@@ -373,10 +386,10 @@ __global__ void __launch_bounds__(kDnThreads, 1)
   }
   if (!ok) call_record_fail(p.rec, p.call);
   tc_fence_before();
-  __syncthreads();
+  cluster_sync();   // both CTAs are done with the pair's tensor memory and barriers
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem, DnShape<WT>::kCols);
+    tmem_dealloc_pair(tmem, DnShape<WT>::kCols);
   }
 }
 
@@ -389,38 +402,37 @@ bool dense_route_applies(const sdq_plan_s* pl, int M) {
 }
 
 namespace {
-// K7's launch shape: weight tiles per CTA and batch rows per tile with the
-// least time over the waves of CTAs.  Shared memory bounds a K step, not the
-// tensor core: its tiles are written once and read by every MMA, 64 KB + 384
-// bn bytes with two weight tiles and 32 KB + 256 bn with one, at 128 bytes a
-// cycle (256 rows: 0.67 and 0.40 us measured, 0.66 and 0.40 so); a wave's two
-// ends take about 9000 cycles.  A last wave of at most half the SMs runs as
-// single tiles on twice the CTAs.  8192 x 8192 at M = 2048: 211 -> 165 us.
+// K7's launch shape: 256-row weight tiles per pair and batch rows per tile
+// with the least time over the waves of pairs.  A K step takes the longer of
+// its MMAs (2 bn cycles a tile) and its shared-memory traffic in each CTA (tiles
+// written once, read by every MMA, at 128 bytes a cycle: 512 + 1.5 bn with
+// two tiles, 256 + bn with one); a wave's two ends take about 9000 cycles.  A
+// last wave of at most half the pairs runs as single tiles on twice as many.
 struct DenseShape {
-  int wt, bn, ngroups, nfull, grid;
+  int wt, bn, ngroups, nfull, pairs;
 };
 DenseShape dense_shape(const sdq_plan_s* pl, int M) {
   const Geometry& g = pl->geo;
-  const int sms = std::max(1, pl->sm_count);
+  const int slots = std::max(1, pl->pf_clusters[2]), tiles = (g.ntiles + 1) / 2;
   const double steps = g.k_in / kBK, ends = 9000.0;
   DenseShape best{};
   double best_t = 0;
   for (int wt = 2; wt >= 1; --wt)
-    for (int bn = kDnBN; bn >= 96; bn -= 16) {
+    for (int bn = kDnBN; bn >= 96; bn -= 32) {
       DenseShape s;
       s.wt = wt;
       s.bn = bn;
-      s.ngroups = (g.ntiles + wt - 1) / wt;
+      s.ngroups = (tiles + wt - 1) / wt;
       const int mt = (M + bn - 1) / bn;
-      if (mt > 1 && (M + mt - 1) / mt <= bn - 16) continue;   // smaller equal tiles cover M
-      const int units = s.ngroups * mt, full = units / sms, rest = units - full * sms;
-      const bool split = wt == 2 && full > 0 && rest > 0 && 2 * rest <= sms;
-      s.nfull = split ? full * sms : units;
-      s.grid = s.nfull + wt * (units - s.nfull);
-      const double step = 512.0 + 3.0 * bn, one = 256.0 + 2.0 * bn;   // cycles
-      const double t = full * ((wt == 2 ? step : one) * steps + ends) +
-                       (rest ? (split || wt == 1 ? one : step) * steps + ends : 0.0);
-      if (!best.grid || t < best_t * 0.99) {
+      if (mt > 1 && (M + mt - 1) / mt <= bn - 32) continue;   // smaller equal tiles cover M
+      const int units = s.ngroups * mt, full = units / slots, rest = units - full * slots;
+      const bool split = wt == 2 && full > 0 && rest > 0 && 2 * rest <= slots;
+      s.nfull = split ? full * slots : units;
+      s.pairs = s.nfull + wt * (units - s.nfull);
+      const double two = std::max(4.0 * bn, 512.0 + 1.5 * bn), one = std::max(2.0 * bn, 256.0 + bn);   // cycles
+      const double t = full * ((wt == 2 ? two : one) * steps + ends) +
+                       (rest ? (split || wt == 1 ? one : two) * steps + ends : 0.0);
+      if (!best.pairs || t < best_t * 0.99) {
         best = s;
         best_t = t;
       }
@@ -468,7 +480,7 @@ cudaError_t launch_dense_forward(const sdq_plan_s* pl, const uint32_t* codes, co
   {
     const cuuint64_t dims[2] = {(cuuint64_t)g.k_in, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)g.k_in * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)sh.bn};
+    const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)(sh.bn / 2)};
     if (enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(x), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -500,11 +512,11 @@ cudaError_t launch_dense_forward(const sdq_plan_s* pl, const uint32_t* codes, co
   if (sh.wt == 2) {
     e = cudaFuncSetAttribute(dense_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, DnShape<2>::kSmem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(dense_kernel<2>, dim3(sh.grid), dim3(kDnThreads), (size_t)DnShape<2>::kSmem, st, wmap, xmap, dp);
+    return launch_pdl(dense_kernel<2>, dim3(2 * sh.pairs), dim3(kDnThreads), (size_t)DnShape<2>::kSmem, st, wmap, xmap, dp);
   }
   e = cudaFuncSetAttribute(dense_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, DnShape<1>::kSmem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(dense_kernel<1>, dim3(sh.grid), dim3(kDnThreads), (size_t)DnShape<1>::kSmem, st, wmap, xmap, dp);
+  return launch_pdl(dense_kernel<1>, dim3(2 * sh.pairs), dim3(kDnThreads), (size_t)DnShape<1>::kSmem, st, wmap, xmap, dp);
 }
 
 }  // namespace sdq

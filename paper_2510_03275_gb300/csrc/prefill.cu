@@ -76,9 +76,6 @@ struct PrefillParams {
   int bn, stages, split, early, add;   // add: y += the result
 };
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
 // 16 bytes of the shared memory of the cluster's CTA `rank`, at this CTA's address `a`.
 __device__ __forceinline__ float4 ld_cluster4(uint32_t a, uint32_t rank) {
   uint32_t r;
