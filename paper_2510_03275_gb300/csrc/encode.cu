@@ -316,7 +316,10 @@ struct TileParams {
   uint32_t pad0;     // first padding word of a row
 };
 
-template <int PT>
+// kTable: half the table in shared memory (np at most 32 PT); else it is read
+// where it is (every warp of the CTA reads the same rows at about the same
+// time: the L1 serves them) and the samples are done 32 PT pairs at a time.
+template <int PT, bool kTable>
 __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel(TileParams p) {
   extern __shared__ __align__(16) float smem[];
   __shared__ uint32_t s_amax[kTMaxTeams][2][kTMaxRows];   // bit patterns of the rows' maxima (non-negative floats)
@@ -326,34 +329,36 @@ __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel
   const int team = warp / p.gw, tw = warp - team * p.gw, nteam = nwarp / p.gw, tt = 32 * tw + lane;
   auto team_sync = [&]() { named_bar_sync(1 + team, 32 * p.gw); };
   const int np = p.n_b / 2, xs_stride = p.n_b + 1;
+  const size_t table = kTable ? (size_t)p.B * np : 0;
   float* ts = smem;                                        // B x np
-  float* wt = ts + (size_t)p.B * np + (size_t)warp * tile_weight_floats(p.B);
-  float* xs0 = ts + (size_t)p.B * np + (size_t)nwarp * tile_weight_floats(p.B) +
+  float* wt = ts + table + (size_t)warp * tile_weight_floats(p.B);
+  float* xs0 = ts + table + (size_t)nwarp * tile_weight_floats(p.B) +
                (size_t)team * p.gw * kTv * xs_stride;   // the team's samples
   float* xs = xs0 + (size_t)tw * kTv * xs_stride;
-  tile_load_table(ts, p.at, p.B, p.n_b);
+  if constexpr (kTable) tile_load_table(ts, p.at, p.B, p.n_b);
   for (int i = threadIdx.x; i < kTMaxTeams * 2 * kTMaxRows; i += blockDim.x) (&s_amax[0][0][0])[i] = 0u;
   __syncthreads();
 
   const int tv = kTv * p.gw, ngroups = (p.n_out + p.rows - 1) / p.rows;
   float acc[kTv][PT], acc2[kTv][PT];
 
-  // x_up of virtual rows v0 .. v0 + 7 of the group at row0 (nv in all) into
-  // acc (samples l + 32 q) and acc2 (the same + n_b / 2)
-  auto compute = [&](int row0, int v0, int nv) {
-    {
-      // the 8 x B weights, transposed to [k][8]: lane = (virtual row, float4)
-      const int v = v0 + (lane >> 2), r = min(v, nv - 1) / p.nblk, b = min(v, nv - 1) - r * p.nblk;
-      const float4* src = reinterpret_cast<const float4*>(p.W + (size_t)(row0 + r) * p.k_in + (size_t)b * p.B);
-      __syncwarp();
-      for (int k4 = lane & 3; k4 < p.B / 4; k4 += 4) {
-        const float4 w = v < nv ? __ldg(src + k4) : make_float4(0.f, 0.f, 0.f, 0.f);
-        float* d = wt + k4 * kWk4 + (lane >> 2);
-        d[0] = w.x; d[8] = w.y; d[16] = w.z; d[24] = w.w;
-      }
-      __syncwarp();
+  // the 8 x B weights of virtual rows v0 .. v0 + 7 of the group at row0 (nv in
+  // all), transposed to [k][8]: lane = (virtual row, float4)
+  auto load_weights = [&](int row0, int v0, int nv) {
+    const int v = v0 + (lane >> 2), r = min(v, nv - 1) / p.nblk, b = min(v, nv - 1) - r * p.nblk;
+    const float4* src = reinterpret_cast<const float4*>(p.W + (size_t)(row0 + r) * p.k_in + (size_t)b * p.B);
+    __syncwarp();
+    for (int k4 = lane & 3; k4 < p.B / 4; k4 += 4) {
+      const float4 w = v < nv ? __ldg(src + k4) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float* d = wt + k4 * kWk4 + (lane >> 2);
+      d[0] = w.x; d[8] = w.y; d[16] = w.z; d[24] = w.w;
     }
-    tile_upsample<PT>(ts + lane, np, np - lane, wt, p.B, acc, acc2);
+    __syncwarp();
+  };
+  // their x_up into acc (samples j0 + l + 32 q) and acc2 (the same + n_b / 2)
+  auto compute = [&](int j0) {
+    if constexpr (kTable) tile_upsample<PT>(ts + lane, np, np - lane, wt, p.B, acc, acc2);
+    else tile_upsample<PT>(p.at + j0 + lane, p.n_b, np - j0 - lane, wt, p.B, acc, acc2);
   };
   // row maxima of the warp's 8 virtual rows (pairs past np hold zeros)
   auto maxima = [&](int v0, int nv, uint32_t* am) {
@@ -367,15 +372,17 @@ __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel
       if (lane == 0 && v0 + v < nv) atomicMax(&am[(v0 + v) / p.nblk], __float_as_uint(m));
     }
   };
-  auto store = [&]() {
+  auto store = [&](int j0) {
 #pragma unroll
     for (int v = 0; v < kTv; ++v)
 #pragma unroll
-      for (int q = 0; q < PT; ++q)
-        if (lane + 32 * q < np) {
-          xs[v * xs_stride + lane + 32 * q] = acc[v][q];
-          xs[v * xs_stride + np + lane + 32 * q] = acc2[v][q];
+      for (int q = 0; q < PT; ++q) {
+        const int j = j0 + lane + 32 * q;
+        if (j < np) {
+          xs[v * xs_stride + j] = acc[v][q];
+          xs[v * xs_stride + np + j] = acc2[v][q];
         }
+      }
   };
   // Eq. (8) over virtual row `lv` of the tile: i = (i + x) - y_prev from 0,
   // the codes packed into whole words.
@@ -414,14 +421,21 @@ __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel
     const int steps = n0 + (p.only_alpha ? 0 : tiles);
     for (int step = 0; step < steps; ++step) {
       const int t = step < n0 ? step : step - n0, v0 = t * tv + tw * kTv;
-      if (v0 < nv) {
-        compute(row0, v0, nv);
-        if (step < n0 || single) maxima(v0, nv, am);
+      const bool pass0 = step < n0;
+      if (v0 < nv) load_weights(row0, v0, nv);
+      for (int j0 = 0; j0 < np; j0 += 32 * PT) {
+        if (v0 < nv) {
+          compute(j0);
+          if (pass0 || single) maxima(v0, nv, am);
+        }
+        if (pass0) continue;
+        if (j0 == 0) {
+          team_sync();   // the tile before is scanned
+          if (t == 0 && tt < kTMaxRows) am_next[tt] = 0u;
+        }
+        if (v0 < nv) store(j0);
       }
-      if (step < n0) continue;
-      team_sync();   // the tile before is scanned; the maxima are in
-      if (t == 0 && tt < kTMaxRows) am_next[tt] = 0u;
-      if (v0 < nv) store();
+      if (pass0) continue;
       team_sync();
       // 32 virtual rows per scanning warp
       const int part = (tw - turn + p.gw) % p.gw;
@@ -446,10 +460,13 @@ __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel
 }
 
 // Warps, warps per team and rows per group of the tile encoder, 0 warps where
-// it does not apply: the half-shift table, whole words of codes per block, at
-// most 192 pairs, and half the table in shared memory beside at least 4 warps'
-// buffers (n_b / 2 x B words; 10 B + 8 (n_b + 1) words a warp).
+// it does not apply: the half-shift table, whole words of codes per block, and
+// at least 2 warps' buffers (10 B + 8 (n_b + 1) words each) in shared memory;
+// half the table (n_b / 2 x B words) joins them where it has at most 192
+// pairs and leaves room for 4 warps, else it is read from global memory (B =
+// 256 and 512 at OSR 2: 6x and 4x the row encoder).
 struct TileShape {
+  bool table;
   int warps, gw, rows, pt;
   size_t smem;
 };
@@ -457,12 +474,16 @@ TileShape tile_shape(const sdq_plan_s* pl, bool given) {
   const Geometry& g = pl->geo;
   TileShape t{};
   const int np = g.n_b / 2;
-  if (!pl->half_shift || g.block < 16 || np > 192 || (g.n_b * g.bits) % 32) return t;
-  const size_t table = sizeof(float) * (size_t)g.block * np;
+  if (!pl->half_shift || g.block < 16 || (g.n_b * g.bits) % 32) return t;
+  size_t table = sizeof(float) * (size_t)g.block * np;
   const size_t per_warp = sizeof(float) * ((size_t)tile_weight_floats(g.block) + (size_t)kTv * (g.n_b + 1));
   const size_t room = 226 * 1024;
-  if (table + 4 * per_warp > room) return t;
-  t.pt = (np + 31) / 32;
+  t.table = np <= 192 && table + 4 * per_warp <= room;
+  if (!t.table) {
+    table = 0;
+    if (2 * per_warp > room) return t;
+  }
+  t.pt = t.table ? (np + 31) / 32 : 4;
   const int most = (int)std::min<size_t>(tile_max_warps(t.pt), (room - table) / per_warp);
   const int64_t sms = std::max(1, pl->sm_count);
   // Teams of 4 warps or of all (most of them in whole teams), and the row
@@ -473,6 +494,7 @@ TileShape tile_shape(const sdq_plan_s* pl, bool given) {
   double best = 0;
   const int widths[2] = {4, most & ~1};
   for (int gw : widths) {
+    if (gw > most) continue;
     const int nteam = most / gw, tv = kTv * gw;
     for (int r = 1; r <= kTMaxRows; ++r) {
       const int64_t groups = (g.n_out + r - 1) / r;
@@ -503,8 +525,10 @@ cudaError_t launch_encode_tile(const sdq_plan_s* pl, const TileShape& t, const f
   p.wpr = g.words_per_row; p.quantizer = pl->desc.quantizer; p.rows = t.rows;
   p.given = given; p.only_alpha = only_alpha; p.gw = t.gw;
   p.pad0 = (uint32_t)(g.k_eff * g.bits / 32);
-  auto kern = t.pt <= 1 ? encode_tile_kernel<1> : t.pt == 2 ? encode_tile_kernel<2> : t.pt == 3 ? encode_tile_kernel<3>
-            : t.pt == 4 ? encode_tile_kernel<4> : t.pt == 5 ? encode_tile_kernel<5> : encode_tile_kernel<6>;
+  auto kern = !t.table ? encode_tile_kernel<4, false>
+              : t.pt <= 1 ? encode_tile_kernel<1, true> : t.pt == 2 ? encode_tile_kernel<2, true>
+              : t.pt == 3 ? encode_tile_kernel<3, true> : t.pt == 4 ? encode_tile_kernel<4, true>
+              : t.pt == 5 ? encode_tile_kernel<5, true> : encode_tile_kernel<6, true>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
   if (e != cudaSuccess) return e;
   const int groups = (g.n_out + t.rows - 1) / t.rows;

@@ -17,11 +17,11 @@ __host__ __device__ constexpr int tile_weight_floats(int B) { return B / 4 * kWk
 // x_up of the 8 virtual rows whose weights are in `wt`, pairs (j, j + np) for
 // j = lane's first pair + 32 q, q < PT (pairs past `left` of them give
 // zeros): acc gets sample j, acc2 sample j + np.  `tp` points at the lane's
-// first pair in row 0 of the table's first half (B x np).  Canonical order: k
-// ascending, every product and every sum rounded, the first product taken as
+// first pair in row 0 of the table's first half (B rows, `ld` apart; shared
+// or global memory).  Canonical order: k ascending, every product and every sum rounded, the first product taken as
 // is; acc2 subtracts the products of k >= B / 2 that acc adds.
 template <int PT>
-__device__ __forceinline__ void tile_upsample(const float* tp, int np, int left, const float* wt, int B,
+__device__ __forceinline__ void tile_upsample(const float* tp, int ld, int left, const float* wt, int B,
                                               float (&acc)[kTv][PT], float (&acc2)[kTv][PT]) {
   const int half = B / 2;
   bool in[PT];
@@ -35,7 +35,7 @@ __device__ __forceinline__ void tile_upsample(const float* tp, int np, int left,
   };
   auto table = [&](int k, float (&a)[PT]) {
 #pragma unroll
-    for (int q = 0; q < PT; ++q) a[q] = in[q] ? tp[k * np + 32 * q] : 0.f;
+    for (int q = 0; q < PT; ++q) a[q] = in[q] ? tp[(size_t)k * ld + 32 * q] : 0.f;
   };
   {
     float w[kTv], a[PT];

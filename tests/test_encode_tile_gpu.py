@@ -2,7 +2,8 @@
 alpha bit-exact with the oracle's canonical fp32 encoder.
 
 The tile encoder takes blocks of at least 16 inputs whose codes fill whole
-32-bit words, up to 192 sample pairs; the others stay with the row encoder.
+32-bit words, with half its table in shared memory (up to 192 sample pairs) or
+read from global memory; the others stay with the row encoder.
 Both sides of each line, one computation of the samples for alpha and scan
 (the group's blocks fit in one tile) and two (more blocks than virtual rows
 in a tile), rows that do not fill the last group, every pair count per lane
@@ -20,7 +21,7 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(5, 32, 16, 2), (9, 48, 16, 1), (33, 192, 64, 1), (7, 320, 64, Fraction(3, 2)), (161, 128, 64, 3),
           (3, 8192, 64, 2), (2, 20480, 128, 1), (17, 384, 128, Fraction(3, 2)), (700, 256, 128, 2),
           (1, 18560, 128, 2), (6, 896, 128, Fraction(5, 2)), (5, 640, 128, 3), (4, 256, 128, Fraction(7, 2)),
-          (6, 384, 128, Fraction(9, 8)), (3, 512, 256, Fraction(3, 2)), (6, 64, 8, 2), (5, 640, 64, 5)]
+          (6, 384, 128, Fraction(9, 8)), (3, 512, 256, Fraction(3, 2)), (35, 768, 256, 2), (3, 2048, 256, 3), (5, 1024, 512, 2), (20, 1536, 512, Fraction(5, 2)), (2, 512, 512, 3), (3, 1024, 1024, 2), (6, 64, 8, 2), (5, 640, 64, 5)]
 
 
 @pytest.mark.parametrize("q", [O.TERNARY, O.BINARY])
