@@ -3,7 +3,7 @@
 //
 // Two kernels, the same codes bit for bit.  encode_tile_kernel (second half of
 // this file) takes the layers whose tables and sizes allow it; the row
-// encoder takes the others, alpha as a mean, and the GPTQ blocks.
+// encoder takes the others.
 //
 // The row encoder: one warp owns 4 output rows.  For every block of B input columns it
 // rebuilds the upsampled block x_up = A_enc w (A_enc = U Had^T, the
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) encode_kernel(EncodeParams p) 
 
 // ------------------------------------------------------------ tile encoder
 // The encoder for layers whose table has the half-shift symmetry (below) and
-// whose codes of a block fill whole words, MAXABS alpha (or alpha given).
+// whose codes of a block fill whole words.
 //
 // A_enc row j + n_b / 2 is row j shifted by half a block, and a shift by B / 2
 // of an index below B flips its top bit: in the Hadamard domain
@@ -297,7 +297,10 @@ __global__ void __launch_bounds__(32 * kMaxWarps) encode_kernel(EncodeParams p) 
 // computation of x_up, else pass 0 takes the maxima and pass 1 recomputes.
 // The scan (eq. 8) of a tile runs with one lane per virtual row, 32 to a
 // warp, beside the other warps' next tile: blocks are independent, so 32
-// lanes of a warp scan where 4 did with a lane per row.
+// lanes of a warp scan where 4 did with a lane per row.  Alpha as a mean is one
+// chain of rounded sums per row: lane r of the team's first warp adds row r's
+// samples, beside the other teams' products (4096 x 4096, B = 128, OSR 2: 3.18
+// ms with the row encoder, 1.27 with its pass 0 alone, 0.59 so).
 // 11008 x 4096, OSR 2 (46 G rounded operations as two plain passes, 14 G so):
 // 6.24 ms with the row encoder, 0.71 ms (0.95 with one
 // team per CTA, whose barriers had the other warps wait for the scan).
@@ -311,7 +314,8 @@ struct TileParams {
   uint32_t* codes;
   float* alpha;
   const float* at;   // B x n_b
-  int n_out, k_in, B, n_b, nblk, wpr, quantizer, rows, given, only_alpha;
+  int n_out, k_in, B, n_b, nblk, wpr, quantizer, rows, mean, only_alpha;
+  float k_eff;
   int gw;            // warps of a team
   uint32_t pad0;     // first padding word of a row
 };
@@ -416,34 +420,54 @@ __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel
     const int row0 = g * p.rows, nv = min(p.rows, p.n_out - row0) * p.nblk;
     const int tiles = (nv + tv - 1) / tv;
     uint32_t *am = s_amax[team][buf], *am_next = s_amax[team][buf ^ 1];
-    const bool single = tiles == 1 && !p.given && !p.only_alpha;   // one computation for alpha and the scan
-    const int n0 = p.given || single ? 0 : tiles;                  // steps of pass 0
+    const bool single = tiles == 1 && !p.only_alpha;   // one computation for alpha and the scan
+    const int n0 = single ? 0 : tiles;                 // steps of pass 0
     const int steps = n0 + (p.only_alpha ? 0 : tiles);
+    float mean_acc = 0.f;   // MEANABS: lane r of the team's first warp adds row r's samples
+    bool mean_first = true;
     for (int step = 0; step < steps; ++step) {
       const int t = step < n0 ? step : step - n0, v0 = t * tv + tw * kTv;
-      const bool pass0 = step < n0;
+      const bool pass0 = step < n0, samples = !pass0 || p.mean;
       if (v0 < nv) load_weights(row0, v0, nv);
       for (int j0 = 0; j0 < np; j0 += 32 * PT) {
         if (v0 < nv) {
           compute(j0);
-          if (pass0 || single) maxima(v0, nv, am);
+          if (!p.mean && (pass0 || single)) maxima(v0, nv, am);
         }
-        if (pass0) continue;
+        if (!samples) continue;
         if (j0 == 0) {
-          team_sync();   // the tile before is scanned
-          if (t == 0 && tt < kTMaxRows) am_next[tt] = 0u;
+          team_sync();   // the tile before is scanned (summed)
+          if (!pass0 && t == 0 && tt < kTMaxRows) am_next[tt] = 0u;
         }
         if (v0 < nv) store(j0);
       }
-      if (pass0) continue;
+      if (!samples) continue;
       team_sync();
+      if (p.mean && (pass0 || single)) {
+        // the canonical mean: one rounded sum in (block, index) order per row
+        if (tw == 0 && lane * p.nblk < nv) {
+          const int vb = min((lane + 1) * p.nblk, min((t + 1) * tv, nv));
+          for (int v = max(lane * p.nblk, t * tv); v < vb; ++v) {
+            const float* x = xs0 + (size_t)(v - t * tv) * xs_stride;
+#pragma unroll 16
+            for (int j = 0; j < p.n_b; ++j) {
+              const float a = fabsf(x[j]);
+              mean_acc = mean_first ? a : __fadd_rn(mean_acc, a);
+              mean_first = false;
+            }
+          }
+          if (t == tiles - 1) am[lane] = __float_as_uint(__fdiv_rn(mean_acc, p.k_eff));
+        }
+        if (single) team_sync();
+      }
+      if (pass0) continue;
       // 32 virtual rows per scanning warp
       const int part = (tw - turn + p.gw) % p.gw;
       const int lv = 32 * part + lane, v = t * tv + lv;
       if (lv < tv && v < nv) {
         const int r = v / p.nblk, b = v - r * p.nblk, row = row0 + r;
-        const float a = p.given ? p.alpha[row] : __uint_as_float(am[r]);
-        if (!p.given && b == 0) p.alpha[row] = a;
+        const float a = __uint_as_float(am[r]);
+        if (b == 0) p.alpha[row] = a;
         scan(row, b, lv, a);
       }
       turn = (turn + (tv + 31) / 32) % p.gw;
@@ -463,14 +487,14 @@ __global__ void __launch_bounds__(32 * tile_max_warps(PT), 1) encode_tile_kernel
 // it does not apply: the half-shift table, whole words of codes per block, and
 // at least 2 warps' buffers (10 B + 8 (n_b + 1) words each) in shared memory;
 // half the table (n_b / 2 x B words) joins them where it has at most 192
-// pairs and leaves room for 4 warps, else it is read from global memory (B =
-// 256 and 512 at OSR 2: 6x and 4x the row encoder).
+// pairs and leaves room for 4 warps, else it is read from global memory (4096 x
+// 4096, OSR 2, B = 256 and 512: 0.64 and 1.6 ms, the row encoder 9.0 and 14.4).
 struct TileShape {
   bool table;
   int warps, gw, rows, pt;
   size_t smem;
 };
-TileShape tile_shape(const sdq_plan_s* pl, bool given) {
+TileShape tile_shape(const sdq_plan_s* pl) {
   const Geometry& g = pl->geo;
   TileShape t{};
   const int np = g.n_b / 2;
@@ -486,6 +510,7 @@ TileShape tile_shape(const sdq_plan_s* pl, bool given) {
   t.pt = t.table ? (np + 31) / 32 : 4;
   const int most = (int)std::min<size_t>(tile_max_warps(t.pt), (room - table) / per_warp);
   const int64_t sms = std::max(1, pl->sm_count);
+  const bool mean = pl->desc.alpha_mode == SDQ_ALPHA_MEANABS;
   // Teams of 4 warps or of all (most of them in whole teams), and the row
   // count whose groups take the least time on the busiest SM: a tile's
   // products on the warps that have virtual rows in it, twice where alpha
@@ -502,8 +527,11 @@ TileShape tile_shape(const sdq_plan_s* pl, bool given) {
       const int64_t tiles = ((int64_t)r * g.nblk + tv - 1) / tv;
       const double live = tiles == 1 ? (double)((r * g.nblk + kTv - 1) / kTv) : (double)gw;   // warps at work
       // the SM's issue slots shared by its teams' warps, at least one warp per quadrant's own pace
-      const double products = tiles * std::max(live * nteam / 12.0, 0.35) * (given || tiles == 1 ? 1.0 : 2.0);
-      const double c = (double)turns * (products + (nteam > 1 ? 0.08 : 0.3) * tiles);
+      const double products = tiles * std::max(live * nteam / 12.0, 0.35) * (tiles == 1 ? 1.0 : 2.0);
+      // MEANABS: a row's sum is one chain of about 5 cycles a sample
+      const double chain = mean ? 5.0 * (double)g.k_eff / (1.9 * np * g.block) : 0.0;
+      const double c = (double)turns * std::max(products + (nteam > 1 ? 0.08 : 0.3) * tiles,
+                                                products / nteam + chain + 0.2 * tiles);
       if (!t.warps || c < best * 0.999) {
         best = c;
         t.warps = gw * nteam;
@@ -517,13 +545,14 @@ TileShape tile_shape(const sdq_plan_s* pl, bool given) {
 }
 
 cudaError_t launch_encode_tile(const sdq_plan_s* pl, const TileShape& t, const float* W, uint32_t* codes, float* alpha,
-                               cudaStream_t st, bool given, bool only_alpha) {
+                               cudaStream_t st, bool only_alpha) {
   const Geometry& g = pl->geo;
   TileParams p;
   p.W = W; p.codes = codes; p.alpha = alpha; p.at = pl->d_at;
   p.n_out = g.n_out; p.k_in = g.k_in; p.B = g.block; p.n_b = g.n_b; p.nblk = g.nblk;
   p.wpr = g.words_per_row; p.quantizer = pl->desc.quantizer; p.rows = t.rows;
-  p.given = given; p.only_alpha = only_alpha; p.gw = t.gw;
+  p.mean = pl->desc.alpha_mode == SDQ_ALPHA_MEANABS; p.only_alpha = only_alpha; p.gw = t.gw;
+  p.k_eff = (float)g.k_eff;
   p.pad0 = (uint32_t)(g.k_eff * g.bits / 32);
   auto kern = !t.table ? encode_tile_kernel<4, false>
               : t.pt <= 1 ? encode_tile_kernel<1, true> : t.pt == 2 ? encode_tile_kernel<2, true>
@@ -540,21 +569,15 @@ cudaError_t launch_encode_tile(const sdq_plan_s* pl, const TileShape& t, const f
 
 cudaError_t launch_encode(const sdq_plan_s* pl, const float* W, uint32_t* codes, float* alpha,
                           cudaStream_t st) {
-  const bool mean = pl->desc.alpha_mode == SDQ_ALPHA_MEANABS;   // alpha in sequence order: the row encoder's pass 0
-  const TileShape t = tile_shape(pl, mean);
-  if (!t.warps) return launch_encode_range(pl, W, codes, alpha, st, 0, 2, 0, pl->geo.nblk, nullptr, nullptr);
-  if (mean) {
-    const cudaError_t e = launch_encode_range(pl, W, codes, alpha, st, 0, 1, 0, pl->geo.nblk, nullptr, nullptr);
-    if (e != cudaSuccess) return e;
-  }
-  return launch_encode_tile(pl, t, W, codes, alpha, st, mean, false);
+  const TileShape t = tile_shape(pl);
+  return t.warps ? launch_encode_tile(pl, t, W, codes, alpha, st, false)
+                 : launch_encode_range(pl, W, codes, alpha, st, 0, 2, 0, pl->geo.nblk, nullptr, nullptr);
 }
 
 cudaError_t launch_encode_alpha(const sdq_plan_s* pl, const float* W, uint32_t* codes, float* alpha, cudaStream_t st) {
-  const TileShape t = tile_shape(pl, false);
-  if (!t.warps || pl->desc.alpha_mode == SDQ_ALPHA_MEANABS)
-    return launch_encode_range(pl, W, codes, alpha, st, 0, 1, 0, pl->geo.nblk, nullptr, nullptr);
-  return launch_encode_tile(pl, t, W, codes, alpha, st, false, true);
+  const TileShape t = tile_shape(pl);
+  return t.warps ? launch_encode_tile(pl, t, W, codes, alpha, st, true)
+                 : launch_encode_range(pl, W, codes, alpha, st, 0, 1, 0, pl->geo.nblk, nullptr, nullptr);
 }
 
 cudaError_t launch_encode_range(const sdq_plan_s* pl, const float* W, uint32_t* codes, float* alpha,

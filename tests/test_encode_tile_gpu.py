@@ -21,7 +21,9 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(5, 32, 16, 2), (9, 48, 16, 1), (33, 192, 64, 1), (7, 320, 64, Fraction(3, 2)), (161, 128, 64, 3),
           (3, 8192, 64, 2), (2, 20480, 128, 1), (17, 384, 128, Fraction(3, 2)), (700, 256, 128, 2),
           (1, 18560, 128, 2), (6, 896, 128, Fraction(5, 2)), (5, 640, 128, 3), (4, 256, 128, Fraction(7, 2)),
-          (6, 384, 128, Fraction(9, 8)), (3, 512, 256, Fraction(3, 2)), (35, 768, 256, 2), (3, 2048, 256, 3), (5, 1024, 512, 2), (20, 1536, 512, Fraction(5, 2)), (2, 512, 512, 3), (3, 1024, 1024, 2), (6, 64, 8, 2), (5, 640, 64, 5)]
+          (6, 384, 128, Fraction(9, 8)), (3, 512, 256, Fraction(3, 2)), (35, 768, 256, 2), (3, 2048, 256, 3),
+          (5, 1024, 512, 2), (20, 1536, 512, Fraction(5, 2)), (2, 512, 512, 3), (3, 1024, 1024, 2), (6, 64, 8, 2),
+          (5, 640, 64, 5)]
 
 
 @pytest.mark.parametrize("q", [O.TERNARY, O.BINARY])
