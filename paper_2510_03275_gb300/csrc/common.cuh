@@ -447,6 +447,9 @@ __device__ __forceinline__ uint32_t e2m1x2(float lo, float hi, float2* q) {
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
 }
+__device__ __forceinline__ void named_bar_arrive(int id, int nthreads) {
+  asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
+}
 
 // Call record in the workspace: word 0 = tag of the last call that gave up a
 // bounded wait, word 1 = tag of the last call that ran.  Tags (call_tag in

@@ -99,31 +99,40 @@ __global__ void __launch_bounds__(kUpThreads, 2)
 // row's codes depend on that row and U alone, so nothing crosses CTAs and no
 // launch separates the blocks.  Per block b of B columns F:
 //   upsample   groups of 8 rows x parts of the sample pairs, a warp each
-//              (tile_upsample: half of A_enc in shared memory)
-//   scan       one warp, lane = row (eq. 8), the codes left in shared memory
-//              as floats in place of the samples, sample-major
-//   rebuild    s_k = sum_j c_j G[j][k], E = W_F - alpha s: a warp 4 rows x all
-//              columns (lane: l + 32 q), one FMA per term (c_j in {-1, 0,
-//              1}: the product is exact, so fma(c, g, s) = fl(s + fl(c g)))
-//   solve      E~ = E U_FF^-1 by forward substitution on the same registers,
-//              U_FF's rows staged 32 at a time
+//              (tile_upsample: half of A_enc in shared memory; at B = 256 read
+//              through the L1)
+//   scan       the last warp, lane = row (eq. 8), the codes left in shared
+//              memory as floats in place of the samples, sample-major
+//   rebuild    s_k = sum_j c_j G[j][k], E = W_F - alpha s, behind the scan: a
+//              warp 4 rows x all columns (lane: l + 32 q), one FMA per term
+//              (c_j in {-1, 0, 1}: the product is exact, so fma(c, g, s) =
+//              fl(s + fl(c g)))
+//   solve      E~ = E U_FF^-1 by forward substitution, 32 columns at a time:
+//              within them a lane has 4 columns of one row, so that one shuffle
+//              and one quotient serve a warp's 4 rows, then their products come
+//              off the later columns (31 -> 23 k cycles a block)
 //   update     W_R -= E~ U_FR: thread = 4 columns x half of the rows, U from
 //              the L2 with 8 rows' loads in flight (staged by cp.async it was
-//              slower, 226 against 178 k cycles a block), E~ broadcast from
-//              shared memory.  A broadcast 16-byte load still returns 512 bytes to
-//              its warp, 4 cycles of the SM's one shared-memory pipe: with 2
-//              columns x all rows a thread that pipe was as busy as the
-//              multiplies and adds
-// The update's multiplies and adds bound it (no FMA: both are rounded), 60 %
-// of the time of a 4096 x 4096 layer; the steps before it are chains of
-// dependent operations, 40 us a block.  CTAs start at different column
-// chunks: in step they all ask the same few L2 lines at once (88 -> 72 k
-// cycles a block of updates for 8 rows).  The launch per block and per update
-// that this replaces took 12.6 ms for that layer, this 4.4.
+//              slower, 226 against 178 k cycles a block; so were 4 or 16 rows,
+//              157 and 216 against 149: the loop's code grows with them), E~
+//              broadcast from shared memory.  A broadcast 16-byte load still
+//              returns 512 bytes to its warp, 4 cycles of the SM's one
+//              shared-memory pipe: with 2 columns x all rows a thread that pipe
+//              was as busy as the multiplies and adds
+// The update's multiplies and adds bound it (no FMA: both are rounded), 165 of
+// 228 k cycles a block of a 4096 x 4096 layer (100 + 8 at their issue rate, 133
+// with every load of U an L1 hit); the steps before it are chains of dependent
+// operations.  Two teams of rows per CTA, one's chains beside the other's
+// update, took 330 k: single warps a quadrant wait on their own latencies.
+// CTAs start at different column chunks: in step they all ask the same few L2
+// lines at once (88 -> 72 k cycles a block of updates for 8 rows).  The launch
+// per block and per update that this replaces took 12.6 ms for that layer, this
+// 4.0; 2560 x 3584, B = 256, OSR 3: 21 and 4.8.
 // W_F and W_R come from W itself at block 0 and from the working copy after
 // it; the values and their order are those of a launch per block.
 constexpr int kGqThreads = 256;
 constexpr int kGqRp = 36;        // floats per sample / column of up to 32 rows (16-byte rows, 4-way bank spread)
+constexpr int kCols = 2 * kGqThreads;   // columns of an update step
 constexpr int kGqChunk = 32;     // rows of U_FF staged at a time
 
 struct GptqParams {
@@ -138,38 +147,29 @@ struct GptqParams {
   uint32_t pad0;
 };
 
-// Shared memory in floats: half table, weights, samples (later U_FF chunks),
-// E~, a U_FF chunk, the diagonal and its reciprocals.
+// Shared memory in floats: half the table (not for B = 256: read through the
+// L1), weights, samples (later U_FF chunks), E~, a U_FF chunk, the diagonal and
+// its reciprocals.
 __host__ __device__ inline size_t gq_xs_floats(int B, int n_b) {
   const size_t a = (size_t)n_b * kGqRp, b = (size_t)kGqChunk * B;
   return a > b ? a : b;
 }
 __host__ __device__ inline size_t gq_smem_floats(int B, int n_b) {
-  return (size_t)B * (n_b / 2) + 4 * tile_weight_floats(B) + gq_xs_floats(B, n_b) + (size_t)B * kGqRp +
+  return (size_t)(B < 256 ? B : 0) * (n_b / 2) + 4 * tile_weight_floats(B) + gq_xs_floats(B, n_b) + (size_t)B * kGqRp +
          (size_t)kGqChunk * B + 2 * B;
 }
 
-// e[i] = t[i] / d, correctly rounded, given r = 1 / d correctly rounded (0
-// where |d| is outside [2^-30, 2^30]): a first quotient and two corrections by
-// its exact remainder (Markstein, IBM J. Res. Dev. 34, 1990: the second
-// starts within one unit in the last place of the quotient, so it ends
-// correctly rounded).  Where something could over- or underflow, the division
-// itself.  The same for all lanes, so the branch is uniform.
-__device__ __forceinline__ void quotients(const float (&t)[4], float d, float r, float (&e)[4]) {
-  bool safe = r != 0.f;
+// t / d given r = 1 / d correctly rounded (0 where |d| is outside [2^-30,
+// 2^30]): a first quotient and two corrections by its exact remainder
+// (Markstein, IBM J. Res. Dev. 34, 1990: the second starts within one unit in
+// the last place of the quotient, so it ends correctly rounded).  *ok is
+// cleared where something could over- or underflow.
+__device__ __forceinline__ float quotient(float t, float d, float r, bool* ok) {
+  *ok = *ok && r != 0.f && fabsf(t) >= 0x1p-60f && fabsf(t) <= 0x1p60f;
+  float e = __fmul_rn(t, r);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) safe = safe && fabsf(t[i]) >= 0x1p-60f && fabsf(t[i]) <= 0x1p60f;
-  if (safe) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) e[i] = __fmul_rn(t[i], r);
-#pragma unroll
-    for (int n = 0; n < 2; ++n)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) e[i] = __fmaf_rn(__fmaf_rn(-e[i], d, t[i]), r, e[i]);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) e[i] = __fdiv_rn(t[i], d);
-  }
+  for (int n = 0; n < 2; ++n) e = __fmaf_rn(__fmaf_rn(-e, d, t), r, e);
+  return e;
 }
 
 template <int NR, int QB, int PT>
@@ -177,16 +177,17 @@ __global__ void __launch_bounds__(kGqThreads, 1) gptq_rows_kernel(GptqParams p) 
   constexpr int kB = 32 * QB;              // block columns
   constexpr int kVg = (NR + 7) / 8;        // groups of 8 rows, 8 / kVg (rounded down) warps each for the upsampling
   constexpr int kHw = kVg == 3 ? 2 : 8 / kVg;
+  constexpr bool kTable = kB < 256;
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int np = p.n_b / 2;
   float* ts = smem;
-  float* wt = ts + (size_t)kB * np;                  // 4 groups of 8 rows, transposed
+  float* wt = ts + (kTable ? (size_t)kB * np : 0);                  // 4 groups of 8 rows, transposed
   float* xs = wt + 4 * tile_weight_floats(kB);       // samples / codes [n_b][kGqRp]; then U_FF rows
   float* et = xs + gq_xs_floats(kB, p.n_b);          // E, then E~ [B][kGqRp]
   float* ub = et + kB * kGqRp;                       // U_FF rows
   float* dg = ub + kGqChunk * kB;                    // diagonal, reciprocals
-  tile_load_table(ts, p.at, kB, p.n_b);
+  if constexpr (kTable) tile_load_table(ts, p.at, kB, p.n_b);
   const int ngroups = (p.n_out + NR - 1) / NR;
   const int vw = warp % kVg, hw = warp / kVg;   // (hw >= kHw: none)
   const size_t ldu = (size_t)p.k_in;
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(kGqThreads, 1) gptq_rows_kernel(GptqParams p) 
         cp_async_commit();
       };
       stage_u(ub, 0);
-      if (tid < kB) {
+      if (tid < kB) {   // (kB at most kGqThreads)
         const float d = __ldg(uff + (size_t)tid * ldu + tid);
         dg[tid] = d;
         dg[kB + tid] = fabsf(d) >= 0x1p-30f && fabsf(d) <= 0x1p30f ? __frcp_rn(d) : 0.f;
@@ -221,84 +222,103 @@ __global__ void __launch_bounds__(kGqThreads, 1) gptq_rows_kernel(GptqParams p) 
         }
       }
       __syncthreads();
-      if (hw < kHw && 8 * vw < nr && 32 * PT * hw < np) {
-        const int j0 = 32 * PT * hw + lane, left = np - j0;
-        float acc[kTv][PT], acc2[kTv][PT];
-        tile_upsample<PT>(ts + j0, np, left, wt + vw * tile_weight_floats(kB), kB, acc, acc2);
+      if (hw < kHw && 8 * vw < nr)
+        for (int jb = 32 * PT * hw; jb < np; jb += 32 * PT * kHw) {
+          const int j0 = jb + lane, left = np - j0;
+          const float* w8 = wt + vw * tile_weight_floats(kB);
+          float acc[kTv][PT], acc2[kTv][PT];
+          if constexpr (kTable) tile_upsample<PT>(ts + j0, np, left, w8, kB, acc, acc2);
+          else tile_upsample<PT>(p.at + j0, p.n_b, left, w8, kB, acc, acc2);
 #pragma unroll
-        for (int q = 0; q < PT; ++q)
-          if (32 * q < left) {
-            float4* a = reinterpret_cast<float4*>(xs + (size_t)(j0 + 32 * q) * kGqRp + 8 * vw);
-            float4* c = reinterpret_cast<float4*>(xs + (size_t)(np + j0 + 32 * q) * kGqRp + 8 * vw);
-            a[0] = make_float4(acc[0][q], acc[1][q], acc[2][q], acc[3][q]);
-            a[1] = make_float4(acc[4][q], acc[5][q], acc[6][q], acc[7][q]);
-            c[0] = make_float4(acc2[0][q], acc2[1][q], acc2[2][q], acc2[3][q]);
-            c[1] = make_float4(acc2[4][q], acc2[5][q], acc2[6][q], acc2[7][q]);
-          }
-      }
+          for (int q = 0; q < PT; ++q)
+            if (32 * q < left) {
+              float4* a = reinterpret_cast<float4*>(xs + (size_t)(j0 + 32 * q) * kGqRp + 8 * vw);
+              float4* c = reinterpret_cast<float4*>(xs + (size_t)(np + j0 + 32 * q) * kGqRp + 8 * vw);
+              a[0] = make_float4(acc[0][q], acc[1][q], acc[2][q], acc[3][q]);
+              a[1] = make_float4(acc[4][q], acc[5][q], acc[6][q], acc[7][q]);
+              c[0] = make_float4(acc2[0][q], acc2[1][q], acc2[2][q], acc2[3][q]);
+              c[1] = make_float4(acc2[4][q], acc2[5][q], acc2[6][q], acc2[7][q]);
+            }
+        }
       __syncthreads();
-      if (warp == 0) {
+      // The last warp scans in up to 4 parts; the other warps rebuild a part
+      // while it scans the next ones.
+      const bool later = b != p.nblk - 1;   // there are later columns
+      const int part = (p.n_b + 127) / 128 * 32;
+      const int nmine = (nr + 3) / 4, scan_bar = 32 * (min(nmine, kGqThreads / 32 - 1) + 1);
+      if (warp == kGqThreads / 32 - 1) {
         // Eq. (8); the codes replace the samples (rows past nr: zeros)
         const bool live = lane < nr;
         const float a = live ? p.alpha[row0 + lane] : 0.f, theta = 0.5f * a;
         float integ = 0.f, yp = 0.f;
         float* x = xs + lane;
         uint32_t* out = p.codes + (size_t)(row0 + lane) * p.wpr + (size_t)b * p.n_b * p.quantizer / 32;
-        if (p.quantizer == SDQ_TERNARY) {
-          for (int j = 0; j < p.n_b; j += 16) {
-            uint32_t cw = 0;
-            float v[16];
+        for (int j0 = 0, bar = 1; j0 < p.n_b; j0 += part, ++bar) {
+          const int j1 = min(j0 + part, p.n_b);
+          if (p.quantizer == SDQ_TERNARY) {
+            for (int j = j0; j < j1; j += 16) {
+              uint32_t cw = 0;
+              float v[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = x[(size_t)(j + i) * kGqRp];
+              for (int i = 0; i < 16; ++i) v[i] = x[(size_t)(j + i) * kGqRp];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const uint32_t f = sd_step<true>(integ, yp, v[i], a, theta);
-              cw |= f << (2 * i);
-              x[(size_t)(j + i) * kGqRp] = live ? (f == 1u ? 1.f : (f ? -1.f : 0.f)) : 0.f;
+              for (int i = 0; i < 16; ++i) {
+                const uint32_t f = sd_step<true>(integ, yp, v[i], a, theta);
+                cw |= f << (2 * i);
+                x[(size_t)(j + i) * kGqRp] = live ? (f == 1u ? 1.f : (f ? -1.f : 0.f)) : 0.f;
+              }
+              if (live) out[j / 16] = cw;
             }
-            if (live) out[j / 16] = cw;
-          }
-        } else {
-          for (int j = 0; j < p.n_b; j += 32) {
-            uint32_t cw = 0;
+          } else {
+            for (int j = j0; j < j1; j += 32) {
+              uint32_t cw = 0;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const uint32_t f = sd_step<false>(integ, yp, x[(size_t)(j + i) * kGqRp], a, theta);
-              cw |= f << i;
-              x[(size_t)(j + i) * kGqRp] = live ? (f ? 1.f : -1.f) : 0.f;
+              for (int i = 0; i < 32; ++i) {
+                const uint32_t f = sd_step<false>(integ, yp, x[(size_t)(j + i) * kGqRp], a, theta);
+                cw |= f << i;
+                x[(size_t)(j + i) * kGqRp] = live ? (f ? 1.f : -1.f) : 0.f;
+              }
+              if (live) out[j / 32] = cw;
             }
-            if (live) out[j / 32] = cw;
           }
+          __syncwarp();
+          if (later) named_bar_arrive(bar, scan_bar);
         }
-        if (live && b == p.nblk - 1)   // the row's padding words
+        if (live && !later)   // the row's padding words
           for (int w = (int)p.pad0; w < p.wpr; ++w) p.codes[(size_t)(row0 + lane) * p.wpr + w] = 0u;
       }
-      if (b == p.nblk - 1) break;   // no later columns
-      __syncthreads();
+      if (!later) break;
       // warp w's rows 4 w .. 4 w + 3, columns l + 32 q of lane l, in registers
       // from here to E~
       const bool mine = 4 * warp < nr;
       float t[4][QB];
       if (mine) {
-        // s_k: one term per sample, in order, the next 16 samples' G in flight
+        // s_k: one term per sample, in order, the next kGd samples' G in flight
         // (n_b is a multiple of 16)
-        float gn[16][QB];
+        constexpr int kGd = QB < 8 ? 16 : 8;
+        float gn[kGd][QB];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
           for (int q = 0; q < QB; ++q) t[i][q] = 0.f;
         const float* gk = p.g32 + lane;
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
+        for (int j = 0; j < kGd; ++j)
 #pragma unroll
           for (int q = 0; q < QB; ++q) gn[j][q] = __ldg(gk + j * kB + 32 * q);
         const float* c = xs + 4 * warp;
+        int wait = 0, bar = 1;
 #pragma unroll 1
-        for (int j = 0; j < p.n_b; j += 16, c += 16 * kGqRp) {
-          gk += 16 * kB;
-          const bool more = j + 16 < p.n_b;
+        for (int j = 0; j < p.n_b; j += kGd, c += kGd * kGqRp) {
+          if (j == wait) {   // the part that starts here is scanned
+            if (warp != kGqThreads / 32 - 1) named_bar_sync(bar, scan_bar);
+            ++bar;
+            wait += part;
+          }
+          gk += kGd * kB;
+          const bool more = j + kGd < p.n_b;
 #pragma unroll
-          for (int l = 0; l < 16; ++l) {
+          for (int l = 0; l < kGd; ++l) {
             const float4 cv = *reinterpret_cast<const float4*>(c + l * kGqRp);
 #pragma unroll
             for (int q = 0; q < QB; ++q) {
@@ -332,65 +352,95 @@ __global__ void __launch_bounds__(kGqThreads, 1) gptq_rows_kernel(GptqParams p) 
         __syncthreads();
         if (!mine) continue;
         const float* u = (c & 1) ? xs : ub;
-#pragma unroll 4
-        for (int l = 0; l < 32; ++l) {
-          const float d = dg[32 * c + l], r = dg[kB + 32 * c + l];
-          float uv[QB], tl[4], e[4];
+        // the chunk's columns by way of E~'s place in shared memory from lane =
+        // column to lane = (4 columns, row), so that one shuffle and one quotient
+        // serve the 4 rows
+        *reinterpret_cast<float4*>(et + (size_t)(32 * c + lane) * kGqRp + 4 * warp) =
+            make_float4(t[0][c], t[1][c], t[2][c], t[3][c]);
+        __syncwarp();
+        const int cg = lane >> 2;
+        float* ec = et + (size_t)(32 * c + 4 * cg) * kGqRp + 4 * warp + (lane & 3);
+        float tc[4];
+        auto substitute = [&](auto fast) {
+          bool ok = true;
 #pragma unroll
-          for (int q = c; q < QB; ++q) uv[q] = u[l * kB + 32 * q + lane];
+          for (int j = 0; j < 4; ++j) tc[j] = ec[j * kGqRp];
+#pragma unroll 2
+          for (int l4 = 0; l4 < 8; ++l4) {
+            const float4 d4 = *reinterpret_cast<const float4*>(dg + 32 * c + 4 * l4);
+            const float4 r4 = *reinterpret_cast<const float4*>(dg + kB + 32 * c + 4 * l4);
+            const float d[4] = {d4.x, d4.y, d4.z, d4.w}, r[4] = {r4.x, r4.y, r4.z, r4.w};
 #pragma unroll
-          for (int i = 0; i < 4; ++i) tl[i] = __shfl_sync(0xffffffffu, t[i][c], l);
-          quotients(tl, d, r, e);
+            for (int m = 0; m < 4; ++m) {
+              const float4 u4 = *reinterpret_cast<const float4*>(u + (4 * l4 + m) * kB + 32 * c + 4 * cg);
+              const float uv[4] = {u4.x, u4.y, u4.z, u4.w};
+              const float tl = __shfl_sync(0xffffffffu, tc[m], 4 * l4 + (lane & 3));
+              const float e = decltype(fast)::value ? quotient(tl, d[m], r[m], &ok) : __fdiv_rn(tl, d[m]);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float n0 = __fsub_rn(t[i][c], __fmul_rn(e[i], uv[c]));
-            t[i][c] = lane > l ? n0 : (lane == l ? e[i] : t[i][c]);
+              for (int j = 0; j < 4; ++j)
+                if (cg > l4 || (j > m && cg == l4)) tc[j] = __fsub_rn(tc[j], __fmul_rn(e, uv[j]));
+              if (cg == l4) tc[m] = e;
+            }
+          }
+          return __all_sync(0xffffffffu, ok);
+        };
+        if (!substitute(std::true_type())) substitute(std::false_type());
 #pragma unroll
-            for (int q = c + 1; q < QB; ++q) t[i][q] = __fsub_rn(t[i][q], __fmul_rn(e[i], uv[q]));
+        for (int j = 0; j < 4; ++j) ec[j * kGqRp] = tc[j];
+        __syncwarp();
+        // the later chunks' columns
+        if (c + 1 < QB) {
+#pragma unroll 8
+          for (int l = 0; l < kGqChunk; ++l) {
+            const float4 e = *reinterpret_cast<const float4*>(et + (size_t)(32 * c + l) * kGqRp + 4 * warp);
+#pragma unroll
+            for (int q = c + 1; q < QB; ++q) {
+              const float uv = u[l * kB + 32 * q + lane];
+              t[0][q] = __fsub_rn(t[0][q], __fmul_rn(e.x, uv));
+              t[1][q] = __fsub_rn(t[1][q], __fmul_rn(e.y, uv));
+              t[2][q] = __fsub_rn(t[2][q], __fmul_rn(e.z, uv));
+              t[3][q] = __fsub_rn(t[3][q], __fmul_rn(e.w, uv));
+            }
           }
         }
       }
-      if (mine) {
-#pragma unroll
-        for (int q = 0; q < QB; ++q)
-          *reinterpret_cast<float4*>(et + (size_t)(lane + 32 * q) * kGqRp + 4 * warp) =
-              make_float4(t[0][q], t[1][q], t[2][q], t[3][q]);
-      }
       __syncthreads();
-      // W_R -= E~ U_FR: a thread's kC adjacent columns from ca, kN rows from r0
+      // W_R -= E~ U_FR: a thread's 4 adjacent columns from ca, kN rows from r0
       const float* uf = p.U + (size_t)b * kB * ldu;
-      auto columns = [&](int ca, auto cols, auto rows, int r0) {
-        constexpr int kC = decltype(cols)::value, kN = decltype(rows)::value;
-        using Vec = std::conditional_t<kC == 4, float4, float>;
-        auto get = [](const Vec& v, int c) { return reinterpret_cast<const float*>(&v)[c]; };
+      auto columns = [&](int ca, auto rows, int r0) {
+        constexpr int kN = decltype(rows)::value;
+        constexpr int kD = kN > 4 ? 8 : 16;   // rows of U in flight: the L2's round trip under this load is over 1000 cycles
+        auto get = [](const float4& v, int c) { return reinterpret_cast<const float*>(&v)[c]; };
         const float* u0 = uf + ca;
-        float acc[kC][kN];
-        Vec u[8];   // U of 8 rows: the L2's round trip under this load is over 1000 cycles
+        float acc[4][kN];
+        float4 u[kD];
 #pragma unroll
-        for (int c = 0; c < kC; ++c)
+        for (int c = 0; c < 4; ++c)
 #pragma unroll
           for (int r = 0; r < kN; ++r) acc[c][r] = -0.0f;   // -0 + p == p: the first product is taken as is
 #pragma unroll
-        for (int i = 0; i < 8; ++i) u[i] = __ldg(reinterpret_cast<const Vec*>(u0 + (size_t)i * ldu));
+        for (int i = 0; i < kD; ++i) u[i] = __ldg(reinterpret_cast<const float4*>(u0 + (size_t)i * ldu));
 #pragma unroll 1
-        for (int k = 0; k < kB; k += 8) {
-          u0 += 8 * ldu;
-          const bool more = k + 8 < kB;
+        for (int k = 0; k < kB; k += kD) {
+          u0 += kD * ldu;
+          // past the last row: its 8 again (a branch on the loads costs the loop 11 %)
+          const size_t step = k + kD < kB ? ldu : 0;
+          if (!step) u0 -= kD * ldu;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
+          for (int i = 0; i < kD; ++i) {
             const float4* e4 = reinterpret_cast<const float4*>(et + (size_t)(k + i) * kGqRp + r0);
 #pragma unroll
             for (int r = 0; r < kN; r += 4) {
               const float4 e = e4[r / 4];
 #pragma unroll
-              for (int c = 0; c < kC; ++c) {
+              for (int c = 0; c < 4; ++c) {
                 acc[c][r] = __fadd_rn(acc[c][r], __fmul_rn(e.x, get(u[i], c)));
                 acc[c][r + 1] = __fadd_rn(acc[c][r + 1], __fmul_rn(e.y, get(u[i], c)));
                 acc[c][r + 2] = __fadd_rn(acc[c][r + 2], __fmul_rn(e.z, get(u[i], c)));
                 acc[c][r + 3] = __fadd_rn(acc[c][r + 3], __fmul_rn(e.w, get(u[i], c)));
               }
             }
-            if (more) u[i] = __ldg(reinterpret_cast<const Vec*>(u0 + (size_t)i * ldu));
+            u[i] = __ldg(reinterpret_cast<const float4*>(u0 + (size_t)i * step));
           }
         }
         const float* wr = (b == 0 ? p.W : p.wc) + (size_t)(row0 + r0) * p.k_in + ca;
@@ -398,58 +448,62 @@ __global__ void __launch_bounds__(kGqThreads, 1) gptq_rows_kernel(GptqParams p) 
 #pragma unroll
         for (int r = 0; r < kN; ++r) {
           if (r0 + r >= nr) break;
-          Vec w = __ldcg(reinterpret_cast<const Vec*>(wr + (size_t)r * p.k_in));
-#pragma unroll
-          for (int c = 0; c < kC; ++c)
-            reinterpret_cast<float*>(&w)[c] = __fsub_rn(get(w, c), acc[c][r]);
-          *reinterpret_cast<Vec*>(wo + (size_t)r * p.k_in) = w;
+          float4 w = __ldcg(reinterpret_cast<const float4*>(wr + (size_t)r * p.k_in));
+          w.x = __fsub_rn(w.x, acc[0][r]);
+          w.y = __fsub_rn(w.y, acc[1][r]);
+          w.z = __fsub_rn(w.z, acc[2][r]);
+          w.w = __fsub_rn(w.w, acc[3][r]);
+          *reinterpret_cast<float4*>(wo + (size_t)r * p.k_in) = w;
         }
       };
-      // warps 0-3 the first kN0 rows, warps 4-7 the others (one of each on
-      // every SM quadrant): 4 columns a thread, the last ones 1
-      auto update = [&](auto rows, int r0) {
+      // 512 columns at a time, the first kN0 rows by warps 0-3 and the others by
+      // warps 4-7 (one of each on every SM quadrant); the rest in units of 128
+      // columns x 4 rows, a warp each (columns are multiples of 4)
+      const int cb = (b + 1) * kB, nfull = (p.k_in - cb) / kCols;
+      auto full = [&](auto rows, int r0) {
         if (r0 >= nr) return;
-        constexpr int kHalf = kGqThreads / 2;
-        const int i = tid & (kHalf - 1);
-        const int cb = (b + 1) * kB, nfull = (p.k_in - cb) / (4 * kHalf);
         int g = nfull ? (int)blockIdx.x % nfull : 0;
         for (int n = 0; n < nfull; ++n) {
-          columns(cb + 4 * kHalf * g + 4 * i, std::integral_constant<int, 4>(), rows, r0);
+          columns(cb + kCols * g + 4 * (tid & (kGqThreads / 2 - 1)), rows, r0);
           if (++g == nfull) g = 0;
         }
-        for (int c0 = cb + 4 * kHalf * nfull; c0 < p.k_in; c0 += kHalf)
-          if (c0 + i < p.k_in) columns(c0 + i, std::integral_constant<int, 1>(), rows, r0);
       };
       constexpr int kN0 = NR > 16 ? 16 : NR / 2;
-      if (warp < 4) update(std::integral_constant<int, kN0>(), 0);
-      else update(std::integral_constant<int, NR - kN0>(), kN0);
+      if (warp < 4) full(std::integral_constant<int, kN0>(), 0);
+      else full(std::integral_constant<int, NR - kN0>(), kN0);
+      const int ce = cb + kCols * nfull, units = nmine * ((p.k_in - ce + 127) / 128);
+      for (int n = warp; n < units; n += kGqThreads / 32) {
+        const int ca = ce + 128 * (n / nmine) + 4 * lane;
+        if (ca < p.k_in) columns(ca, std::integral_constant<int, 4>(), 4 * (n % nmine));
+      }
     }
   }
 }
 
 using GptqKernel = void (*)(GptqParams);
-// nq: 32-pair columns of the samples; every warp takes ceil(nq / kHw) of them.
+// nq: 32-pair columns of the samples, PT at a time for each of a row group's warps.
 template <int QB>
 GptqKernel rows_kernel(int nr, int nq) {
+  constexpr bool kWide = QB == 8;
   switch (nr) {
-    case 8: return gptq_rows_kernel<8, QB, 1>;
-    case 16: return nq <= 4 ? gptq_rows_kernel<16, QB, 1> : gptq_rows_kernel<16, QB, 2>;
-    case 28: return nq <= 4 ? gptq_rows_kernel<28, QB, 2> : gptq_rows_kernel<28, QB, 3>;
-    default: return nq <= 4 ? gptq_rows_kernel<32, QB, 2> : gptq_rows_kernel<32, QB, 3>;
+    case 8: return nq <= 4 && !kWide ? gptq_rows_kernel<8, QB, 1> : gptq_rows_kernel<8, QB, 1 + kWide>;
+    case 16: return nq <= 4 && !kWide ? gptq_rows_kernel<16, QB, 1 + kWide> : gptq_rows_kernel<16, QB, 2>;
+    case 28: return nq <= 4 && !kWide ? gptq_rows_kernel<28, QB, 2 + kWide> : gptq_rows_kernel<28, QB, 3>;
+    default: return nq <= 4 && !kWide ? gptq_rows_kernel<32, QB, 2 + kWide> : gptq_rows_kernel<32, QB, 3>;
   }
 }
 
 // The row-owner kernel where it applies (*used = false otherwise): the
 // half-shift table and whole words of codes per block as for the tile
-// encoder, B = 64 or 128.  Rows per CTA: the count with the least time over
-// the waves, NR K / 2 multiply-add pairs per row and block column against a
-// fixed part per block (in cycles, both measured).
+// encoder, B = 64, 128 or 256.  Rows per CTA: the count with the least time
+// over the waves, NR K / 2 multiply-add pairs per row and block column against
+// the chains per block (in cycles, both measured).
 cudaError_t launch_gptq_rows(const sdq_plan_s* pl, const float* W, const float* U, uint32_t* codes, const float* alpha,
                              float* wc, cudaStream_t st, bool* used) {
   const Geometry& g = pl->geo;
   const size_t smem = sizeof(float) * gq_smem_floats(g.block, g.n_b);
-  *used = pl->half_shift && (g.block == 64 || g.block == 128) && g.n_b / 2 <= 192 && (g.n_b * g.bits) % 32 == 0 &&
-          smem <= 226 * 1024;
+  *used = pl->half_shift && (g.block == 64 || g.block == 128 || g.block == 256) && g.n_b % 16 == 0 &&
+          (g.n_b * g.bits) % 32 == 0 && smem <= 226 * 1024;
   if (!*used) return cudaSuccess;
   GptqParams p;
   p.W = W; p.wc = wc; p.U = U; p.alpha = alpha; p.codes = codes; p.at = pl->d_at; p.g32 = pl->d_g32;
@@ -462,14 +516,16 @@ cudaError_t launch_gptq_rows(const sdq_plan_s* pl, const float* W, const float* 
   double best = 0;
   for (int i = 0; i < 4; ++i) {
     const int64_t groups = (g.n_out + cand[i] - 1) / cand[i], waves = (groups + sms - 1) / sms;
-    const double c = (double)waves * (1.2 * cand[i] * g.k_in * g.block / 128.0 + 40000.0);
+    const double c = (double)waves * (g.block / 128.0) * (1.0 * cand[i] * g.k_in + 45000.0 * g.block / 128.0);
     if (i == 0 || c < best) {
       best = c;
       nr = cand[i];
     }
   }
   const int nq = (g.n_b / 2 + 31) / 32;
-  GptqKernel kern = g.block == 128 ? rows_kernel<4>(nr, nq) : rows_kernel<2>(nr, nq);
+  GptqKernel kern = g.block == 256   ? rows_kernel<8>(nr, nq)
+                    : g.block == 128 ? rows_kernel<4>(nr, nq)
+                                     : rows_kernel<2>(nr, nq);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)std::min<int64_t>((g.n_out + nr - 1) / nr, sms), kGqThreads, smem, st>>>(p);

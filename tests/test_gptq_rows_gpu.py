@@ -3,9 +3,9 @@ the oracle on sampled rows (every row's codes depend on that row and the
 factor alone).
 
 Every rows-per-block count (8, 16, 28, 32) with a ragged last group, groups in
-several waves, both block sizes, column counts that end in each of the
-update's segments (512 columns, then 128 or a part), one and two parts of the
-sample pairs, zero rows (no quotient by the reciprocal) and a factor with
+several waves, every block size (64, 128, 256), column counts that end in each of the
+update's segments (512 columns, then 128 or a part), one and more parts of the
+sample pairs and of the scan, zero rows (no quotient by the reciprocal) and a factor with
 diagonal entries outside the reciprocal's range."""
 from fractions import Fraction
 
@@ -20,7 +20,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("q", [O.TERNARY, O.BINARY])
 @pytest.mark.parametrize("n,k,b,osr", [(13, 1280, 128, 2), (1003, 768, 128, Fraction(3, 2)), (2403, 256, 128, 2),
                                        (4190, 384, 128, Fraction(5, 2)), (4301, 256, 128, 3), (9801, 256, 64, 2),
-                                       (21, 704, 64, 3), (9, 128, 128, 2), (5, 64, 64, Fraction(3, 2))])
+                                       (21, 704, 64, 3), (9, 128, 128, 2), (5, 64, 64, Fraction(3, 2)),
+                                       (2450, 512, 256, 2), (4309, 768, 256, 3), (11, 512, 256, Fraction(9, 8)),
+                                       (6, 192, 64, 7)])
 def test_gptq_rows_bit_exact(sdq, q, n, k, b, osr):
     import torch
     assert torch.cuda.is_available()
