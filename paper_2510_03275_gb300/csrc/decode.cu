@@ -67,8 +67,10 @@
 //                 into the ring with bulk copies
 // With `early` set the producers start the code stream (one stage each)
 // before waiting for the preceding grid (codes are never written by the
-// prep kernels), except with bstream, where each stage also copies B rows
-// and scale words that grid writes.
+// prep kernels; with bstream the stage's B rows and scale words, which that
+// grid writes, follow after the wait), and the expanders expand those stages'
+// codes before they wait, so that only the B scales are left to do then (4096 x
+// 4096, M = 1: from the B operand's arrival to the first MMA 1.1 us, so 0.7).
 //
 // bstream (batches whose term rows make a chunk-resident B image bound the k
 // chunk): each stage's image pairs and scale words are bulk-copied into its
@@ -296,12 +298,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
   tc_fence_after();
   pdl_launch_dependents();
   // (the builders wait inside their build; the producers, with `early`,
-  // after their stages)
+  // after their first stages' codes)
   const bool builder = warp >= kExpWarp0 && warp < kProducerWarp0;
   const bool epilogue = warp >= kEpiWarp0 && warp < kExpWarp0;
-  // (with bstream the producers copy B rows the preceding grid writes: they
-  // wait for it before their first stage)
-  const bool early = p.early && !p.bstream;
+  const bool early = p.early != 0;
   if (!builder && !epilogue && (warp < kProducerWarp0 || !early)) pdl_wait();
   const uint32_t tmem = tmem_base;
   bool ok = true;
@@ -336,6 +336,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
         const uint32_t sbytes = (uint32_t)(b1 - b0) * (uint32_t)p.NP * 4u;
         mbar_expect_tx_warp(&c_full[slot], bytes + bb + sbytes);
         bulk_g2s_hint_warp(dst, src, bytes, &c_full[slot], pol);
+        if (!waited) { pdl_wait(); waited = true; }   // that grid writes the rest
         bulk_g2s_warp(dst + p.boff, p.bimg + (size_t)pa0 * p.NP * 128, bb, &c_full[slot]);
         bulk_g2s_warp(dst + p.soff, p.sfbw + (size_t)(kb0 + b0) * p.NP * 4, sbytes, &c_full[slot]);
       } else {
@@ -420,6 +421,85 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
   } else if (warp >= kExpWarp0) {
     // ------------------------------------------------ builders, then expanders
     const int et = tid - 32 * kExpWarp0;
+    // Set x expands stages i = x (mod 4) in order: ring slot i mod ring,
+    // TMEM slot i mod ns (its codes, then its B scales).
+    const int x = (warp - kExpWarp0) >> 2, q = warp & 3, r = 32 * q + lane;
+    const int MT = p.M * p.T;
+    const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16);
+    const uint32_t aslot = (uint32_t)(kAColsPerBlk * p.sb);
+    const uint32_t slab = p.blk_bytes / 2;
+    int u = 0, j = x, slot = x, rnd = 0;
+    while (j >= spu) { j -= spu; ++u; }
+    // a stage's codes from the ring slot at cs into registers, ...
+    auto load = [&](const uint8_t* cs, int nb, uint32_t (&w)[kMaxSb][8]) {
+#pragma unroll
+      for (int bb = 0; bb < kMaxSb; ++bb) {
+        if (bb < nb) {
+          const uint8_t* cb = cs + bb * p.blk_bytes;
+          if constexpr (kTernary) {
+            const uint4 g0 = *reinterpret_cast<const uint4*>(cb + r * 16);
+            const uint4 g1 = *reinterpret_cast<const uint4*>(cb + slab + r * 16);
+            w[bb][0] = g0.x; w[bb][1] = g0.y; w[bb][2] = g0.z; w[bb][3] = g0.w;
+            w[bb][4] = g1.x; w[bb][5] = g1.y; w[bb][6] = g1.z; w[bb][7] = g1.w;
+          } else {
+            const uint2 g0 = *reinterpret_cast<const uint2*>(cb + r * 8);
+            const uint2 g1 = *reinterpret_cast<const uint2*>(cb + slab + r * 8);
+            w[bb][0] = ~g0.x; w[bb][1] = ~g0.y; w[bb][2] = ~g1.x; w[bb][3] = ~g1.y;
+          }
+        }
+      }
+    };
+    // ... and expanded into TMEM slot s
+    auto put = [&](const uint32_t (&w)[kMaxSb][8], int nb, int s) {
+      // Few, wide TMEM stores: a tcgen05.st costs its warp a few hundred
+      // cycles here whatever its width.  The codes first, two blocks per
+      // store ...
+#pragma unroll
+      for (int bp = 0; bp < kMaxSb; bp += 2) {
+        if (bp < nb) {
+          // e2m1 nibble [sign, code bit 0, 0, 0]: +-2.0 or 0 (decode_stage_k order)
+          uint32_t v[32];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int bb = bp + h;
+            if constexpr (kTernary) {
+#pragma unroll
+              for (int wi = 0; wi < 8; ++wi) {
+                v[16 * h + 2 * wi] = (w[bb][wi] << 2) & 0xCCCCCCCCu;   // even codes
+                v[16 * h + 2 * wi + 1] = w[bb][wi] & 0xCCCCCCCCu;      // odd codes
+              }
+            } else {   // words hold the inverted bits: 1 = -1
+#pragma unroll
+              for (int wi = 0; wi < 4; ++wi)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                  v[16 * h + 4 * wi + k] = ((w[bb][wi] << (3 - k)) & 0x88888888u) | 0x44444444u;
+            }
+          }
+          const uint32_t ad = lane_addr + (uint32_t)s * aslot + (uint32_t)(kAColsPerBlk * bp);
+          if (bp + 1 < nb) {
+            tmem_st32(ad, v);
+          } else {
+            uint32_t v16[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v16[i] = v[i];
+            tmem_st16(ad, v16);
+          }
+        }
+      }
+    };
+    // with `early` the first stage's codes before the preceding grid completes
+    // (with bstream the slot fills after it: no bounded wait spans that grid)
+    const bool ahead = early && !p.bstream && x < nstages;
+    if (ahead) {
+      ok = warp_wait(&c_full[slot], 0);
+      if (ok) {
+        uint32_t w[kMaxSb][8];
+        const int nb = sblk[j + 1] - sblk[j];
+        load(ring + (size_t)slot * p.slot_bytes, nb, w);
+        put(w, nb, x);   // (x < ns)
+      }
+    }
     pdl_wait();
     if (p.bstream) {
       // (the B rows and scale words arrive with each stage)
@@ -457,18 +537,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
     named_bar_sync(3, kBuildThreads);
     if (et == 0) mbar_arrive(&b_full);   // (every issuer waits on its one phase)
 
-    // Set x expands stages i = x (mod 4) in order: ring slot i mod ring,
-    // TMEM slot i mod ns (its codes, then its B scales).
-    const int x = (warp - kExpWarp0) >> 2, q = warp & 3, r = 32 * q + lane;
-    const int MT = p.M * p.T;
-    const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16);
-    const uint32_t aslot = (uint32_t)(kAColsPerBlk * p.sb);
-    const uint32_t slab = p.blk_bytes / 2;
-    int u = 0, j = x, slot = x, rnd = 0;
-    while (j >= spu) { j -= spu; ++u; }
     for (int i = x; i < nstages && ok; i += kExpSets) {
       const int s = i & (p.ns - 1);
-      ok = warp_wait(&c_full[slot], rnd & 1);
+      const bool done = ahead && i == x;   // the codes are in TMEM
+      if (!done) ok = warp_wait(&c_full[slot], rnd & 1);
       if (!ok) break;
       // Codes into registers first, so that the ring slot goes back to the
       // producer before this set waits for its TMEM slot.
@@ -477,22 +549,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
       while (j >= spu) { j -= spu; ++u; }
       const uint8_t* cs = ring + (size_t)slot * p.slot_bytes;
       uint32_t w[kMaxSb][8];
-#pragma unroll
-      for (int bb = 0; bb < kMaxSb; ++bb) {
-        if (bb < nb) {
-          const uint8_t* cb = cs + bb * p.blk_bytes;
-          if constexpr (kTernary) {
-            const uint4 g0 = *reinterpret_cast<const uint4*>(cb + r * 16);
-            const uint4 g1 = *reinterpret_cast<const uint4*>(cb + slab + r * 16);
-            w[bb][0] = g0.x; w[bb][1] = g0.y; w[bb][2] = g0.z; w[bb][3] = g0.w;
-            w[bb][4] = g1.x; w[bb][5] = g1.y; w[bb][6] = g1.z; w[bb][7] = g1.w;
-          } else {
-            const uint2 g0 = *reinterpret_cast<const uint2*>(cb + r * 8);
-            const uint2 g1 = *reinterpret_cast<const uint2*>(cb + slab + r * 8);
-            w[bb][0] = ~g0.x; w[bb][1] = ~g0.y; w[bb][2] = ~g1.x; w[bb][3] = ~g1.y;
-          }
-        }
-      }
+      if (!done) load(cs, nb, w);
       __syncwarp();
       if (lane == 0 && !p.bstream) mbar_arrive(&c_empty[slot]);
       // (bstream: the slot's scale words are read below; the MMAs release it)
@@ -505,42 +562,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
         if (!ok) break;
         tc_fence_after();
       }
-      // Few, wide TMEM stores: a tcgen05.st costs its warp a few hundred
-      // cycles here whatever its width.  The codes first, two blocks per
-      // store ...
-#pragma unroll
-      for (int bp = 0; bp < kMaxSb; bp += 2) {
-        if (bp < nb) {
-          // e2m1 nibble [sign, code bit 0, 0, 0]: +-2.0 or 0 (decode_stage_k order)
-          uint32_t v[32];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int bb = bp + h;
-            if constexpr (kTernary) {
-#pragma unroll
-              for (int wi = 0; wi < 8; ++wi) {
-                v[16 * h + 2 * wi] = (w[bb][wi] << 2) & 0xCCCCCCCCu;   // even codes
-                v[16 * h + 2 * wi + 1] = w[bb][wi] & 0xCCCCCCCCu;      // odd codes
-              }
-            } else {   // words hold the inverted bits: 1 = -1
-#pragma unroll
-              for (int wi = 0; wi < 4; ++wi)
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                  v[16 * h + 4 * wi + k] = ((w[bb][wi] << (3 - k)) & 0x88888888u) | 0x44444444u;
-            }
-          }
-          const uint32_t ad = lane_addr + (uint32_t)s * aslot + (uint32_t)(kAColsPerBlk * bp);
-          if (bp + 1 < nb) {
-            tmem_st32(ad, v);
-          } else {
-            uint32_t v16[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v16[i] = v[i];
-            tmem_st16(ad, v16);
-          }
-        }
-      }
+      if (!done) put(w, nb, s);
       // ... then the stage's B scales (one store for the slot when a block's
       // set is 4 columns)
       const uint32_t sc = lane_addr + (uint32_t)p.sfs + (uint32_t)(s * p.sss);
@@ -651,13 +673,17 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) sum[i] = 0.f;
 #pragma unroll
-        for (int e = 0; e < kMaxPipes; ++e) {
-          if ((in >> e) & 1u) {
-            uint32_t rr[16];
-            tmem_ld16(lq + (uint32_t)(p.dbase + (e * p.nbuf + kc[e] % p.nbuf) * p.NP + c0), rr);
-            tmem_ld_wait();
+        for (int e0 = 0; e0 < kMaxPipes; e0 += 2) {   // two pipelines' loads per wait
+          if (((in >> e0) & 3u) == 0u) continue;
+          uint32_t r0[16], r1[16];
+          tmem_ld16(lq + (uint32_t)(p.dbase + (e0 * p.nbuf + kc[e0] % p.nbuf) * p.NP + c0), r0);
+          tmem_ld16(lq + (uint32_t)(p.dbase + (min(e0 + 1, np - 1) * p.nbuf + kc[e0 + 1] % p.nbuf) * p.NP + c0), r1);
+          tmem_ld_wait();
+          const bool h0 = (in >> e0) & 1u, h1 = (in >> (e0 + 1)) & 1u;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) sum[i] += __uint_as_float(rr[i]);
+          for (int i = 0; i < 16; ++i) {
+            if (h0) sum[i] += __uint_as_float(r0[i]);
+            if (h1) sum[i] += __uint_as_float(r1[i]);
           }
         }
         if (c0 + 16 >= MT) {
@@ -668,22 +694,22 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
         }
       };
       if (MT <= 8) {
-        // one batch row: 8 columns of two pipelines' accumulators in flight
-        // per wait (the last tile's epilogue is the call's tail)
+        // one batch row: 8 columns of every pipeline's accumulator, one wait
+        // (the last tile's epilogue is the call's tail: from the last MMA to
+        // the write 1.0 us with two waits, 0.5 so)
         float acc = 0.f;
+        uint32_t rr[kMaxPipes][8];
 #pragma unroll
-        for (int e0 = 0; e0 < kMaxPipes; e0 += 2) {
-          const bool h0 = (in >> e0) & 1u, h1 = (in >> (e0 + 1)) & 1u;
-          uint32_t r0[8], r1[8];
-          if (h0) tmem_ld8(lq + (uint32_t)(p.dbase + (e0 * p.nbuf + kc[e0] % p.nbuf) * p.NP), r0);
-          if (h1) tmem_ld8(lq + (uint32_t)(p.dbase + ((e0 + 1) * p.nbuf + kc[e0 + 1] % p.nbuf) * p.NP), r1);
-          if (h0 || h1) tmem_ld_wait();
+        for (int e = 0; e < kMaxPipes; ++e)   // (pipelines not in this tile: read and not used)
+          tmem_ld8(lq + (uint32_t)(p.dbase + (min(e, np - 1) * p.nbuf + kc[e] % p.nbuf) * p.NP), rr[e]);
+        tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            if (h0 && i < MT) acc += __uint_as_float(r0[i]);
-            if (h1 && i < MT) acc += __uint_as_float(r1[i]);
+        for (int e = 0; e < kMaxPipes; ++e)
+          if ((in >> e) & 1u) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (i < MT) acc += __uint_as_float(rr[e][i]);
           }
-        }
         tc_fence_before();
 #pragma unroll
         for (int e = 0; e < kMaxPipes; ++e)

@@ -144,12 +144,15 @@ __global__ void __launch_bounds__(128) prep_kernel(PrepParams p) {
 // kap = 2 byte + nibble (decode_pos order); its scales are the bytes of
 // word (kb, n) of `sfbw`: byte 2 mu + beta = 2^(e - 3t) of K group beta of
 // the block's MMA mu.  The CTA's x tile and G rows arrive in one round of
-// asynchronous copies (k chunks of up to 256).
+// asynchronous copies (k chunks of up to 256).  Latency bounds it (8 to 100
+// CTAs): 2.2 us from the preceding grid's end at 4096 x 11008, M = 1 (2.5 with
+// x_tilde also written where only the image is read, and the library's frexp
+// and ldexp; 5.2 -> 3.8 at 5120 x 5120, M = 8).
 struct DecPrepParams {
   const uint16_t* x;
   const uint16_t* g_hi;
   const uint16_t* g_lo;
-  float* xt;          // M x kpad fp32
+  float* xt;          // M x kpad fp32 (null: not wanted, the image alone)
   uint8_t* bimg;      // B operand image (null: x_tilde only)
   uint8_t* sfbw;      // B scale words, KB x NP x 4 bytes
   float* y_zero;      // cleared (M x n_out) for the decode kernel's atomic split-K, or null
@@ -241,20 +244,27 @@ __global__ void __launch_bounds__(128) prep_decode_kernel(DecPrepParams p) {
     __syncthreads();
   }
 
-  // x_tilde of the tile: to global memory (fp32) and to shared memory (the G
-  // tiles are no longer read) for the terms below
-  float* tile = reinterpret_cast<float*>(dsm);   // TB x 64
+  // x_tilde of the tile: to global memory (fp32, where it is asked for) and to
+  // shared memory (the G tiles are no longer read) for the terms below
+  constexpr int kTld = 72;
+  float* tile = reinterpret_cast<float*>(dsm);   // TB x kTld
 #pragma unroll
   for (int n = 0; n < NTW; ++n)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int bl = g + (e >> 1) * 8, jl = wcol + n * 8 + 2 * t + (e & 1);
-      const int b = b0 + bl, j = j0 + jl;
-      if (b < p.nblk && j < p.n_b) p.xt[(size_t)m * p.kpad + (int64_t)b * p.n_b + j] = acc[n][e];
-      tile[bl * 64 + jl] = acc[n][e];
-    }
+    for (int h = 0; h < 2; ++h)
+      *reinterpret_cast<float2*>(tile + (g + 8 * h) * kTld + wcol + n * 8 + 2 * t) =
+          make_float2(acc[n][2 * h], acc[n][2 * h + 1]);
+  if (p.xt) {
+#pragma unroll
+    for (int n = 0; n < NTW; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int b = b0 + g + (e >> 1) * 8, j = j0 + wcol + n * 8 + 2 * t + (e & 1);
+        if (b < p.nblk && j < p.n_b) p.xt[(size_t)m * p.kpad + (int64_t)b * p.n_b + j] = acc[n][e];
+      }
+  }
   // K padding of this batch row
-  if (jt == 0 && bt == 0)
+  if (p.xt && jt == 0 && bt == 0)
     for (int64_t k = p.k_eff + tid; k < p.kpad; k += 128) p.xt[(size_t)m * p.kpad + k] = 0.f;
   if (!p.bimg) return;
   __syncthreads();
@@ -274,18 +284,14 @@ __global__ void __launch_bounds__(128) prep_decode_kernel(DecPrepParams p) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int kl = decode_stage_k(8 * g8 + i, ter);
-      v[i] = act ? tile[bl * 64 + (kl - kl0)] : 0.f;
+      v[i] = act ? tile[bl * kTld + (kl - kl0)] : 0.f;
       mx = fmaxf(mx, fabsf(v[i]));
     }
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    int ex = -125;
-    if (mx > 0.f) {   // mx < 2^E, so |v 2^-(E - 2)| < 4
-      int E = 0;
-      frexpf(mx, &E);
-      ex = E - 2;
-    }
-    const float inv = ldexpf(1.f, -ex);
+    // mx < 2^E, E - 126 its exponent field, so |v 2^-(E - 2)| < 4
+    const int ex = max(-125, min(126, (int)(__float_as_uint(mx) >> 23) - 128));
+    const float inv = __uint_as_float((uint32_t)(127 - ex) << 23);
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] *= inv;
     if (act) {
@@ -333,8 +339,8 @@ cudaError_t launch_prep(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws
     const DecodeConfig& dc = decode_config(pl, M);
     DecPrepParams p;
     p.x = x; p.g_hi = pl->d_g_hi; p.g_lo = pl->d_g_lo;
-    p.xt = reinterpret_cast<float*>(base + L.xt);
     p.bimg = decode_image(pl) ? base + L.bimg : nullptr;
+    p.xt = forward && p.bimg ? nullptr : reinterpret_cast<float*>(base + L.xt);
     p.sfbw = base + L.sfbw;
     p.T = dc.T; p.NP = dc.NP;
     p.y_zero = y_zero;
