@@ -84,8 +84,8 @@ WsLayout workspace_layout(const sdq_plan_s* pl, int M) {
     off = align_up(off + 2 * sizeof(uint64_t), 256);
     L.least = off;
     if (prefill_route(pl, M)) {
-      // call record, bf16 x_tilde, then (sdq_prep_activations alone) fp32
-      // x_tilde; a forward call needs the first two, less than the above
+      // call record, bf16 x_tilde, then fp32 x_tilde; a forward call needs the
+      // first two, less than the above
       L.err = 0;
       L.xtb = 256;
       L.xt = L.xtb + align_up(sizeof(uint16_t) * (size_t)M * g.k_eff_pad, 256);
@@ -297,7 +297,9 @@ extern "C" int sdq_linear_forward(sdq_plan p, const uint32_t* codes_tiled, const
     const cudaError_t e = launch_dense_forward(p, codes_tiled, alpha, x, M, y, ws, (cudaStream_t)stream);
     if (e != cudaErrorNotSupported) return cuda_status(e);
   }
-  st = cuda_status(launch_prep(p, x, M, ws, (cudaStream_t)stream, zero_y ? y : nullptr, /*forward=*/true));
+  // (fp32 x_tilde, for sdq_read_prep, where the workspace has room for it)
+  st = cuda_status(launch_prep(p, x, M, ws, (cudaStream_t)stream, zero_y ? y : nullptr,
+                               ws_bytes >= workspace_layout(p, M).total));
   if (st != SDQ_OK) return st;
   return contract(p, codes_tiled, alpha, M, y, ws, ws_bytes, stream, 1, zero_y ? kYZeroed : kYStore);
 }

@@ -47,10 +47,10 @@ cudaError_t launch_pack(const sdq_plan_s* p, const uint32_t* plain, uint32_t* ti
 cudaError_t launch_unpack(const sdq_plan_s* p, const uint32_t* tiled, uint32_t* plain,
                           uint32_t* bad, cudaStream_t st);
 // y_zero (M x n_out, may be null): cleared by the decode prepare kernel.
-// forward: only what this call's contraction reads (else also the fp32 x_tilde
-// of a decode batch that contracts with the prefill kernel).
+// keep_xt: also the fp32 x_tilde of a decode batch that contracts with the
+// prefill kernel (which does not read it).
 cudaError_t launch_prep(const sdq_plan_s* p, const uint16_t* x, int M, void* ws, cudaStream_t st,
-                        float* y_zero = nullptr, bool forward = false);
+                        float* y_zero = nullptr, bool keep_xt = true);
 // Decode batches from here on contract with the prefill kernel (kMaxDecodeM +
 // 1: none do).
 int wide_min_batch(const sdq_plan_s* p);
@@ -442,6 +442,13 @@ __device__ __forceinline__ uint32_t e2m1x2(float lo, float hi, float2* q) {
       : "=h"(b), "=r"(h2) : "f"(lo), "f"(hi));
   *q = __half22float2(*reinterpret_cast<const __half2*>(&h2));
   return b;
+}
+
+// r[0 .. 7] to the 32 bytes at p (32-byte aligned), one store.
+__device__ __forceinline__ void st_global32(void* p, const uint32_t* r) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+               "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
 }
 
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {

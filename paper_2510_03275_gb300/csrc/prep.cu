@@ -146,13 +146,13 @@ __global__ void __launch_bounds__(128) prep_kernel(PrepParams p) {
 // the block's MMA mu.  The CTA's x tile and G rows arrive in one round of
 // asynchronous copies (k chunks of up to 256).  Latency bounds it (8 to 100
 // CTAs): 2.2 us from the preceding grid's end at 4096 x 11008, M = 1 (2.5 with
-// x_tilde also written where only the image is read, and the library's frexp
-// and ldexp; 5.2 -> 3.8 at 5120 x 5120, M = 8).
+// the fp32 x_tilde written 4 bytes at a time and the library's frexp and ldexp;
+// 5.2 -> 3.8 at 5120 x 5120, M = 8).
 struct DecPrepParams {
   const uint16_t* x;
   const uint16_t* g_hi;
   const uint16_t* g_lo;
-  float* xt;          // M x kpad fp32 (null: not wanted, the image alone)
+  float* xt;          // M x kpad fp32
   uint8_t* bimg;      // B operand image (null: x_tilde only)
   uint8_t* sfbw;      // B scale words, KB x NP x 4 bytes
   float* y_zero;      // cleared (M x n_out) for the decode kernel's atomic split-K, or null
@@ -244,8 +244,9 @@ __global__ void __launch_bounds__(128) prep_decode_kernel(DecPrepParams p) {
     __syncthreads();
   }
 
-  // x_tilde of the tile: to global memory (fp32, where it is asked for) and to
-  // shared memory (the G tiles are no longer read) for the terms below
+  // x_tilde of the tile to shared memory (the G tiles are no longer read), and
+  // from there, or where n_b is no multiple of 64 from the registers, to global
+  // memory
   constexpr int kTld = 72;
   float* tile = reinterpret_cast<float*>(dsm);   // TB x kTld
 #pragma unroll
@@ -254,7 +255,73 @@ __global__ void __launch_bounds__(128) prep_decode_kernel(DecPrepParams p) {
     for (int h = 0; h < 2; ++h)
       *reinterpret_cast<float2*>(tile + (g + 8 * h) * kTld + wcol + n * 8 + 2 * t) =
           make_float2(acc[n][2 * h], acc[n][2 * h + 1]);
-  if (p.xt) {
+  if (p.bimg) {
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // 16 lanes a block's 64 codes
+      const int bl = 8 * h + (tid >> 4), b = b0 + bl, c4 = 4 * (tid & 15);
+      if (b < p.nblk)
+        *reinterpret_cast<float4*>(p.xt + (size_t)m * p.kpad + (int64_t)b * p.n_b + j0 + c4) =
+            *reinterpret_cast<const float4*>(tile + bl * kTld + c4);
+    }
+    // Terms: thread = (block bl of the tile, 32-code group gm of the tile's 64
+    // codes, quarter s4): 8 MMA positions of one 32-position scale group; the
+    // four quarters of a group are consecutive lanes and share its maximum.
+    {
+      const bool ter = p.ternary != 0;
+      const int bl = tid >> 3, gm = (tid >> 2) & 1, s4 = tid & 3, b = b0 + bl;
+      const bool act = b < p.nblk;
+      const int64_t kk0 = (int64_t)b * p.n_b + j0;   // 64-aligned: n_b % 64 == 0
+      const int64_t kb = kk0 >> 7;
+      const int kl0 = (int)(kk0 & 127);
+      const int g8 = (kl0 >> 3) + 4 * gm + s4;
+      float v[8];
+      float mx = 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int kl = decode_stage_k(8 * g8 + i, ter);
+        v[i] = act ? tile[bl * kTld + (kl - kl0)] : 0.f;
+        mx = fmaxf(mx, fabsf(v[i]));
+      }
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+      // mx < 2^E, E - 126 its exponent field, so |v 2^-(E - 2)| < 4
+      const int ex = max(-125, min(126, (int)(__float_as_uint(mx) >> 23) - 128));
+      const float inv = __uint_as_float((uint32_t)(127 - ex) << 23);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] *= inv;
+      if (act) {
+        uint8_t* img = p.bimg + (size_t)(kb >> 1) * p.NP * 128;
+        const int chunk = 4 * (int)(kb & 1) + (g8 >> 2), off = 4 * (g8 & 3);
+        for (int tt = 0; tt < p.T; ++tt) {
+          uint32_t word = 0;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float2 q;
+            word |= e2m1x2(v[2 * i], v[2 * i + 1], &q) << (8 * i);
+            v[2 * i] = (v[2 * i] - q.x) * 8.f;
+            v[2 * i + 1] = (v[2 * i + 1] - q.y) * 8.f;
+          }
+          const int row = m * p.T + tt;
+          *reinterpret_cast<uint32_t*>(img + row * 128 + ((chunk ^ (row & 7)) << 4) + off) = word;
+          if (s4 == 0) p.sfbw[((size_t)kb * p.NP + row) * 4 + (g8 >> 2)] = (uint8_t)max(1, min(254, 127 + ex - 3 * tt));
+        }
+      }
+    }
+    // the K padding (the last block's second half, MMA positions 64..127 =
+    // bytes 32..63 of its 64, when K_eff is an odd number of 64-code halves):
+    // zero terms, unit scales
+    if (jt == 0 && bt == 0 && p.kpad > p.k_eff && tid < 2 * p.T) {
+      const int64_t kb = p.k_eff >> 7;
+      const int tt = tid >> 1, c = 4 * (int)(kb & 1) + 2 + (tid & 1), row = m * p.T + tt;
+      uint8_t* img = p.bimg + (size_t)(kb >> 1) * p.NP * 128;
+      *reinterpret_cast<uint4*>(img + row * 128 + ((c ^ (row & 7)) << 4)) = make_uint4(0, 0, 0, 0);
+      if ((tid & 1) == 0) {
+        p.sfbw[((size_t)kb * p.NP + row) * 4 + 2] = 127;
+        p.sfbw[((size_t)kb * p.NP + row) * 4 + 3] = 127;
+      }
+    }
+  } else {
 #pragma unroll
     for (int n = 0; n < NTW; ++n)
 #pragma unroll
@@ -264,73 +331,14 @@ __global__ void __launch_bounds__(128) prep_decode_kernel(DecPrepParams p) {
       }
   }
   // K padding of this batch row
-  if (p.xt && jt == 0 && bt == 0)
+  if (jt == 0 && bt == 0)
     for (int64_t k = p.k_eff + tid; k < p.kpad; k += 128) p.xt[(size_t)m * p.kpad + k] = 0.f;
-  if (!p.bimg) return;
-  __syncthreads();
-  // Terms: thread = (block bl of the tile, 32-code group gm of the tile's 64
-  // codes, quarter s4): 8 MMA positions of one 32-position scale group; the
-  // four quarters of a group are consecutive lanes and share its maximum.
-  {
-    const bool ter = p.ternary != 0;
-    const int bl = tid >> 3, gm = (tid >> 2) & 1, s4 = tid & 3, b = b0 + bl;
-    const bool act = b < p.nblk;
-    const int64_t kk0 = (int64_t)b * p.n_b + j0;   // 64-aligned: n_b % 64 == 0
-    const int64_t kb = kk0 >> 7;
-    const int kl0 = (int)(kk0 & 127);
-    const int g8 = (kl0 >> 3) + 4 * gm + s4;
-    float v[8];
-    float mx = 0.f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int kl = decode_stage_k(8 * g8 + i, ter);
-      v[i] = act ? tile[bl * kTld + (kl - kl0)] : 0.f;
-      mx = fmaxf(mx, fabsf(v[i]));
-    }
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    // mx < 2^E, E - 126 its exponent field, so |v 2^-(E - 2)| < 4
-    const int ex = max(-125, min(126, (int)(__float_as_uint(mx) >> 23) - 128));
-    const float inv = __uint_as_float((uint32_t)(127 - ex) << 23);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] *= inv;
-    if (act) {
-      uint8_t* img = p.bimg + (size_t)(kb >> 1) * p.NP * 128;
-      const int chunk = 4 * (int)(kb & 1) + (g8 >> 2), off = 4 * (g8 & 3);
-      for (int tt = 0; tt < p.T; ++tt) {
-        uint32_t word = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float2 q;
-          word |= e2m1x2(v[2 * i], v[2 * i + 1], &q) << (8 * i);
-          v[2 * i] = (v[2 * i] - q.x) * 8.f;
-          v[2 * i + 1] = (v[2 * i + 1] - q.y) * 8.f;
-        }
-        const int row = m * p.T + tt;
-        *reinterpret_cast<uint32_t*>(img + row * 128 + ((chunk ^ (row & 7)) << 4) + off) = word;
-        if (s4 == 0) p.sfbw[((size_t)kb * p.NP + row) * 4 + (g8 >> 2)] = (uint8_t)max(1, min(254, 127 + ex - 3 * tt));
-      }
-    }
-  }
-  // the K padding (the last block's second half, MMA positions 64..127 =
-  // bytes 32..63 of its 64, when K_eff is an odd number of 64-code halves):
-  // zero terms, unit scales
-  if (jt == 0 && bt == 0 && p.kpad > p.k_eff && tid < 2 * p.T) {
-    const int64_t kb = p.k_eff >> 7;
-    const int tt = tid >> 1, c = 4 * (int)(kb & 1) + 2 + (tid & 1), row = m * p.T + tt;
-    uint8_t* img = p.bimg + (size_t)(kb >> 1) * p.NP * 128;
-    *reinterpret_cast<uint4*>(img + row * 128 + ((c ^ (row & 7)) << 4)) = make_uint4(0, 0, 0, 0);
-    if ((tid & 1) == 0) {
-      p.sfbw[((size_t)kb * p.NP + row) * 4 + 2] = 127;
-      p.sfbw[((size_t)kb * p.NP + row) * 4 + 3] = 127;
-    }
-  }
 }
 
 }  // namespace
 
 cudaError_t launch_prep(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws, cudaStream_t st, float* y_zero,
-                        bool forward) {
+                        bool keep_xt) {
   const Geometry& g = pl->geo;
   const WsLayout L = workspace_layout(pl, M);
   uint8_t* base = static_cast<uint8_t*>(ws);
@@ -340,7 +348,7 @@ cudaError_t launch_prep(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws
     DecPrepParams p;
     p.x = x; p.g_hi = pl->d_g_hi; p.g_lo = pl->d_g_lo;
     p.bimg = decode_image(pl) ? base + L.bimg : nullptr;
-    p.xt = forward && p.bimg ? nullptr : reinterpret_cast<float*>(base + L.xt);
+    p.xt = reinterpret_cast<float*>(base + L.xt);
     p.sfbw = base + L.sfbw;
     p.T = dc.T; p.NP = dc.NP;
     p.y_zero = y_zero;
@@ -359,7 +367,7 @@ cudaError_t launch_prep(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws
     return launch_pdl(prep_decode_kernel, grid, dim3(128), smem, st, p);
   }
   bool used = false;
-  cudaError_t et = launch_prep_tc(pl, x, M, ws, st, &used, M <= kMaxDecodeM && !forward);
+  cudaError_t et = launch_prep_tc(pl, x, M, ws, st, &used, M <= kMaxDecodeM && keep_xt);
   if (et != cudaSuccess || used) return et;
   PrepParams p;
   p.x = x; p.g_hi = pl->d_g_hi; p.g_lo = pl->d_g_lo;

@@ -51,3 +51,19 @@ def test_wide_decode(sdq, q, m, n, k, b, osr):
     bound = EB.forward_bound(xf, codes, alpha, b, d.n_b, signs, T=3)
     EB.check(y.cpu().numpy(), yr, bound, "forward")
     assert np.abs(y2.cpu().numpy() - 2 * y.cpu().numpy()).max() <= 2e-5 * np.abs(yr).max()
+
+
+@pytest.mark.parametrize("m", [1, 5, 40, 64])
+def test_read_prep_after_forward(sdq, m):
+    import torch
+    n, k, b = 256, 896, 128
+    plan = sdq.Plan(sdq.LayerDesc(n, k, b, Fraction(5, 2), O.TERNARY, 1, 0))
+    bits = W.float_to_bf16(np.random.default_rng(m).standard_normal((m, k)).astype(np.float32))
+    x = torch.from_numpy(bits.view(np.int16)).view(torch.bfloat16).cuda()
+    ws = plan.alloc_workspace(m)
+    ws.fill_(0xFF)
+    plan.forward(plan.alloc_tiled().zero_(), torch.ones(n, device="cuda"), x, ws=ws)
+    xt = torch.empty((m, plan.k_eff), dtype=torch.float32, device="cuda")
+    sdq.sdq_read_prep(plan.handle, m, ws, xt)
+    want = O.prep_activations(W.bf16_to_float(bits), b, b * 5 // 2, None)
+    assert np.abs(xt.cpu().numpy() - want).max() < 2e-5 * np.abs(want).max()
