@@ -728,6 +728,39 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
           acc += sum[i];
           if (++t == p.T) { emit(m, acc); acc = 0.f; t = 0; ++m; }
         }
+      } else if (np == 1) {
+        // one pipeline: a running sum, and more columns per wait (each wait
+        // is about 0.3 us of the tail: 125M layer, M = 16, 38.2 -> 35.2 us)
+        auto terms1 = [&](auto tc) {
+          constexpr int T = decltype(tc)::value, kCh = T == 4 ? 32 : 24;   // whole rows
+          const uint32_t at = lq + (uint32_t)(p.dbase + (kc[0] % p.nbuf) * p.NP);
+          int m = 0;
+#pragma unroll 1
+          for (int c0 = 0; c0 < MT; c0 += kCh) {
+            uint32_t rr[kCh / 8][8];
+#pragma unroll
+            for (int h = 0; h < kCh / 8; ++h)   // (inside the NP columns)
+              tmem_ld8(at + (uint32_t)min(c0 + 8 * h, p.NP - 8), rr[h]);
+            tmem_ld_wait();
+            if (c0 + kCh >= MT) {
+              tc_fence_before();
+              mbar_arrive(&acc_empty[0][kc[0] % p.nbuf]);
+            }
+            float acc = 0.f;
+#pragma unroll
+            for (int i = 0; i < kCh; ++i) {
+              acc += __uint_as_float(rr[i / 8][i % 8]);
+              if (i % T == T - 1) {
+                emit(m, acc);   // (rows past the last: not written)
+                acc = 0.f;
+                ++m;
+              }
+            }
+          }
+        };
+        if (p.T == 3) terms1(std::integral_constant<int, 3>());
+        else if (p.T == 4) terms1(std::integral_constant<int, 4>());
+        else terms1(std::integral_constant<int, 6>());
       } else {
         // many batch rows: 16 kSub columns hold whole rows, so where each
         // row's terms end is known at compile time and the sums stay in
@@ -943,7 +976,8 @@ DecodeConfig decode_config_search(const sdq_plan_s* pl, int M) {
             // beside the next tile's MMAs with two accumulators, else between
             const double t_stream = tile_bytes / rate;
             const double t_tile = nbuf == 2 ? std::max(t_stream, t_epi[pi]) : t_stream + t_epi[pi];
-            const double t_cta = units * (t_tile + 0.3e-6 + 0.1e-6 * np + 0.1e-6 * S);
+            const double t_cta = units * (t_tile + 0.3e-6 + 0.1e-6 * np + 0.1e-6 * S) +
+                                 (nbuf == 2 ? t_epi[pi] : 0.0);   // (the last tile's hides behind nothing)
             const double t = waves * t_cta + t_build + t_tail;
             if (t < best_t * 0.999) {
               best_t = t;
