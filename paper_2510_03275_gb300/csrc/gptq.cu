@@ -3,8 +3,10 @@
 // (2 X X^T + lambda I)^-1 given through its upper Cholesky factor U,
 // U^T U = H^-1).
 //
-// Blocks are encoded in order on a working copy of W.  After block b is
-// encoded (encode_kernel, one block per launch), each row's block error E =
+// Blocks are encoded in order on a working copy of W: by the row-owner kernel
+// (second half of this file) where it applies, else with encode_kernel and
+// gptq_update_kernel, a launch of each per block.  After block b is encoded,
+// each row's block error E =
 // W_F - alpha (c . G) is normalised by the factor's diagonal block, E~ =
 // E U_FF^-1, and the later columns take the update W_R -= E~ U_FR: the exact
 // block update of GPTQ / optimal brain surgeon (for B = 1 it is GPTQ's
@@ -119,15 +121,15 @@ __global__ void __launch_bounds__(kUpThreads, 2)
 //              returns 512 bytes to its warp, 4 cycles of the SM's one
 //              shared-memory pipe: with 2 columns x all rows a thread that pipe
 //              was as busy as the multiplies and adds
-// The update's multiplies and adds bound it (no FMA: both are rounded), 165 of
-// 228 k cycles a block of a 4096 x 4096 layer (100 + 8 at their issue rate, 133
+// The update's multiplies and adds bound it (no FMA: both are rounded), 155 of
+// 218 k cycles a block of a 4096 x 4096 layer (100 + 8 at their issue rate, 133
 // with every load of U an L1 hit); the steps before it are chains of dependent
 // operations.  Two teams of rows per CTA, one's chains beside the other's
 // update, took 330 k: single warps a quadrant wait on their own latencies.
 // CTAs start at different column chunks: in step they all ask the same few L2
 // lines at once (88 -> 72 k cycles a block of updates for 8 rows).  The launch
 // per block and per update that this replaces took 12.6 ms for that layer, this
-// 4.0; 2560 x 3584, B = 256, OSR 3: 21 and 4.8.
+// 3.8; 2560 x 3584, B = 256, OSR 3: 21 and 4.8.
 // W_F and W_R come from W itself at block 0 and from the working copy after
 // it; the values and their order are those of a launch per block.
 constexpr int kGqThreads = 256;
@@ -411,6 +413,10 @@ __global__ void __launch_bounds__(kGqThreads, 1) gptq_rows_kernel(GptqParams p) 
         constexpr int kN = decltype(rows)::value;
         constexpr int kD = kN > 4 ? 8 : 16;   // rows of U in flight: the L2's round trip under this load is over 1000 cycles
         auto get = [](const float4& v, int c) { return reinterpret_cast<const float*>(&v)[c]; };
+        const float* wr = (b == 0 ? p.W : p.wc) + (size_t)(row0 + r0) * p.k_in + ca;
+#pragma unroll
+        for (int r = 0; r < kN; ++r)   // into the L2 by the time they are read
+          if (r0 + r < nr) asm volatile("prefetch.global.L2 [%0];" ::"l"(wr + (size_t)r * p.k_in));
         const float* u0 = uf + ca;
         float acc[4][kN];
         float4 u[kD];
@@ -443,17 +449,26 @@ __global__ void __launch_bounds__(kGqThreads, 1) gptq_rows_kernel(GptqParams p) 
             u[i] = __ldg(reinterpret_cast<const float4*>(u0 + (size_t)i * step));
           }
         }
-        const float* wr = (b == 0 ? p.W : p.wc) + (size_t)(row0 + r0) * p.k_in + ca;
         float* wo = p.wc + (size_t)(row0 + r0) * p.k_in + ca;
+        // four rows' loads before their stores: a round trip per four rows, not
+        // one per row (8192 x 8192: 29.2 ms, 26.0 so, 25.5 with the prefetch above;
+        // all rows' loads first cost the loop above registers: 158 k cycles a block
+        // against 149)
 #pragma unroll
-        for (int r = 0; r < kN; ++r) {
-          if (r0 + r >= nr) break;
-          float4 w = __ldcg(reinterpret_cast<const float4*>(wr + (size_t)r * p.k_in));
-          w.x = __fsub_rn(w.x, acc[0][r]);
-          w.y = __fsub_rn(w.y, acc[1][r]);
-          w.z = __fsub_rn(w.z, acc[2][r]);
-          w.w = __fsub_rn(w.w, acc[3][r]);
-          *reinterpret_cast<float4*>(wo + (size_t)r * p.k_in) = w;
+        for (int r4 = 0; r4 < kN; r4 += 4) {
+          float4 w[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (r0 + r4 + r < nr) w[r] = __ldcg(reinterpret_cast<const float4*>(wr + (size_t)(r4 + r) * p.k_in));
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            if (r0 + r4 + r >= nr) break;
+            w[r].x = __fsub_rn(w[r].x, acc[0][r4 + r]);
+            w[r].y = __fsub_rn(w[r].y, acc[1][r4 + r]);
+            w[r].z = __fsub_rn(w[r].z, acc[2][r4 + r]);
+            w[r].w = __fsub_rn(w[r].w, acc[3][r4 + r]);
+            *reinterpret_cast<float4*>(wo + (size_t)(r4 + r) * p.k_in) = w[r];
+          }
         }
       };
       // 512 columns at a time, the first kN0 rows by warps 0-3 and the others by
