@@ -199,7 +199,9 @@ size_t sdq_gptq_workspace_bytes(sdq_plan plan);
  * acc = fl(...fl(fl(E~_0 U_0c) + fl(E~_1 U_1c))...) in ascending k and
  * W = fl(W - acc).  E~ U_FR is the exact block update E H_FR H_RR^-1 (the
  * printed update E H^-1_{F,R} read with GPTQ's normalisation by the factor's
- * diagonal block).  Requires B a multiple of 4; 2 nblk launches on `stream`.
+ * diagonal block).  Requires B a multiple of 4.  Two kernels on `stream` for B
+ * 64, 128 and 256 (alpha, then the block loop with every row's blocks in one
+ * thread block; csrc/gptq.cu says where it applies), else 2 nblk launches.
  * Pointers 16-byte aligned; SDQ_ERR_WORKSPACE if ws_bytes is below
  * sdq_gptq_workspace_bytes; SDQ_ERR_UNSUPPORTED for B not a multiple of 4. */
 int sdq_encode_rows_gptq(sdq_plan plan, const float* W, const float* U, uint32_t* codes_plain,
@@ -324,7 +326,8 @@ int sdq_forward_route(sdq_plan plan, int32_t M);
 int sdq_workspace_status(sdq_plan plan, int32_t M, const void* ws, void* stream);
 
 /* Copy x_tilde for M <= 64 out of the workspace as fp32 (M x K_eff,
- * device), for checking sdq_prep_activations. */
+ * device), for checking sdq_prep_activations (sdq_linear_forward leaves it
+ * too where ws_bytes was at least sdq_workspace_bytes). */
 int sdq_read_prep(sdq_plan plan, int32_t M, const void* ws, float* xt_out, void* stream);
 
 /* Allocation-free decode forward, for callers that may not allocate device

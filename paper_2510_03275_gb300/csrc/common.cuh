@@ -97,10 +97,6 @@ cudaError_t smem_limit_once(Kern kernel, int bytes, int device, std::atomic<int>
 }
 
 // ------------------------------------------------------------------ device
-__device__ __forceinline__ float bf16_bits_to_float(uint16_t b) {
-  return __uint_as_float((uint32_t)b << 16);
-}
-
 // Round-to-nearest-even fp32 -> bf16 bits (finite inputs).
 __device__ __forceinline__ uint16_t float_to_bf16_bits(float f) {
   uint32_t u = __float_as_uint(f);

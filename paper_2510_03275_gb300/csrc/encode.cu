@@ -15,10 +15,10 @@
 // Sigma-Delta recursion of eq. (8) over their row, reset at every block, and
 // write the codes in the plain packed layout.
 //
-// The kernel covers a range of passes and blocks.  The encoder with GPTQ
-// block compensation (Algorithm 1's outer loop with the inverse Hessian)
-// runs pass 1 one block at a time on a working copy of W: after the scan,
-// the warp rebuilds the block Q = alpha (c . G), forms E = W_F - Q and the
+// The kernel covers a range of passes and blocks.  Where the encoder with GPTQ
+// block compensation (Algorithm 1's outer loop with the inverse Hessian) has
+// no kernel of its own for a layer (csrc/gptq.cu), it runs pass 1 here one
+// block at a time on a working copy of W: after the scan, the warp rebuilds the block Q = alpha (c . G), forms E = W_F - Q and the
 // normalised error E~ = E U_FF^-1 (forward substitution over the block's
 // columns), which gptq_update_kernel then applies to the later columns.
 #include <algorithm>
