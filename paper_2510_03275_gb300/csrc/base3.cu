@@ -16,7 +16,7 @@
 // words a lane: an odd stride, no bank conflicts), and its base-3 bytes 512.
 // Persistent blocks: the table is filled once, and a warp's next loads are in
 // flight while it converts.  28672 x 16384 codes (211 MB in and out, 31 us at
-// the copy rate): 52 us either way, from 82 us with one table per block and a
+// the copy rate): 45 us either way, from 82 us with one table per block and a
 // word or byte group per thread.
 #include <algorithm>
 
@@ -37,6 +37,7 @@ constexpr int kB3BlocksPerSm = 4;     // 42 KB of shared memory each, 64 registe
 
 struct Base3Params {
   int n_out, wpr, bpr, gpr, rpr;   // plain words / base-3 bytes / groups / runs per row
+  int srow, sseg;                  // a step in rows and runs: all warps' runs
   int64_t k_eff, total;            // total = n_out * rpr runs
 };
 
@@ -81,13 +82,35 @@ __device__ __forceinline__ uint32_t below_k_eff(uint32_t w, int64_t first, int64
   return keep >= 16 ? w : (keep <= 0 ? 0u : w & ((1u << (2 * keep)) - 1u));
 }
 
-// Row and run within the row of a run (past the last one: row 0, run rpr,
-// which has nothing to read or write).
-__device__ __forceinline__ void run_place(const Base3Params& p, int64_t run, int64_t& row, int& seg) {
-  const bool v = run < p.total;
-  row = v ? run / p.rpr : 0;
-  seg = v ? (int)(run - row * p.rpr) : p.rpr;
-}
+// A warp's next kB3Runs runs: row and run within the row (past the last row:
+// row 0, run rpr, which has nothing to read or write).  Stepped without a
+// division: a 64-bit one per run was 50 of the 254 instructions a thread
+// issued per 80 codes, which bound both kernels (52 us for the layer above, 45
+// so).
+struct RunPlace {
+  uint32_t row;
+  int seg;
+  __device__ __forceinline__ RunPlace(const Base3Params& p, int64_t run0)
+      : row((uint32_t)(run0 / p.rpr)), seg((int)(run0 - (int64_t)row * p.rpr)) {}
+  __device__ __forceinline__ void place(const Base3Params& p, int u, uint32_t& r, int& sg) const {
+    const bool wrap = seg + u >= p.rpr;   // u <= 1
+    r = row + (wrap ? 1u : 0u);
+    sg = seg + u - (wrap ? p.rpr : 0);
+    if (r >= (uint32_t)p.n_out) {
+      r = 0u;
+      sg = p.rpr;
+    }
+  }
+  __device__ __forceinline__ void next(const Base3Params& p) {
+    row += (uint32_t)p.srow;
+    seg += p.sseg;
+    if (seg >= p.rpr) {
+      seg -= p.rpr;
+      ++row;
+    }
+  }
+};
+static_assert(kB3Runs == 2, "RunPlace wraps once");
 
 // A warp's step is kB3Runs runs: a run is 32 groups (160 plain words, 512
 // base-3 bytes) of one row, lane = group.  gpr = bpr / 16.
@@ -98,23 +121,25 @@ __global__ void __launch_bounds__(kB3Threads) pack_base3_kernel(const uint32_t* 
   uint32_t(*stage)[kB3Words] = reinterpret_cast<uint32_t(*)[kB3Words]>(b3_smem + kB3Table) + kB3Runs * warp;
   const uint8_t* mine = reinterpret_cast<const uint8_t*>(b3_smem + lane);   // this lane's copy, 128 bytes a word
   const int64_t step = (int64_t)gridDim.x * kB3Warps * kB3Runs;
+  int64_t run0 = ((int64_t)blockIdx.x * kB3Warps + warp) * kB3Runs;
+  RunPlace at(p, run0);
   const int n4 = p.wpr / 4;
-  int64_t row[kB3Runs];
+  uint32_t row[kB3Runs];
   int seg[kB3Runs];
   uint4 a[kB3Runs], b[kB3Runs];
-  auto load = [&](int64_t run0) {
+  auto load = [&]() {
 #pragma unroll
     for (int u = 0; u < kB3Runs; ++u) {
-      run_place(p, run0 + u, row[u], seg[u]);
-      const uint4* src = reinterpret_cast<const uint4*>(plain + row[u] * p.wpr);
+      at.place(p, u, row[u], seg[u]);
+      const uint4* src = reinterpret_cast<const uint4*>(plain + (int64_t)row[u] * p.wpr);
       const int i = seg[u] * (kB3Words / 4) + lane;
       a[u] = b[u] = make_uint4(0u, 0u, 0u, 0u);
       if (seg[u] < p.rpr && i < n4) a[u] = __ldcs(src + i);
       if (seg[u] < p.rpr && lane < 8 && i + 32 < n4) b[u] = __ldcs(src + i + 32);
     }
+    at.next(p);
   };
-  int64_t run0 = ((int64_t)blockIdx.x * kB3Warps + warp) * kB3Runs;
-  load(run0);
+  load();
   {
     uint32_t w = 0;   // table word i: the bytes of the field patterns 4 i .. 4 i + 3
 #pragma unroll
@@ -122,7 +147,7 @@ __global__ void __launch_bounds__(kB3Threads) pack_base3_kernel(const uint32_t* 
     fill_table(b3_smem, w);
   }
   for (; run0 < p.total; run0 += step) {
-    int64_t r[kB3Runs];
+    uint32_t r[kB3Runs];
     int sg[kB3Runs];
 #pragma unroll
     for (int u = 0; u < kB3Runs; ++u) {
@@ -133,7 +158,7 @@ __global__ void __launch_bounds__(kB3Threads) pack_base3_kernel(const uint32_t* 
       sg[u] = seg[u];
     }
     __syncwarp();
-    load(run0 + step);
+    load();
 #pragma unroll
     for (int u = 0; u < kB3Runs; ++u) {
       const int g = sg[u] * 32 + lane;
@@ -163,7 +188,7 @@ __global__ void __launch_bounds__(kB3Threads) pack_base3_kernel(const uint32_t* 
         }
         o[k] = __byte_perm(__byte_perm(y[0], y[1], 0x0040), __byte_perm(y[2], y[3], 0x0040), 0x5410);
       }
-      *reinterpret_cast<uint4*>(out + r[u] * p.bpr + 16 * g) = make_uint4(o[0], o[1], o[2], o[3]);
+      *reinterpret_cast<uint4*>(out + (int64_t)r[u] * p.bpr + 16 * g) = make_uint4(o[0], o[1], o[2], o[3]);
     }
     __syncwarp();
   }
@@ -182,26 +207,28 @@ __global__ void __launch_bounds__(kB3Threads) unpack_base3_kernel(const uint8_t*
   const uint8_t* table = reinterpret_cast<const uint8_t*>(b3_smem);
   const uint32_t lane4 = 4u * lane;
   const int64_t step = (int64_t)gridDim.x * kB3Warps * kB3Runs;
+  int64_t run0 = ((int64_t)blockIdx.x * kB3Warps + warp) * kB3Runs;
+  RunPlace at(p, run0);
   const int n4 = p.wpr / 4;
-  int64_t row[kB3Runs];
+  uint32_t row[kB3Runs];
   int seg[kB3Runs];
   uint4 raw[kB3Runs];
-  auto load = [&](int64_t run0) {
+  auto load = [&]() {
 #pragma unroll
     for (int u = 0; u < kB3Runs; ++u) {
-      run_place(p, run0 + u, row[u], seg[u]);
+      at.place(p, u, row[u], seg[u]);
       const int g = seg[u] * 32 + lane;
       raw[u] = make_uint4(0u, 0u, 0u, 0u);
       if (seg[u] < p.rpr && 16 * g < p.bpr)
-        raw[u] = __ldcs(reinterpret_cast<const uint4*>(in + row[u] * p.bpr + 16 * g));
+        raw[u] = __ldcs(reinterpret_cast<const uint4*>(in + (int64_t)row[u] * p.bpr + 16 * g));
     }
+    at.next(p);
   };
-  int64_t run0 = ((int64_t)blockIdx.x * kB3Warps + warp) * kB3Runs;
-  load(run0);
+  load();
   fill_table(b3_smem, byte_fields(threadIdx.x));
   int nbad = 0;
   for (; run0 < p.total; run0 += step) {
-    int64_t r[kB3Runs];
+    uint32_t r[kB3Runs];
     int sg[kB3Runs];
     uint4 x4[kB3Runs];
 #pragma unroll
@@ -210,15 +237,17 @@ __global__ void __launch_bounds__(kB3Threads) unpack_base3_kernel(const uint8_t*
       r[u] = row[u];
       sg[u] = seg[u];
     }
-    load(run0 + step);
+    load();
 #pragma unroll
     for (int u = 0; u < kB3Runs; ++u) {
       const uint32_t xw[4] = {x4[u].x, x4[u].y, x4[u].z, x4[u].w};
+      const uint32_t inv[4] = {invalid_bytes(xw[0]), invalid_bytes(xw[1]), invalid_bytes(xw[2]), invalid_bytes(xw[3])};
+      if (inv[0] | inv[1] | inv[2] | inv[3])
+        nbad += __popc(inv[0]) + __popc(inv[1]) + __popc(inv[2]) + __popc(inv[3]);
       uint32_t w[5] = {0u, 0u, 0u, 0u, 0u};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const uint32_t x = xw[k], inv = invalid_bytes(x);
-        if (inv) nbad += __popc(inv);
+        const uint32_t x = xw[k];
 #pragma unroll
         for (int j = 0; j < 4; j += 2) {
           // table words of bytes j, j + 1: 128 bytes apart, this lane's copy
@@ -242,7 +271,7 @@ __global__ void __launch_bounds__(kB3Threads) unpack_base3_kernel(const uint8_t*
 #pragma unroll
     for (int u = 0; u < kB3Runs; ++u) {
       if (sg[u] >= p.rpr) continue;
-      uint4* dst = reinterpret_cast<uint4*>(plain + r[u] * p.wpr);
+      uint4* dst = reinterpret_cast<uint4*>(plain + (int64_t)r[u] * p.wpr);
       const uint4* st = reinterpret_cast<const uint4*>(stage[u]);
       const int i = sg[u] * (kB3Words / 4) + lane;
       if (i < n4) dst[i] = st[lane];
@@ -262,6 +291,9 @@ Base3Params base3_params(const sdq_plan_s* pl, int bpr, int gpr, int64_t* blocks
   bp.k_eff = g.k_eff; bp.total = (int64_t)g.n_out * bp.rpr;
   *blocks = std::min((bp.total + kB3Warps * kB3Runs - 1) / (kB3Warps * kB3Runs),
                      (int64_t)kB3BlocksPerSm * std::max(1, pl->sm_count));
+  const int64_t step = *blocks * kB3Warps * kB3Runs;
+  bp.srow = (int)(step / bp.rpr);
+  bp.sseg = (int)(step - (int64_t)bp.srow * bp.rpr);
   return bp;
 }
 

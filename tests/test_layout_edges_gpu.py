@@ -2,7 +2,7 @@
 against the oracle: rows around a 128-row tile, group counts around a block's
 8 groups (plain <-> tiled), and rows around one and several runs of 32 groups
 of 80 codes (plain <-> base-3), with more runs than one step of the persistent
-grid in the last case."""
+grid (1, 2 and 6 runs a row) in the last cases."""
 from fractions import Fraction
 
 import numpy as np
@@ -42,7 +42,8 @@ def test_pack_unpack_tile_edges(sdq, torch_cuda, q, n, keff):
     assert torch.equal(back, plain) and int(bad.item()) == 0
 
 
-@pytest.mark.parametrize("n,keff", [(3, 2496), (5, 2560), (2, 2624), (9, 5184), (1, 64), (6500, 2624)])
+@pytest.mark.parametrize("n,keff", [(3, 2496), (5, 2560), (2, 2624), (9, 5184), (1, 64), (6500, 2624),
+                                    (20001, 64), (2001, 12864)])
 def test_base3_run_edges(sdq, torch_cuda, n, keff):
     torch = torch_cuda
     plan = sdq.Plan(sdq.LayerDesc(n, keff, 64, Fraction(1), O.TERNARY))
