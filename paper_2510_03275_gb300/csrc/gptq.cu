@@ -207,11 +207,17 @@ __global__ void __launch_bounds__(kGqThreads, 1) gptq_rows_kernel(GptqParams p) 
         }
         cp_async_commit();
       };
-      stage_u(ub, 0);
-      if (tid < kB) {   // (kB at most kGqThreads)
-        const float d = __ldg(uff + (size_t)tid * ldu + tid);
-        dg[tid] = d;
-        dg[kB + tid] = fabsf(d) >= 0x1p-30f && fabsf(d) <= 0x1p30f ? __frcp_rn(d) : 0.f;
+      // The last block has no solve: staged for it too, the copies would still be
+      // in flight when the next group of rows stages its first into the same rows
+      // (asynchronous copies keep no order among them).
+      const bool later = b != p.nblk - 1;
+      if (later) {
+        stage_u(ub, 0);
+        if (tid < kB) {   // (kB at most kGqThreads)
+          const float d = __ldg(uff + (size_t)tid * ldu + tid);
+          dg[tid] = d;
+          dg[kB + tid] = fabsf(d) >= 0x1p-30f && fabsf(d) <= 0x1p30f ? __frcp_rn(d) : 0.f;
+        }
       }
       // the rows' weights, each warp a part of its 8 rows' columns
       if (hw < kHw) {
@@ -245,7 +251,6 @@ __global__ void __launch_bounds__(kGqThreads, 1) gptq_rows_kernel(GptqParams p) 
       __syncthreads();
       // The last warp scans in up to 4 parts; the other warps rebuild a part
       // while it scans the next ones.
-      const bool later = b != p.nblk - 1;   // there are later columns
       const int part = (p.n_b + 127) / 128 * 32;
       const int nmine = (nr + 3) / 4, scan_bar = 32 * (min(nmine, kGqThreads / 32 - 1) + 1);
       if (warp == kGqThreads / 32 - 1) {

@@ -1,0 +1,41 @@
+"""Rules of the kernels' asynchronous copies, waits and barriers that no run
+shows (a broken one corrupts memory or hangs only when the timing is bad),
+checked on the kernels' source text."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2510_03275_gb300", "csrc")
+
+
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def _block(text, start):
+    """The brace block that begins at or after `start`: (first, last + 1)."""
+    i = text.index("{", start)
+    depth = 0
+    for j in range(i, len(text)):
+        depth += (text[j] == "{") - (text[j] == "}")
+        if depth == 0:
+            return i, j + 1
+    raise AssertionError("unbalanced braces")
+
+
+def _kernel(text, name):
+    start = text.index(f" {name}(")
+    a, b = _block(text, start)
+    return text[a:b]
+
+
+def test_gptq_block_loop_leaves_no_copy_behind():
+    """Leaving the block loop early waits for nothing, so every copy staged
+    before that exit is under the condition that the exit is not taken."""
+    k = _kernel(_source("gptq.cu"), "gptq_rows_kernel")
+    end = k.index("if (!later) break;")
+    calls = [m.start() for m in re.finditer(r"stage_u\(\w+, \d", k[:end])]
+    assert calls
+    guarded = [_block(k, m.end()) for m in re.finditer(r"if \(later\) (?=\{)", k[:end])]
+    for c in calls:
+        assert any(a < c < b for a, b in guarded), k[c:c + 20]
