@@ -454,6 +454,16 @@ __device__ __forceinline__ void named_bar_arrive(int id, int nthreads) {
   asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// Barrier over `nthreads` threads that also ANDs a predicate across them.
+__device__ __forceinline__ bool group_and(int id, int nthreads, bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, %2, %3, p;\n"
+      " selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r) : "r"((uint32_t)v), "r"(id), "r"(nthreads) : "memory");
+  return r != 0;
+}
+
 // Call record in the workspace: word 0 = tag of the last call that gave up a
 // bounded wait, word 1 = tag of the last call that ran.  Tags (call_tag in
 // capi.cu) are 48-bit values with bit 47 set, distinct for 2^47 calls and

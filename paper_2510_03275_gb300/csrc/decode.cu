@@ -142,16 +142,6 @@ struct DecodeParams {
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity));
 }
-// Barrier over `nthreads` threads that also ANDs a predicate across them.
-__device__ __forceinline__ bool group_and(int id, int nthreads, bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, %2, %3, p;\n"
-      " selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r) : "r"((uint32_t)v), "r"(id), "r"(nthreads) : "memory");
-  return r != 0;
-}
-
 // Stage j of a row tile (spu stages over the chunk's ncb blocks) covers
 // blocks [first, last).
 __device__ __forceinline__ int stage_block(int j, int ncb, int spu) { return j * ncb / spu; }

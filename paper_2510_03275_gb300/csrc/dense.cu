@@ -196,7 +196,9 @@ __global__ void __launch_bounds__(kRbThreads, 1)
     int n = 0;   // halves stored
     for (int it = 0; it < nmine && ok; ++it) {
       const int a = it & 1;
-      ok = mbar_wait_warp(&acc_full[a], (it >> 1) & 1);
+      // one outcome for the four warps: one that gave up alone would leave the
+      // others in the barriers below for good
+      ok = group_and(2, 128, mbar_wait_warp(&acc_full[a], (it >> 1) & 1));
       if (!ok) break;
       tc_fence_after();
       const int item = (int)blockIdx.x + it * (int)gridDim.x;

@@ -39,3 +39,21 @@ def test_gptq_block_loop_leaves_no_copy_behind():
     guarded = [_block(k, m.end()) for m in re.finditer(r"if \(later\) (?=\{)", k[:end])]
     for c in calls:
         assert any(a < c < b for a, b in guarded), k[c:c + 20]
+
+
+def test_barriers_behind_bounded_waits_are_reached_together():
+    """A loop that leaves on its own bounded wait's outcome and has a barrier of
+    several warps takes one outcome for all of them first: a warp that gave up
+    alone would leave the others in the barrier for good."""
+    seen = 0
+    for name in sorted(f for f in os.listdir(CSRC) if f.endswith(".cu")):
+        text = _source(name)
+        for m in re.finditer(r"\bfor \([^{;]*;[^{;]*;[^{;\n]*\) \{[ \t]*$", text, re.M):
+            a, b = _block(text, m.end() - 1)
+            body = text[a:b]
+            bar, wait = body.find("named_bar_sync("), re.search(r"\b(mbar_wait|mbar_wait_warp|warp_wait)\(", body)
+            if bar < 0 or not wait or wait.start() > bar:
+                continue
+            seen += 1
+            assert "group_and(" in body[:bar], f"{name}: {m.group(0)}"
+    assert seen
