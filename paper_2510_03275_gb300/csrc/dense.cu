@@ -26,8 +26,8 @@
 // (or 2 x 256) weight rows x up to 256 batch rows, both operands TMA-loaded
 // (128-byte swizzle), 6 (4) stages; epilogue as K5's.
 // Every wait on an mbarrier is bounded (about 2 s); a timeout writes the call
-// number into the workspace's call record and the CTA finishes without
-// further waits.
+// number into the workspace's call record and the CTA waits (again bounded)
+// for its own copies and MMAs before it frees TMEM and ends.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kRbThreads, 1)
                  const __grid_constant__ CUtensorMap wmap, ReconParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t g_full, full[kRbStages], empty[kRbStages], a_full[kRbStages],
-      acc_full[2], acc_empty[2];
+      acc_full[2], acc_empty[2], mma_done;
   __shared__ uint32_t tmem_base;
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(kRbThreads, 1)
 
   if (tid == 0) {
     mbar_init(&g_full, 1);
+    mbar_init(&mma_done, 1);
     for (int s = 0; s < kRbStages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
@@ -114,8 +115,9 @@ __global__ void __launch_bounds__(kRbThreads, 1)
       tma_load_2d_warp(base + c * gchunk, &ghmap, c * kBK, 0, &g_full);
       tma_load_2d_warp(base + (spb + c) * gchunk, &glmap, c * kBK, 0, &g_full);
     }
-    for (int i = 0; i < nst && ok; ++i) {
-      const int s = i % kRbStages, r = i / kRbStages;
+    int n = 0;   // slabs copied
+    for (; n < nst; ++n) {
+      const int i = n, s = i % kRbStages, r = i / kRbStages;
       const int item = (int)blockIdx.x + (i / spb) * (int)gridDim.x, sc = i % spb;
       const int tile = item / p.nblk, b = item - tile * p.nblk;
       if (r > 0) ok = mbar_wait_warp(&empty[s], (r - 1) & 1);
@@ -124,6 +126,10 @@ __global__ void __launch_bounds__(kRbThreads, 1)
       const uint32_t* src = p.codes + (size_t)((int64_t)tile * p.ngroups + b * spb + sc) * (slab_bytes / 4);
       bulk_g2s_warp(c_tiles + s * kRbCTile, src, slab_bytes, &full[s]);
     }
+    // every copy issued has landed before the CTA ends
+    if (!mbar_wait_warp(&g_full, 0)) ok = false;
+    for (int j = max(0, n - kRbStages); j < n; ++j)
+      if (!mbar_wait_warp(&full[j % kRbStages], (j / kRbStages) & 1)) ok = false;
   } else if (warp == 1) {
     constexpr uint32_t idesc = f16_idesc(128);
     ok = mbar_wait_warp(&g_full, 0);
@@ -149,6 +155,8 @@ __global__ void __launch_bounds__(kRbThreads, 1)
       umma_commit_warp(&empty[s]);
       if (sc == spb - 1) umma_commit_warp(&acc_full[a]);
     }
+    umma_commit_warp(&mma_done);   // ... and every MMA is done before TMEM is freed
+    if (!mbar_wait_warp(&mma_done, 0)) ok = false;
   } else if (warp < kRbEpiWarp0) {
     // Expanders: set x = (warp - 2) / 4 expands stages i = x (mod 2), thread
     // = code row 32 q + lane (q = warp % 4): 64 codes -> 32 TMEM columns.

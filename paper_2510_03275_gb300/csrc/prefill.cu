@@ -420,7 +420,8 @@ __global__ void __launch_bounds__(kPtThreads, 1)
     prep_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap ghmap,
                    const __grid_constant__ CUtensorMap glmap, PrepTcParams p) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t g_full, x_full[kPtMaxSlots], x_empty[kPtMaxSlots], acc_full[2], acc_empty[2];
+  __shared__ __align__(8) uint64_t g_full, x_full[kPtMaxSlots], x_empty[kPtMaxSlots], acc_full[2], acc_empty[2],
+      mma_done;
   __shared__ uint32_t tmem_base;
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31, j0 = (int)blockIdx.y * p.ncol;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -432,6 +433,7 @@ __global__ void __launch_bounds__(kPtThreads, 1)
 
   if (tid == 0) {
     mbar_init(&g_full, 1);
+    mbar_init(&mma_done, 1);
     for (int s = 0; s < kPtMaxSlots; ++s) {
       mbar_init(&x_full[s], 1);
       mbar_init(&x_empty[s], 1);
@@ -503,6 +505,8 @@ __global__ void __launch_bounds__(kPtThreads, 1)
       }
       if (ok) umma_commit_warp(&acc_full[a]);
     }
+    umma_commit_warp(&mma_done);   // every MMA is done before TMEM is freed
+    if (!mbar_wait_warp(&mma_done, 0)) ok = false;
   } else {
     pdl_wait();   // the workspace belongs to the preceding grid until then
     const int et = tid - 64, q = warp & 3, half = (warp - 2) >> 2;

@@ -57,3 +57,39 @@ def test_barriers_behind_bounded_waits_are_reached_together():
             seen += 1
             assert "group_and(" in body[:bar], f"{name}: {m.group(0)}"
     assert seen
+
+
+def test_copies_are_waited_for_before_a_thread_block_ends():
+    """Whatever ends the loop of a warp that issues bulk copies (a bounded wait
+    that ran out among it), the warp then waits for those in flight: each such
+    warp's branch ends in waits on the barriers that its copies complete on."""
+    seen = 0
+    for name in ("decode.cu", "prefill.cu", "dense.cu"):
+        text = _source(name)
+        for m in re.finditer(r"\bif \(warp [^{]*\{", text):
+            a, b = _block(text, m.end() - 1)
+            body = text[a:b]
+            loads = list(re.finditer(r"\b(?:tma_load_2d|tma_load_2d_pair|bulk_g2s|bulk_g2s_hint)_warp\(", body))
+            if not loads:
+                continue
+            seen += 1
+            last = list(re.finditer(r"\bmbar_wait_warp\(&\w*full\[", body))[-1].start()
+            assert last > loads[-1].start(), f"{name}: {m.group(0)}"
+    assert seen == 6
+
+
+def test_mmas_are_waited_for_before_tensor_memory_is_freed():
+    """The issuing warp's branch ends in a wait on a commit of all its MMAs."""
+    seen = 0
+    for name in ("decode.cu", "prefill.cu", "dense.cu"):
+        text = _source(name)
+        for m in re.finditer(r"\bif \(warp [^{]*\{", text):
+            a, b = _block(text, m.end() - 1)
+            body = text[a:b]
+            mmas = list(re.finditer(r"\bumma_(?:bf16|bf16_ts|bf16_pair|mxf4_ts)_warp\(", body))
+            if not mmas:
+                continue
+            seen += 1
+            assert re.search(r"umma_commit(?:_pair)?_warp\(&(mma_done|acc_bar).*mbar_wait_warp\(&\1", body[mmas[-1].end():],
+                             re.S), f"{name}: {m.group(0)}"
+    assert seen == 6   # (the decode kernel: a branch within the branch)
