@@ -286,7 +286,8 @@ int sdq_contract_add(sdq_plan plan, const uint32_t* codes_tiled, const float* al
  * into it with float reductions (as sdq_contract_add): results agree with
  * sdq_contract to within the order of those additions, not bit for bit.
  * The contraction may start streaming the codes before the prepare kernel
- * completes (it reads nothing the prepare kernel writes until then).  Large
+ * completes, but after all earlier work of the stream has (it reads nothing
+ * the prepare kernel writes until that is complete too).  Large
  * batches take the dense route where sdq_forward_route says 3: the weights
  * are rebuilt into the workspace (sdq_workspace_bytes includes n_out x k_in
  * bf16 for those batch sizes), then multiplied by x in one GEMM. */

@@ -279,9 +279,9 @@ extern "C" int sdq_contract_add(sdq_plan p, const uint32_t* codes_tiled, const f
 }
 
 // The prepare kernel, then the contraction; behind its own prepare kernel the
-// decode kernel may start reading the codes before the preceding grid
-// finishes: that grid waited for everything before it in the stream, and it
-// does not write the codes.
+// contraction may start reading the codes (and the scales) before that grid
+// finishes: every prepare kernel lets its dependents start only after its own
+// wait for everything before it in the stream, and it writes neither.
 extern "C" int sdq_linear_forward(sdq_plan p, const uint32_t* codes_tiled, const float* alpha,
                                   const uint16_t* x, int32_t M, float* y, void* ws, size_t ws_bytes,
                                   void* stream) {

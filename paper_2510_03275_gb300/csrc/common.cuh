@@ -66,8 +66,9 @@ void* tensor_map_encoder();
 // (the decode layout's xt region).
 cudaError_t launch_prep_tc(const sdq_plan_s* p, const uint16_t* x, int M, void* ws, cudaStream_t st,
                            bool* used, bool fp32_too);
-// early = 1: the decode kernel starts streaming codes before waiting for the
-// preceding grid (valid only behind this library's own prep kernels).
+// early = 1: the contraction starts streaming codes before waiting for the
+// preceding grid (valid only behind this library's own prep kernels, which
+// trigger their dependents after their own wait).
 // y_mode: kYStore: y = the result (split-K by the deterministic ticket
 // route); kYZeroed: y holds zeros (the prepare kernel of the same call
 // cleared it), so that split-K partial sums are added into it by float

@@ -66,8 +66,9 @@
 //                 sb * 128 codes = contiguous slabs of the tiled layout)
 //                 into the ring with bulk copies
 // With `early` set the producers start the code stream (one stage each)
-// before waiting for the preceding grid (codes are never written by the
-// prep kernels; with bstream the stage's B rows and scale words, which that
+// before waiting for the preceding grid (a prepare kernel of the same call,
+// which writes no codes and lets this kernel start only once the grids before
+// it are complete; with bstream the stage's B rows and scale words, which that
 // grid writes, follow after the wait), and the expanders expand those stages'
 // codes before they wait, so that only the B scales are left to do then (4096 x
 // 4096, M = 1: from the B operand's arrival to the first MMA 1.1 us, so 0.7).
@@ -606,6 +607,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
       }
       cp_async_commit();
     };
+    if (!early) pdl_wait();   // (alpha too may be the preceding grid's)
 #pragma unroll
     for (int k = 0; k < kAlphaAhead; ++k) alpha_fetch(k);
     pdl_wait();   // y and the workspace belong to the preceding grid until then

@@ -168,9 +168,6 @@ __global__ void __launch_bounds__(128) prep_decode_kernel(DecPrepParams p) {
   uint16_t* xs = reinterpret_cast<uint16_t*>(dsm);   // TB x ld
   uint16_t* ghs = xs + TB * ld;                        // 64 x ld
   uint16_t* gls = ghs + 64 * ld;                       // 64 x ld
-  // The decode kernel may start right away: it waits for this grid to
-  // complete before it reads anything this grid writes (y, the workspace).
-  pdl_launch_dependents();
   const int jt = blockIdx.x, bt = blockIdx.y, m = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int b0 = bt * TB, j0 = jt * 64, wcol = warp * 16;
@@ -189,6 +186,11 @@ __global__ void __launch_bounds__(128) prep_decode_kernel(DecPrepParams p) {
   };
   if (p.vec) load_g(0);
   pdl_wait();
+  // The decode kernel may start from here on, not before: it reads the codes
+  // and the scales, which the grids before this one may have written, without
+  // a wait of its own (and waits for this grid before it reads what this grid
+  // writes: y, the workspace).
+  pdl_launch_dependents();
   if (p.y_zero) {   // grid-stride clear of y
     const int64_t nthr = (int64_t)gridDim.x * gridDim.y * gridDim.z * 128;
     const int64_t i0 = ((int64_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * 128 + tid;
