@@ -339,9 +339,13 @@ int sdq_read_prep(sdq_plan plan, int32_t M, const void* ws, float* xt_out, void*
  * the scratch is a library-owned device array of sdq_noalloc_scratch_bytes()
  * (16 MiB) per GPU, reserved when the library loads and held until the
  * process exits.  No cudaMalloc / cudaFree / allocating call is made.
- *   - M must be 1..64 (the decode path), and sdq_workspace_bytes(plan, M)
- *     must not exceed the array: otherwise SDQ_ERR_INVALID_ARG or
- *     SDQ_ERR_WORKSPACE is returned and nothing is launched.
+ *   - M must be 1..64 (the decode path), and the decode workspace without the
+ *     split-K partials and tickets that sdq_workspace_bytes also counts
+ *     (sdq_contract's alone) must fit in the array: (4 M + N / 2 + N / 32) K_pad
+ *     bytes, K_pad = 128 ceil(K_eff / 128), N = M T rounded up to 16 (see
+ *     sdq_contract), and at most 128 N + 1 KB more.  Otherwise
+ *     SDQ_ERR_INVALID_ARG or SDQ_ERR_WORKSPACE is returned and nothing is
+ *     launched.
  *   - The current device must be the plan's (else SDQ_ERR_INVALID_ARG): the
  *     array of the current device is used.
  *   - The first call on a device looks up the array's device address

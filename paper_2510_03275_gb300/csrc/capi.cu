@@ -76,12 +76,13 @@ WsLayout workspace_layout(const sdq_plan_s* pl, int M) {
     off = align_up(off + (kb + 1) / 2 * dc.NP * 128, 256);
     L.sfbw = off;                                  // B scale words: KB x NP x 4 bytes
     off = align_up(off + kb * dc.NP * 4, 256);
+    L.err = off;                                   // call record
+    off = align_up(off + 2 * sizeof(uint64_t), 256);
+    L.used = off;                                  // (a forward adds its k chunks' shares into y)
     L.part = off;
     off = align_up(off + (dc.S > 1 ? sizeof(float) * (size_t)dc.S * M * g.ntiles * kTileRows : 0), 256);
     L.cnt = off;                                   // one 64-bit ticket per row tile
     off = align_up(off + sizeof(uint64_t) * (size_t)g.ntiles, 256);
-    L.err = off;                                   // call record
-    off = align_up(off + 2 * sizeof(uint64_t), 256);
     L.least = off;
     if (prefill_route(pl, M)) {
       // call record, bf16 x_tilde, then fp32 x_tilde; a forward call needs the
@@ -98,7 +99,7 @@ WsLayout workspace_layout(const sdq_plan_s* pl, int M) {
     if (dense_route_applies(pl, M)) off = align_up(off + sizeof(uint16_t) * (size_t)g.n_out * g.k_in, 256);
     L.bimg = L.sfbw = L.part = L.cnt = L.err = off;   // call record only
     off = align_up(off + 2 * sizeof(uint64_t), 256);
-    L.least = off;
+    L.used = L.least = off;
   }
   L.total = off;
   return L;
@@ -237,14 +238,13 @@ extern "C" int sdq_unpack(sdq_plan p, const uint32_t* tiled, uint32_t* plain, ui
   return cuda_status(launch_unpack(p, tiled, plain, bad_count, (cudaStream_t)stream));
 }
 
-// `forward`: the workspace of sdq_linear_forward, which may be smaller.
-static int check_ws(sdq_plan p, int32_t M, const void* ws, size_t ws_bytes, bool forward = false) {
+// `need`: the layout's size that the call asks for.
+static int check_ws(sdq_plan p, int32_t M, const void* ws, size_t ws_bytes, size_t WsLayout::*need = &WsLayout::total) {
   if (!p || M < 1 || M > 65535) return SDQ_ERR_INVALID_ARG;
   const int dv = sdq_check_device(p);
   if (dv != SDQ_OK) return dv;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SDQ_ERR_INVALID_ARG;
-  const WsLayout L = workspace_layout(p, M);
-  return ws_bytes < (forward ? L.least : L.total) ? SDQ_ERR_WORKSPACE : SDQ_OK;
+  return ws_bytes < workspace_layout(p, M).*need ? SDQ_ERR_WORKSPACE : SDQ_OK;
 }
 
 extern "C" int sdq_prep_activations(sdq_plan p, const uint16_t* x, int32_t M, void* ws,
@@ -256,8 +256,9 @@ extern "C" int sdq_prep_activations(sdq_plan p, const uint16_t* x, int32_t M, vo
 }
 
 static int contract(sdq_plan p, const uint32_t* codes_tiled, const float* alpha, int32_t M, float* y,
-                    void* ws, size_t ws_bytes, void* stream, int early, int y_mode) {
-  int st = check_ws(p, M, ws, ws_bytes, early != 0);   // (early: behind this call's own prepare kernel)
+                    void* ws, size_t ws_bytes, void* stream, int early, int y_mode,
+                    size_t WsLayout::*need = &WsLayout::total) {
+  int st = check_ws(p, M, ws, ws_bytes, need);
   if (st != SDQ_OK) return st;
   if (!codes_tiled || !alpha || !y || !aligned16(codes_tiled) || !aligned16(y)) return SDQ_ERR_INVALID_ARG;
   cudaError_t e = prefill_route(p, M)
@@ -282,13 +283,12 @@ extern "C" int sdq_contract_add(sdq_plan p, const uint32_t* codes_tiled, const f
 // contraction may start reading the codes (and the scales) before that grid
 // finishes: every prepare kernel lets its dependents start only after its own
 // wait for everything before it in the stream, and it writes neither.
-extern "C" int sdq_linear_forward(sdq_plan p, const uint32_t* codes_tiled, const float* alpha,
-                                  const uint16_t* x, int32_t M, float* y, void* ws, size_t ws_bytes,
-                                  void* stream) {
+static int forward(sdq_plan p, const uint32_t* codes_tiled, const float* alpha, const uint16_t* x, int32_t M,
+                   float* y, void* ws, size_t ws_bytes, void* stream, size_t WsLayout::*need) {
   // Decode batches: the prepare kernel also clears y, and the decode kernel
   // adds its split-K partial sums into it with float atomics.
   const bool zero_y = p && M >= 1 && M <= kMaxDecodeM && !prefill_route(p, M) && decode_config(p, M).S > 1;
-  int st = check_ws(p, M, ws, ws_bytes, true);
+  int st = check_ws(p, M, ws, ws_bytes, need);
   if (st != SDQ_OK) return st;
   if (!x || !aligned16(x) || !y || !aligned16(y)) return SDQ_ERR_INVALID_ARG;
   if (M > kMaxDecodeM && dense_route_applies(p, M)) {
@@ -301,8 +301,21 @@ extern "C" int sdq_linear_forward(sdq_plan p, const uint32_t* codes_tiled, const
   st = cuda_status(launch_prep(p, x, M, ws, (cudaStream_t)stream, zero_y ? y : nullptr,
                                ws_bytes >= workspace_layout(p, M).total));
   if (st != SDQ_OK) return st;
-  return contract(p, codes_tiled, alpha, M, y, ws, ws_bytes, stream, 1, zero_y ? kYZeroed : kYStore);
+  return contract(p, codes_tiled, alpha, M, y, ws, ws_bytes, stream, 1, zero_y ? kYZeroed : kYStore, need);
 }
+
+extern "C" int sdq_linear_forward(sdq_plan p, const uint32_t* codes_tiled, const float* alpha,
+                                  const uint16_t* x, int32_t M, float* y, void* ws, size_t ws_bytes,
+                                  void* stream) {
+  return forward(p, codes_tiled, alpha, x, M, y, ws, ws_bytes, stream, &WsLayout::least);
+}
+
+namespace sdq {
+int forward_on_scratch(sdq_plan p, const uint32_t* codes_tiled, const float* alpha, const uint16_t* x, int32_t M,
+                       float* y, void* ws, size_t ws_bytes, void* stream) {
+  return forward(p, codes_tiled, alpha, x, M, y, ws, ws_bytes, stream, &WsLayout::used);
+}
+}  // namespace sdq
 
 extern "C" int sdq_forward_kernels(sdq_plan p, int32_t M, const uint16_t* x) {
   if (!p || !x || M < 1 || M > 65535) return 0;

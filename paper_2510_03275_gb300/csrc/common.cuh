@@ -20,7 +20,8 @@ inline const DecodeConfig& decode_config(const sdq_plan_s* plan, int M) { return
 struct WsLayout {
   size_t xt, bimg, sfbw, part, cnt, err, total;
   size_t xtb;    // bf16 x_tilde of the prefill contraction (prefill_route)
-  size_t least;  // bytes that sdq_linear_forward needs
+  size_t used;   // the decode layout without sdq_contract's partials and tickets (what the allocation-free entry asks for)
+  size_t least;  // bytes that sdq_linear_forward asks its caller for
   size_t what;   // rebuilt weights W' (n_out x k_in bf16) of the dense large-batch route
 };
 WsLayout workspace_layout(const sdq_plan_s* plan, int M);
@@ -34,6 +35,9 @@ int sdq_check_device(const sdq_plan_s* p);
 // says the last call gave up a bounded wait, else SDQ_OK; synchronizes
 // `stream`.
 int workspace_record_status(const sdq_plan_s* p, int32_t M, const void* ws, void* stream);
+// sdq_linear_forward on a workspace that may be as small as WsLayout::used.
+int forward_on_scratch(sdq_plan_s* p, const uint32_t* codes_tiled, const float* alpha, const uint16_t* x, int32_t M,
+                       float* y, void* ws, size_t ws_bytes, void* stream);
 // Number of a contraction call, from one process-wide counter (never 0).
 uint64_t next_call_number();
 // Tag of call number n for the workspace's tickets and call record: a

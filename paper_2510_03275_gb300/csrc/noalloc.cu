@@ -4,17 +4,18 @@
 // a host runtime that owns every device allocation through its own pool
 // (and forbids cudaMalloc from third-party code), or a serving loop that
 // must not allocate device memory once it has started.  For them this file
-// keeps the decode scratch (x_tilde and the fp8 B operand of the two-kernel
-// route, split-K partials, tickets and the call record) in one file-scope
-// device array of kNoAllocScratchBytes per GPU, reserved when the library is
-// loaded and held until the process exits.
+// keeps the decode workspace without the split-K partials and tickets, which
+// are sdq_contract's alone (x_tilde, the e2m1 B operand and its scales, the call
+// record; the larger batches' bf16 x_tilde takes less), in one file-scope device
+// array of kNoAllocScratchBytes per GPU, reserved when the library is loaded and
+// held until the process exits.
 //
 // The array is shared by every call on a device and keeps whatever the last
-// call left in it: tickets and the call record carry a scrambled 48-bit tag
-// per call, so stale contents do not count (a leftover word matches a call's
-// tag with probability 2^-47), and everything else is written before it is
-// read.  Two calls that overlap on the GPU (different streams,
-// or different host threads) race on the array.
+// call left in it: the call record carries a scrambled 48-bit tag per call, so
+// stale contents do not count (a leftover word matches a call's tag with
+// probability 2^-47), and everything else is written before it is read.  Two
+// calls that overlap on the GPU (different streams, or different host threads)
+// race on the array.
 #include <mutex>
 
 #include "common.cuh"
@@ -51,7 +52,7 @@ int noalloc_scratch(sdq_plan p, int32_t M, void** ws) {
   if (!p || M < 1 || M > sdq::kMaxDecodeM) return SDQ_ERR_INVALID_ARG;
   int st = sdq::sdq_check_device(p);
   if (st != SDQ_OK) return st;
-  const size_t need = sdq::workspace_layout(p, M).least;
+  const size_t need = sdq::workspace_layout(p, M).used;
   if (need > kNoAllocScratchBytes) return SDQ_ERR_WORKSPACE;
   return scratch_for_current_device(ws);
 }
@@ -65,7 +66,7 @@ extern "C" int sdq_linear_forward_noalloc(sdq_plan p, const uint32_t* codes_tile
   void* ws = nullptr;
   const int st = noalloc_scratch(p, M, &ws);
   if (st != SDQ_OK) return st;
-  return sdq_linear_forward(p, codes_tiled, alpha, x, M, y, ws, kNoAllocScratchBytes, stream);
+  return sdq::forward_on_scratch(p, codes_tiled, alpha, x, M, y, ws, kNoAllocScratchBytes, stream);
 }
 
 extern "C" int sdq_noalloc_status(sdq_plan p, int32_t M, void* stream) {

@@ -68,3 +68,27 @@ def test_noalloc_rejects_oversize(sdq):
     with pytest.raises(sdq.SdqError) as e:
         sdq.sdq_linear_forward_noalloc(plan.handle, tiled, alpha, x, 65, y)
     assert e.value.status == -1
+
+
+@pytest.mark.parametrize("n,k,b,osr,q,m", [(57344, 28672, 64, Fraction(5, 2), 2, 5), (11008, 8192, 128, 3, 1, 48),
+                                           (4096, 28672, 64, Fraction(3, 2), 1, 32)])
+def test_noalloc_takes_layers_with_many_k_chunks(sdq, n, k, b, osr, q, m):
+    """The split-K partials that sdq_workspace_bytes counts for sdq_contract are
+    not part of the limit: they depend on the launch shape, which must not
+    decide whether a layer is accepted."""
+    import torch
+    d = sdq.LayerDesc(n, k, b, Fraction(osr), q)
+    plan = sdq.Plan(d)
+    g = torch.Generator(device="cuda").manual_seed(n + m)
+    tiled = torch.randint(-2 ** 31, 2 ** 31, (plan.alloc_tiled().numel(),), generator=g, device="cuda", dtype=torch.int32)
+    if q == O.TERNARY:
+        tiled &= 0x55555555
+    alpha = torch.rand(n, generator=g, device="cuda") + 0.5
+    x = torch.randn((m, k), generator=g, device="cuda").to(torch.bfloat16)
+    ref = plan.forward(tiled, alpha, x)
+    y = torch.full((m, n), float("nan"), device="cuda")
+    for _ in range(2):
+        sdq.sdq_linear_forward_noalloc(plan.handle, tiled, alpha, x, m, y)
+    assert sdq.sdq_noalloc_status(plan.handle, m) == 0
+    # the same kernels; where K is split, the order of the fp32 sums is not fixed
+    assert (y - ref).abs().max() <= 1e-5 * ref.abs().max()
