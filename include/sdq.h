@@ -315,8 +315,8 @@ int sdq_forward_route(sdq_plan plan, int32_t M);
 /* Wait for `stream`, then report whether the last contraction that used
  * `ws` (same plan and M) completed its bounded device-side waits: SDQ_OK or
  * SDQ_ERR_TIMEOUT (a copy or an MMA did not complete within about 2 s; the
- * output of that call is invalid).  Covers the decode (M <= 64) and the
- * prefill (M > 64) kernels.  Workspace contents never need resetting: the
+ * output of that call is invalid), the kernel that prepared its operand
+ * included.  Covers the decode (M <= 64) and the prefill (M > 64) kernels.  Workspace contents never need resetting: the
  * split-K tickets and this record carry a 48-bit tag per call (bit 47 set,
  * the other 47 bits a bijective scramble of a process-wide call counter),
  * so zeros, another call's tickets and structured leftovers of another plan

@@ -77,7 +77,7 @@ WsLayout workspace_layout(const sdq_plan_s* pl, int M) {
     L.sfbw = off;                                  // B scale words: KB x NP x 4 bytes
     off = align_up(off + kb * dc.NP * 4, 256);
     L.err = off;                                   // call record
-    off = align_up(off + 2 * sizeof(uint64_t), 256);
+    off = align_up(off + 4 * sizeof(uint64_t), 256);
     L.used = off;                                  // (a forward adds its k chunks' shares into y)
     L.part = off;
     off = align_up(off + (dc.S > 1 ? sizeof(float) * (size_t)dc.S * M * g.ntiles * kTileRows : 0), 256);
@@ -98,7 +98,7 @@ WsLayout workspace_layout(const sdq_plan_s* pl, int M) {
     L.what = off;                                  // dense route: W', n_out x k_in bf16
     if (dense_route_applies(pl, M)) off = align_up(off + sizeof(uint16_t) * (size_t)g.n_out * g.k_in, 256);
     L.bimg = L.sfbw = L.part = L.cnt = L.err = off;   // call record only
-    off = align_up(off + 2 * sizeof(uint64_t), 256);
+    off = align_up(off + 4 * sizeof(uint64_t), 256);
     L.used = L.least = off;
   }
   L.total = off;

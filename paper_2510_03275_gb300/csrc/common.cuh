@@ -16,7 +16,7 @@ DecodeConfig decode_config_search(const sdq_plan_s* plan, int M);
 inline const DecodeConfig& decode_config(const sdq_plan_s* plan, int M) { return plan->dcfg[M]; }
 
 // Workspace regions (byte offsets).  cnt: one 64-bit split-K ticket per row
-// tile; err: the call record (two 64-bit words, see call_record_*).
+// tile; err: the call record (four 64-bit words, see call_record_*).
 struct WsLayout {
   size_t xt, bimg, sfbw, part, cnt, err, total;
   size_t xtb;    // bf16 x_tilde of the prefill contraction (prefill_route)
@@ -470,17 +470,30 @@ __device__ __forceinline__ bool group_and(int id, int nthreads, bool v) {
 }
 
 // Call record in the workspace: word 0 = tag of the last call that gave up a
-// bounded wait, word 1 = tag of the last call that ran.  Tags (call_tag in
+// bounded wait, word 1 = tag of the last call that ran; words 2 and 3 the same
+// for the kernels that prepare a contraction's operand and have bounded waits
+// (prep_tc_kernel, recon_kernel), which have tags of their own: the
+// contraction behind one that gave up fails too.  Tags (call_tag in
 // capi.cu) are 48-bit values with bit 47 set, distinct for 2^47 calls and
 // scrambled, so that neither zeroed memory nor structured leftovers of
 // another call, plan or batch size (counters, small floats) read as the
 // current call's: nothing in the workspace needs resetting.
-__device__ __forceinline__ void call_record_start(uint64_t* rec, uint64_t call, bool leader) {
-  if (leader) rec[1] = call;
-}
 __device__ __forceinline__ void call_record_fail(uint64_t* rec, uint64_t call) {
   atomicExch(reinterpret_cast<unsigned long long*>(rec), (unsigned long long)call);
 }
+__device__ __forceinline__ void call_record_start(uint64_t* rec, uint64_t call, bool leader) {
+  if (leader) rec[1] = call;
+}
+// (by a contraction whose operand such a kernel prepared, once that is complete)
+__device__ __forceinline__ void call_record_start_prepared(uint64_t* rec, uint64_t call, bool leader) {
+  if (!leader) return;
+  rec[1] = call;
+  if (rec[2] == rec[3] && (rec[3] >> 47) == 1) call_record_fail(rec, call);
+}
+__device__ __forceinline__ void prep_record_start(uint64_t* rec, uint64_t call, bool leader) {
+  if (leader) rec[3] = call;
+}
+__device__ __forceinline__ void prep_record_fail(uint64_t* rec, uint64_t call) { call_record_fail(rec + 2, call); }
 
 __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;\n" ::: "memory"); }
 

@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(kRbThreads, 1)
   tc_fence_after();
   pdl_wait();
   pdl_launch_dependents();
+  prep_record_start(p.rec, p.call, blockIdx.x == 0 && tid == 0);
   const uint32_t tmem = tmem_base;
   bool ok = true;
   // this CTA's items: (row tile, block) = item / nblk, item % nblk
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(kRbThreads, 1)
     }
     if (et == 0) bulk_store_wait_all();   // written before the CTA ends
   }
-  if (!ok) call_record_fail(p.rec, p.call);
+  if (!ok) prep_record_fail(p.rec, p.call);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
@@ -320,7 +321,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kDnThreads, 1)
   tc_fence_after();
   pdl_wait();
   pdl_launch_dependents();
-  call_record_start(p.rec, p.call, blockIdx.x == 0 && threadIdx.x == 0);
+  call_record_start_prepared(p.rec, p.call, blockIdx.x == 0 && threadIdx.x == 0);
   const uint32_t tmem = tmem_base;
   bool ok = true;
   if (warp == 0) {

@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   // with `early` the codes (which the preceding grid does not write) start at once
   if (!(p.early && warp == 2 + kExpWarps)) pdl_wait();
   pdl_launch_dependents();
-  call_record_start(p.rec, p.call, blockIdx.x == 0 && blockIdx.y == 0 && z == 0 && tid == 0);
+  call_record_start_prepared(p.rec, p.call, blockIdx.x == 0 && blockIdx.y == 0 && z == 0 && tid == 0);
   const uint32_t tmem = tmem_base;
   const uint32_t acol = tmem + (uint32_t)p.bn;
   bool ok = true;
@@ -509,6 +509,7 @@ __global__ void __launch_bounds__(kPtThreads, 1)
     if (!mbar_wait_warp(&mma_done, 0)) ok = false;
   } else {
     pdl_wait();   // the workspace belongs to the preceding grid until then
+    prep_record_start(p.rec, p.call, blockIdx.x == 0 && blockIdx.y == 0 && tid == 64);
     const int et = tid - 64, q = warp & 3, half = (warp - 2) >> 2;
     // the K padding of every batch row (k_eff .. kpad, a multiple of 8; by
     // the CTAs of the first columns)
@@ -579,7 +580,7 @@ __global__ void __launch_bounds__(kPtThreads, 1)
       }
     }
   }
-  if (!ok) call_record_fail(p.rec, p.call);
+  if (!ok) prep_record_fail(p.rec, p.call);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
@@ -668,7 +669,7 @@ cudaError_t launch_prep_tc(const sdq_plan_s* pl, const uint16_t* x, int M, void*
   uint8_t* wbase = static_cast<uint8_t*>(ws);
   const int64_t R = (int64_t)M * g.nblk;
   if (R >= (int64_t(1) << 31) - kPtRows) return cudaSuccess;
-  PrepTcParams p;   // (a timeout is recorded under this kernel's own call number)
+  PrepTcParams p;
   p.xtb = reinterpret_cast<uint16_t*>(wbase + L.xtb);
   p.xt = fp32_too ? reinterpret_cast<float*>(wbase + L.xt) : nullptr;
   p.rec = reinterpret_cast<uint64_t*>(wbase + L.err);

@@ -30,6 +30,8 @@ struct PrepParams {
   const uint16_t* g_hi;
   const uint16_t* g_lo;
   uint16_t* xtb;      // bf16 M x kpad (permuted)
+  uint64_t* rec;      // call record
+  uint64_t call;
   int M, K, B, n_b, nblk;
   int64_t k_eff, kpad;
   int vec, ternary;
@@ -47,6 +49,7 @@ __global__ void __launch_bounds__(128) prep_kernel(PrepParams p) {
   pdl_launch_dependents();
   const int jt = blockIdx.x, bt = blockIdx.y, m = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  prep_record_start(p.rec, p.call, jt == 0 && bt == 0 && m == 0 && tid == 0);   // (no waits: it never fails)
   const int b0 = bt * TB, j0 = jt * 64;
   const int wrow = TB == 64 ? warp * 16 : 0;       // warp's first row in the tile
   const int wcol = TB == 64 ? 0 : warp * 16;       // warp's first column
@@ -374,6 +377,8 @@ cudaError_t launch_prep(const sdq_plan_s* pl, const uint16_t* x, int M, void* ws
   PrepParams p;
   p.x = x; p.g_hi = pl->d_g_hi; p.g_lo = pl->d_g_lo;
   p.xtb = reinterpret_cast<uint16_t*>(base + L.xtb);
+  p.rec = reinterpret_cast<uint64_t*>(base + L.err);
+  p.call = call_tag(next_call_number());
   p.M = M; p.K = g.k_in; p.B = g.block; p.n_b = g.n_b; p.nblk = g.nblk;
   p.k_eff = g.k_eff; p.kpad = g.k_eff_pad;
   p.ternary = pl->desc.quantizer == SDQ_TERNARY;
