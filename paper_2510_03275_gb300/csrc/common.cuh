@@ -445,6 +445,16 @@ __device__ __forceinline__ uint32_t e2m1x2(float lo, float hi, float2* q) {
   return b;
 }
 
+// The exponent e of the term scales of a 32-code group whose largest magnitude
+// is mx (x_tilde = sum_t 2^(e - 3t) q_t, t < T): mx < 2^(e + 2) with the
+// exponent field of mx, and no less than 3 T - 129, so that the scale byte
+// 127 + e - 3t of every term is at least 1 (maxima below 2^(3 T - 127), the
+// subnormal among them, then lose their last bits, in steps of 2^-127).
+__device__ __forceinline__ int term_exponent(float mx, int T) {
+  return max(3 * T - 129, min(126, (int)(__float_as_uint(mx) >> 23) - 128));
+}
+__device__ __forceinline__ float exp2_int(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }   // -126 .. 127
+
 // r[0 .. 7] to the 32 bytes at p (32-byte aligned), one store.
 __device__ __forceinline__ void st_global32(void* p, const uint32_t* r) {
   asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]),

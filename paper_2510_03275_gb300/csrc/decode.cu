@@ -180,13 +180,8 @@ __device__ __noinline__ void write_terms(const DecodeParams& p, uint8_t* bop, ui
     for (int i = 0; i < 8; ++i) mx = fmaxf(mx, fabsf(v[i]));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    int e = -125;
-    if (mx > 0.f) {   // mx < 2^E, so |v 2^-(E - 2)| < 4
-      int E = 0;
-      frexpf(mx, &E);
-      e = E - 2;
-    }
-    const float inv = ldexpf(1.f, -e);
+    const int e = term_exponent(mx, p.T);
+    const float inv = exp2_int(-e);
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] *= inv;
     if (!act) continue;
@@ -204,7 +199,7 @@ __device__ __noinline__ void write_terms(const DecodeParams& p, uint8_t* bop, ui
       }
       const int row = m * p.T + t;
       *reinterpret_cast<uint32_t*>(img + row * 128 + ((chunk ^ (row & 7)) << 4) + off) = word;
-      if ((g8 & 3) == 0) sfbs[((size_t)bl * p.NP + row) * 4 + (g8 >> 2)] = (uint8_t)max(1, min(254, 127 + e - 3 * t));
+      if ((g8 & 3) == 0) sfbs[((size_t)bl * p.NP + row) * 4 + (g8 >> 2)] = (uint8_t)(127 + e - 3 * t);
     }
   }
 }

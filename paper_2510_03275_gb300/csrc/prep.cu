@@ -290,9 +290,8 @@ __global__ void __launch_bounds__(128) prep_decode_kernel(DecPrepParams p) {
       }
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      // mx < 2^E, E - 126 its exponent field, so |v 2^-(E - 2)| < 4
-      const int ex = max(-125, min(126, (int)(__float_as_uint(mx) >> 23) - 128));
-      const float inv = __uint_as_float((uint32_t)(127 - ex) << 23);
+      const int ex = term_exponent(mx, p.T);
+      const float inv = exp2_int(-ex);
 #pragma unroll
       for (int i = 0; i < 8; ++i) v[i] *= inv;
       if (act) {
@@ -309,7 +308,7 @@ __global__ void __launch_bounds__(128) prep_decode_kernel(DecPrepParams p) {
           }
           const int row = m * p.T + tt;
           *reinterpret_cast<uint32_t*>(img + row * 128 + ((chunk ^ (row & 7)) << 4) + off) = word;
-          if (s4 == 0) p.sfbw[((size_t)kb * p.NP + row) * 4 + (g8 >> 2)] = (uint8_t)max(1, min(254, 127 + ex - 3 * tt));
+          if (s4 == 0) p.sfbw[((size_t)kb * p.NP + row) * 4 + (g8 >> 2)] = (uint8_t)(127 + ex - 3 * tt);
         }
       }
     }
