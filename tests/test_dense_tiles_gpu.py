@@ -1,5 +1,6 @@
 """GPU: the dense route's tiles: batches around multiples of its batch tiles
-(one and two weight tiles per thread block, a last wave of single tiles), rows
+(one and two weight tiles per pair of thread blocks; the last two shapes end
+in a wave of single tiles on devices of 70 to 76 such pairs), rows
 that end inside a tile (the rebuilt weights' stores are clipped there) and
 every number of 64-code chunks per block (one and two epilogue buffers), each
 element within the bound of the rebuilt weights' bf16 rounding."""
@@ -17,7 +18,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("q", [O.TERNARY, O.BINARY])
 @pytest.mark.parametrize("n,k,osr,m", [(1, 128, 2, 768), (130, 256, Fraction(3, 2), 769), (257, 384, Fraction(5, 2), 1040),
-                                       (4200, 128, 3, 800), (5000, 128, 1, 1601), (2600, 256, 2, 2305)])
+                                       (4200, 128, 3, 800), (5000, 128, 1, 1601), (2600, 256, 2, 2305),
+                                       (6529, 128, 2, 1295), (3713, 128, Fraction(3, 2), 2681)])
 def test_dense_tiles(sdq, q, n, k, osr, m):
     import torch
     assert torch.cuda.is_available()
