@@ -69,9 +69,10 @@
 // before waiting for the preceding grid (a prepare kernel of the same call,
 // which writes no codes and lets this kernel start only once the grids before
 // it are complete; with bstream the stage's B rows and scale words, which that
-// grid writes, follow after the wait), and the expanders expand those stages'
-// codes before they wait, so that only the B scales are left to do then (4096 x
-// 4096, M = 1: from the B operand's arrival to the first MMA 1.1 us, so 0.7).
+// grid writes, follow after the wait).  The expanders expand those stages'
+// codes while the B operand's copies are in flight, so that only the B scales
+// are left to do then (LLaMA-7B layer at M = 1 47.6 us with them expanded ahead
+// of the wait, where they held up the copies, 46.2 so; 48.0 with neither).
 //
 // bstream (batches whose term rows make a chunk-resident B image bound the k
 // chunk): each stage's image pairs and scale words are bulk-copied into its
@@ -474,18 +475,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
         }
       }
     };
-    // with `early` the first stage's codes before the preceding grid completes
-    // (with bstream the slot fills after it: no bounded wait spans that grid)
-    const bool ahead = early && !p.bstream && x < nstages;
-    if (ahead) {
-      ok = warp_wait(&c_full[slot], 0);
-      if (ok) {
-        uint32_t w[kMaxSb][8];
-        const int nb = sblk[j + 1] - sblk[j];
-        load(ring + (size_t)slot * p.slot_bytes, nb, w);
-        put(w, nb, x);   // (x < ns)
-      }
-    }
+    // the set's first stage, expanded while the B operand's copies are in flight
+    const bool ahead = p.bsrc == 2 && !p.bstream && x < nstages;
     pdl_wait();
     if (p.bstream) {
       // (the B rows and scale words arrive with each stage)
@@ -507,6 +498,15 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeParams p) {
       }
       copy_lsu(reinterpret_cast<uint4*>(sfbs), reinterpret_cast<const uint4*>(p.sfbw + (size_t)kb0 * p.NP * 4),
                ncb * p.NP / 4, et);
+      if (ahead) {
+        ok = warp_wait(&c_full[slot], 0);
+        if (ok) {
+          uint32_t w[kMaxSb][8];
+          const int nb = sblk[j + 1] - sblk[j];
+          load(ring + (size_t)slot * p.slot_bytes, nb, w);
+          put(w, nb, x);   // (x < ns)
+        }
+      }
       cp_async_wait_all();
     } else {
       write_terms(p, bop, sfbs, kb0, ncb, et);
