@@ -15,8 +15,8 @@
 // shared memory for the CTA's lifetime (bf16 hi and lo parts, 128 output
 // columns k x n_b codes, K-major, 128-byte swizzle, its K order permuted as
 // the code expansion orders the codes); one 128 x 128 fp32 accumulator per
-// (row tile, block) item, two of them so that an item's epilogue (bf16 W',
-// 16-byte stores) overlaps the next item's MMAs.  Persistent CTAs over the
+// (row tile, block) item, two of them so that an item's epilogue (bf16 W' through
+// a swizzled tile and TMA stores) overlaps the next item's MMAs.  Persistent CTAs over the
 // items.
 //   warp 0     TMEM allocation; G^T once (TMA), then the code slabs
 //   warp 1     8 MMAs per 64 codes (4 K steps x hi / lo)

@@ -643,12 +643,21 @@ cudaError_t prefill_occupancy(sdq_plan_s* pl) {
 }
 
 static bool prep_tc_takes(const Geometry& g) { return g.block >= 64 && g.block <= 512 && g.n_b % 64 == 0; }
-// The crossings of the two contractions per layer size (us a forward call at
-// OSR 2, 4-bit decode kernel / this one): 4096 x 4096 M = 24 16.1 / 13.4;
-// 22016 x 4096 M = 24 32.5 / 34.7, M = 40 42.8 / 37.0; 57344 x 8192 M = 48
-// 116 / 122, M = 64 136 / 124.  This one's time is nearly flat in M: the
-// expanded codes' stores into tensor memory (16 KB per 2 KB of codes) bound
-// it, about 290 cycles a stage and SM.
+// us a forward call at OSR 2, B = 128, ternary (4-bit decode kernel / this one):
+//   4096 x 4096    M = 24 11.8 / 13.4   M = 40 13.2 / 13.8   M = 44 14.7 / 13.7
+//   22016 x 4096   M = 40 30.9 / 37.3   M = 48 34.4 / 37.6   M = 56 41.8 / 38.3
+//   57344 x 8192   M = 48  113 / 120    M = 56  122 / 121    M = 64  125 / 122
+// Binary codes, B = 64 and OSR 3/2 and 3 cross within 12 rows of these or stay
+// with the decode kernel (57344 x 8192 binary, M = 64: 127 / 133), 1024 x 1024
+// crosses at 64; B = 512 crosses lower (4096 x 4096 from M = 16, 22016 x 4096 at
+// 32, 57344 x 8192 at 44).  The lines were drawn when the decode kernel took 16.1
+// us for the first of these and 42.8 for 22016 x 4096 at M = 40, before its launch
+// shapes were fitted anew.  They stay below the crossings because this kernel's
+// operand is the closer one, bf16 x_tilde against three e2m1 terms (error against
+// 64 bits 1.7e-3 and 2.0e-3): at most 1.5x of a call's time is given for it (binary
+// 12288 x 4096, OSR 3, M = 40: 25 / 38 us).  This kernel's time is nearly flat in M:
+// the expanded codes' stores into tensor memory (16 KB per 2 KB of codes) bound it,
+// about 290 cycles a stage and SM.
 int wide_min_batch(const sdq_plan_s* pl) {
   const Geometry& g = pl->geo;
   if (!prep_tc_takes(g) || !encode_fn()) return kMaxDecodeM + 1;

@@ -8,10 +8,12 @@
 // x is bf16 (exact), G is split into bf16 hi + lo parts (relative error of
 // the pair ~2^-16), accumulation in fp32.
 //
-// Decode path (M <= 64): the decode prepare kernel below writes fp32
-// x_tilde, from which each decode CTA forms the e2m1 terms and scales of its
-// k chunk.  Prefill path: bf16 x_tilde in the permuted 64-code stage order
-// of the prefill kernel's operand tiles.
+// Decode batches: the decode prepare kernel below writes fp32 x_tilde and, where
+// n_b is a multiple of 64, the e2m1 terms and scales that the contraction reads
+// (elsewhere its CTAs form those of their k chunks).  Prefill batches, and the
+// decode batches that contract with the prefill kernel: bf16 x_tilde in the
+// permuted 64-code stage order of that kernel's operand tiles (prep_tc_kernel in
+// csrc/prefill.cu where it applies, else prep_kernel).
 #include <algorithm>
 
 #include "common.cuh"
