@@ -17,7 +17,9 @@ fp64 oracle by
                                    <= 0.25 * 8^-(T-1) * max_g |x_tilde|.
                      The group maximum is bounded by the 128-code block's.
   prefill (M > 64)   x_tilde rounded once to bf16 (8 significant bits):
-                     |error| <= 2^-8 |x_tilde_j|.
+                     |error| <= 2^-8 |x_tilde_j|.  The larger decode batches
+                     (from M = 24, 40 or 56 on, by the layer) take this route
+                     too; it is within the decode bound at their T = 3.
   dense (large M)    the route that rebuilds the weights: W'' = 2 C G per
                      block in fp32 (G as bf16 hi + lo, ~2^-16), rounded once
                      to bf16 (|delta W''_rk| <= 2^-9 |W''_rk|), then
